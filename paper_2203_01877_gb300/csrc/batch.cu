@@ -15,6 +15,8 @@
 //   few-group group-bys (at most 64 groups, closed-form sums): the key-range
 //             pass, then the direct kernel (vector reads one warp step ahead,
 //             lane-private tables), each job a contiguous range of blocks
+//   joined aggregations of closed-form shapes: the plain-load probe
+//             (probeagg.cuh), each job a contiguous range of blocks
 //   scan      one persistent launch of the staged scan engine per body kind
 //             (filter, shared filter, group-by, joined aggregation): CTAs draw chunk
 //             tickets across the tables of every job of that kind (uneven
@@ -42,6 +44,7 @@
 #include "bodies.cuh"
 #include "dimgroups.cuh"
 #include "dim.cuh"
+#include "probeagg.cuh"
 #include "finalize.cuh"
 #include "groupdirect.cuh"
 #include "multi.cuh"
@@ -157,6 +160,13 @@ struct DirJob {
     long long first_block, nblocks;
     long long range_first, range_nblocks;
 };
+// A joined aggregation run by the plain-load probe: blocks [first_block,
+// first_block + nblocks) of its launch.
+struct ProbeJob {
+    ProbeAggArgs A;
+    long long first_block, nblocks;
+};
+constexpr long long kPaRowsPerBlock = 32768;     // 32 128-row steps per warp
 constexpr int kDirArgsBytes = (static_cast<int>(sizeof(GroupDirectArgs)) + 127) / 128 * 128;
 constexpr long long kDirRowsPerBlock = 32768;    // direct kernel: 32 128-row steps per warp
 constexpr long long kDirRangeRowsPerBlock = 65536;
@@ -313,6 +323,13 @@ __global__ void __launch_bounds__(kDirThreads, kDirMinBlocks) k_b_gdirect(const 
     group_direct_block<false>(A, dsm, static_cast<long long>(blockIdx.x) - j.first_block, j.nblocks);
 }
 
+__global__ void __launch_bounds__(kPaThreads, kPaMinBlocks) k_b_probe_agg(const ProbeJob* J, const int32_t* bjob) {
+    __shared__ __align__(16) unsigned char args[sizeof(ProbeAggArgs)];
+    const ProbeJob& j = J[bjob[blockIdx.x]];
+    const ProbeAggArgs& A = stage_args(j.A, args);
+    probe_agg_block(A, static_cast<long long>(blockIdx.x) - j.first_block, j.nblocks);
+}
+
 __global__ void __launch_bounds__(kFinThreads) k_b_finalize(const FinJob* F) {
     extern __shared__ __align__(16) unsigned char fsm[];
     const FinJob& f = F[blockIdx.x];
@@ -370,11 +387,12 @@ struct tqp_batch {
     std::vector<TopJob> top;
     std::vector<DirJob> gdir;
     std::vector<FoldJob> fold;
+    std::vector<ProbeJob> probe;
     std::vector<std::vector<TopItem>> levels;
     // block -> job maps, concatenated
     std::vector<int32_t> maps;
     long long fill_blocks = 0, row_blocks = 0, num_blocks = 0, slot_blocks = 0, compact_blocks = 0, top0_blocks = 0,
-              sel_blocks = 0, grange_blocks = 0, gdirect_blocks = 0, fold_blocks = 0;
+              sel_blocks = 0, grange_blocks = 0, gdirect_blocks = 0, fold_blocks = 0, probe_blocks = 0;
     long long scan_chunks[kKinds] = {0, 0, 0, 0};
     // lookup tables and outputs of the shared scans (one blob; per job its offset)
     std::vector<unsigned char> mblob;
@@ -382,7 +400,7 @@ struct tqp_batch {
     unsigned char* d_mblob = nullptr;
     std::vector<long long> level_blocks;
     size_t off_fill = 0, off_row = 0, off_num = 0, off_slot = 0, off_compact = 0, off_top0 = 0, off_sel = 0,
-           off_grange = 0, off_gdirect = 0, off_fold = 0;
+           off_grange = 0, off_gdirect = 0, off_fold = 0, off_probe = 0;
     size_t off_scan[kKinds] = {0, 0, 0, 0};
     std::vector<size_t> off_level;
     // small zeroed counters share one slab (one fill range)
@@ -398,6 +416,7 @@ struct tqp_batch {
     TopJob* d_top = nullptr;
     DirJob* d_gdir = nullptr;
     FoldJob* d_fold = nullptr;
+    ProbeJob* d_probe = nullptr;
     std::vector<TopItem*> d_levels;
     int32_t* d_maps = nullptr;
     unsigned long long* d_ticket[kKinds] = {nullptr, nullptr, nullptr, nullptr};
@@ -744,7 +763,7 @@ static tqp_status add_join_job(tqp_batch* b, const tqp_plan* p, const tqp_result
     // aggregation by join key first (used on the device only if the table is
     // direct-mapped), as in the single-plan path
     if (grouped && A.pjfast && A.fast && A.H.meta && A.G.ntiles > 0 && F->num_rows >= 2 * std::max<long long>(1, ndr)) {
-        A.nk = A.S.nacc + (A.has_sum ? 1 : 0);
+        A.nk = keyfirst_words(A.S.nacc + (A.has_sum ? 1 : 0));
         const size_t kbytes = static_cast<size_t>(A.H.cap) * A.nk * 8;
         A.kacc = static_cast<unsigned long long*>(balloc(b, kbytes));
         if (!A.kacc) return arena_oom(ctx, kbytes);
@@ -768,7 +787,13 @@ static tqp_status add_join_job(tqp_batch* b, const tqp_plan* p, const tqp_result
         b->fold_blocks += Fo.nblocks;
         b->fold.push_back(Fo);
     }
-    if (A.G.ntiles > 0) {
+    ProbeJob P;
+    if (A.G.ntiles > 0 && lower_probe_agg(A, F, &P.A)) {
+        P.first_block = b->probe_blocks;
+        P.nblocks = (F->num_rows + kPaRowsPerBlock - 1) / kPaRowsPerBlock;
+        b->probe_blocks += P.nblocks;
+        b->probe.push_back(P);
+    } else if (A.G.ntiles > 0) {
         b->scan[kJobJoin - 1].push_back(J);
     } else {
         if (A.d_num_joined) b->zero.push_back(A.d_num_joined);
@@ -1094,6 +1119,8 @@ static void build_maps(tqp_batch* b) {
     for (size_t j = 0; j < b->gdir.size(); ++j) push(j, b->gdir[j].nblocks);
     b->off_fold = M.size();
     for (size_t j = 0; j < b->fold.size(); ++j) push(j, b->fold[j].nblocks);
+    b->off_probe = M.size();
+    for (size_t j = 0; j < b->probe.size(); ++j) push(j, b->probe[j].nblocks);
     b->off_compact = M.size();
     for (size_t j = 0; j < b->compact.size(); ++j) push(j, (b->compact[j].n + kCompactRows - 1) / kCompactRows);
     b->off_sel = M.size();
@@ -1161,6 +1188,8 @@ static tqp_status batch_launch(tqp_batch* b, cudaStream_t st) {
     if (b->gdirect_blocks)
         k_b_gdirect<<<static_cast<unsigned>(b->gdirect_blocks), kDirThreads, kDirSmemBytes + kDirArgsBytes, st>>>(
             b->d_gdir, M + b->off_gdirect);
+    if (b->probe_blocks)
+        k_b_probe_agg<<<static_cast<unsigned>(b->probe_blocks), kPaThreads, 0, st>>>(b->d_probe, M + b->off_probe);
     if (b->scan_chunks[0])
         k_b_scan<FilterBody><<<b->scan_grid[0], kEngineThreads, b->scan_smem[0], st>>>(
             b->d_scan[0], M + b->off_scan[0], b->d_ticket[0], b->scan_chunks[0]);
@@ -1241,6 +1270,7 @@ static tqp_status batch_prepare(tqp_ctx* ctx, const tqp_plan* plans, const tqp_r
     TQP_TRY(upload(b, b->top, &b->d_top, st));
     TQP_TRY(upload(b, b->gdir, &b->d_gdir, st));
     TQP_TRY(upload(b, b->fold, &b->d_fold, st));
+    TQP_TRY(upload(b, b->probe, &b->d_probe, st));
     b->d_levels.resize(b->levels.size());
     for (size_t L = 0; L < b->levels.size(); ++L) TQP_TRY(upload(b, b->levels[L], &b->d_levels[L], st));
     TQP_TRY(upload(b, b->maps, &b->d_maps, st));

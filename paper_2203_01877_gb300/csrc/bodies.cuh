@@ -668,11 +668,15 @@ struct PlanJoinArgs {
     ProdForm pacc[kFastSums];  // accumulator a + 1
     // Aggregation by join key first (direct-mapped tables, full tiles): each
     // fact row adds to its key's entry kacc[(fk - min) * nk + i] (count, the
-    // group sums, then the ungrouped sum), and a second kernel folds every
-    // dimension row's key entry into its group.  nullptr: off.
+    // group sums, then the ungrouped sum; three words are padded to four, so
+    // that an entry lies in one 32-byte sector), and a second kernel folds
+    // every dimension row's key entry into its group.  nullptr: off.
     unsigned long long* kacc;
-    int32_t nk;
+    int32_t nk;                // words per entry
 };
+
+// Words per key-first entry for `words` accumulators.
+inline int keyfirst_words(int words) { return words == 3 ? 4 : words; }
 
 struct PlanJoinBody {
     // One CTA per SM: the probe keeps its rows' slot loads, keys and sums in

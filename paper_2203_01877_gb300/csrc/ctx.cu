@@ -579,7 +579,7 @@ tqp_status tqp_ctx_set_tuning(tqp_ctx* ctx, int32_t tile_rows, int32_t stages, i
                     kRowQuantum, kMaxTileRows);
     if (stages < 2 || stages > kMaxStages) return fail(TQP_ERR_INVALID_ARG, "stages must be in [2, %d]", kMaxStages);
     if (ctas_per_sm < 1 || ctas_per_sm > 2) return fail(TQP_ERR_INVALID_ARG, "ctas_per_sm must be 1 or 2");
-    ctx->forced = tqp_tuning{tile_rows, stages, ctas_per_sm, 1};
+    ctx->forced = tqp_tuning{tile_rows, stages, ctas_per_sm, 1, -1};
     return TQP_OK;
 }
 

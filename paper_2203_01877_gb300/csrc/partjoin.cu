@@ -5,6 +5,7 @@
 #include "host.h"
 #include "bodies.cuh"
 #include "partjoin.cuh"
+#include "probeagg.cuh"
 
 namespace tqp {
 
@@ -297,6 +298,37 @@ static bool pj_factor_of(const ProdForm& pf, int k, const ScanGeom& G, const tqp
             return true;
         }
     return false;
+}
+
+bool lower_probe_agg(const PlanJoinArgs& J, const tqp_table* F, ProbeAggArgs* A) {
+    if (!J.pjfast || !J.fast || J.H.cap >= (1LL << 31)) return false;
+    const int nval = J.dgs ? J.S.nacc - 1 : 0;
+    if (nval > kPaVals || J.S.minmax) return false;
+    memset(A, 0, sizeof(*A));
+    A->n = F->num_rows;
+    A->ncond = J.ncond;
+    for (int q = 0; q < J.ncond; ++q)
+        A->cond[q] = PjCond{static_cast<const unsigned char*>(F->cols[J.cond[q].col].data), J.cf[q].type,
+                            J.cf[q].negate, J.cf[q].lo, J.cf[q].span};
+    A->fk = PjCol{static_cast<const unsigned char*>(F->cols[J.fk_col].data), F->cols[J.fk_col].type, 0};
+    A->nval = nval;
+    for (int a = 0; a < nval; ++a)
+        for (int k = 0; k < 2; ++k)
+            if (!pj_factor_of(J.pacc[a], k, J.G, F, &A->f[a][k])) return false;
+    A->has_sum = J.has_sum;
+    for (int k = 0; k < 2; ++k)
+        if (J.has_sum && !pj_factor_of(J.psum, k, J.G, F, &A->fs[k])) return false;
+    A->H = J.H;
+    A->next = J.next;
+    A->dgs = J.dgs;
+    A->gacc = J.S.acc;
+    A->kacc = J.kacc;
+    A->nk = J.nk;
+    A->acc = J.acc;
+    A->d_num_joined = J.d_num_joined;
+    A->d_sum = J.d_sum;
+    A->d_num_rows = J.d_num_rows;
+    return true;
 }
 
 // Scratch of the partitioned path for n fact rows and `nparts` partitions.

@@ -20,6 +20,7 @@
 #include "bodies.cuh"
 #include "dimgroups.cuh"
 #include "dim.cuh"
+#include "probeagg.cuh"
 #include "partjoin.cuh"
 
 namespace tqp {
@@ -104,6 +105,10 @@ __global__ void __launch_bounds__(kEngineThreads, PlanJoinBody::kMinBlocks) k_pl
     const PlanJoinArgs& A = stage_args(P, smem + kHeaderBytes);
     PlanJoinBody body(A, smem + kHeaderBytes + args_bytes<PlanJoinArgs>());
     run_engine(A.G, A.ctl, body, smem, args_bytes<PlanJoinArgs>());
+}
+
+__global__ void __launch_bounds__(kPaThreads, kPaMinBlocks) k_probe_agg(const __grid_constant__ ProbeAggArgs A) {
+    probe_agg_block(A, blockIdx.x, gridDim.x);
 }
 
 void lower_join_fast(PlanJoinArgs* A) {
@@ -477,7 +482,7 @@ static tqp_status run_join_plan(tqp_ctx* ctx, const tqp_plan* p, const tqp_resul
     // one pass over the build rows moves the per-key totals to the groups.
     // Used only if the table turns out direct-mapped; off when scratch is short.
     if (!parted && grouped && A.pjfast && A.fast && H.meta && F->num_rows >= 2 * std::max<long long>(1, D->num_rows)) {
-        A.nk = A.S.nacc + (A.has_sum ? 1 : 0);
+        A.nk = keyfirst_words(A.S.nacc + (A.has_sum ? 1 : 0));
         const size_t used = ctx->used;
         A.kacc = static_cast<unsigned long long*>(arena_alloc(ctx, static_cast<size_t>(H.cap) * A.nk * 8));
         if (!A.kacc) ctx->used = used;
@@ -491,15 +496,24 @@ static tqp_status run_join_plan(tqp_ctx* ctx, const tqp_plan* p, const tqp_resul
     if (parted) {
         // launched: counts, sums and group accumulators come from the partitioned kernels
     } else if (F->num_rows > 0) {
-        static SmemFlags attr_done;
-        TQP_TRY(allow_smem(ctx, reinterpret_cast<const void*>(k_plan_join), attr_done));
-        const int g = engine_grid(ctx, reinterpret_cast<const void*>(k_plan_join), smem, A.G.ntiles, tu.ctas_per_sm);
-        A.ctl.chunk_tiles = (A.G.ntiles + g - 1) / g;
-        A.ctl.nchunks = (A.G.ntiles + A.ctl.chunk_tiles - 1) / A.ctl.chunk_tiles;
-        A.ctl.ticket = sc;
-        A.ctl.err = ctx->d_err;
-        A.ctl.wait_cap = ctx->wait_cap;
-        k_plan_join<<<static_cast<int>(A.ctl.nchunks), kEngineThreads, smem, stream>>>(A);
+        // the plain-load probe for its shapes; the staged body for the rest
+        // (and where the caller set a shape of the staged scans)
+        ProbeAggArgs P;
+        if (!user_shape(ctx) && lower_probe_agg(A, F, &P)) {
+            const long long steps = (F->num_rows + kPaThreads * 4 - 1) / (kPaThreads * 4);
+            const long long g = std::min<long long>(steps, static_cast<long long>(kPaMinBlocks) * ctx->num_sms);
+            k_probe_agg<<<static_cast<unsigned>(g), kPaThreads, 0, stream>>>(P);
+        } else {
+            static SmemFlags attr_done;
+            TQP_TRY(allow_smem(ctx, reinterpret_cast<const void*>(k_plan_join), attr_done));
+            const int g = engine_grid(ctx, reinterpret_cast<const void*>(k_plan_join), smem, A.G.ntiles, tu.ctas_per_sm);
+            A.ctl.chunk_tiles = (A.G.ntiles + g - 1) / g;
+            A.ctl.nchunks = (A.G.ntiles + A.ctl.chunk_tiles - 1) / A.ctl.chunk_tiles;
+            A.ctl.ticket = sc;
+            A.ctl.err = ctx->d_err;
+            A.ctl.wait_cap = ctx->wait_cap;
+            k_plan_join<<<static_cast<int>(A.ctl.nchunks), kEngineThreads, smem, stream>>>(A);
+        }
         TQP_CUDA(cudaGetLastError());
         if (A.kacc) {
             const long long nd = D->num_rows;

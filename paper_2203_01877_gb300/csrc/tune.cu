@@ -27,11 +27,13 @@ int ht_scale(const tqp_ctx* ctx) {
 
 int tuned_variant(const tqp_ctx* ctx) {
     if (ctx->force_variant >= 0) return ctx->force_variant;
-    if (ctx->forced.tile_rows > 0) return ctx->forced.variant;
+    if (ctx->forced.tile_rows > 0) return std::max(ctx->forced.variant, 0);
     tqp_tuning t;
     if (ctx->tuner && ctx->cur_key[0] && ctx->tuner->lookup(ctx->cur_key, &t)) return t.variant;
     return 0;
 }
+
+bool user_shape(const tqp_ctx* ctx) { return ctx->forced.tile_rows > 0 && ctx->forced.variant < 0; }
 
 int row_bytes(const tqp_table* t, std::vector<int> cols) {
     std::sort(cols.begin(), cols.end());
