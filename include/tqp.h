@@ -205,7 +205,8 @@ TQP_API tqp_status tqp_ctx_set_tuning(tqp_ctx* ctx, int32_t tile_rows, int32_t s
  *     aggregation (the probe side partitioned by group, each partition
  *     aggregated in shared memory), 1 = the fused probe (every joined row
  *     added to its key's or group's accumulators with L2 reductions).
- * -1 restores the default (0, or the autotuner's choice, which times both).
+ * -1 restores the default (the autotuner's choice, which times both; else 0 for
+ * tqp_hash_join and 1, the fused probe, for grouped join plans).
  * Errors: TQP_ERR_INVALID_ARG. */
 TQP_API tqp_status tqp_ctx_set_variant(tqp_ctx* ctx, int32_t variant);
 

@@ -24,7 +24,7 @@ struct tqp_tuning {
     int stages;         // 2..kMaxStages
     int ctas_per_sm;    // 0: as many as fit
     int ht_scale;       // hash-table capacity multiplier (1 or 2: half the load factor); 0 = 1
-    int variant;        // algorithm variant of operators that have two (0 = the default; -1: a user's launch shape)
+    int variant;        // algorithm variant of operators that have two (-1: a user's launch shape, the built-in variant)
 };
 
 namespace tqp {
@@ -142,8 +142,8 @@ tqp_tuning default_tuning(const tqp_ctx* ctx, int bytes_per_row, int body_smem);
 
 // Hash-table capacity multiplier of the running call (forced or tuned; 1 by default).
 int ht_scale(const tqp_ctx* ctx);
-// Algorithm variant of the running call (forced or tuned; 0 by default).
-int tuned_variant(const tqp_ctx* ctx);
+// Algorithm variant of the running call: forced or tuned, else the operator's built-in one.
+int tuned_variant(const tqp_ctx* ctx, int built_in = 0);
 // tqp_ctx_set_tuning names a shape of the staged scans: operators that also
 // have a form without stages then take the staged one.
 bool user_shape(const tqp_ctx* ctx);

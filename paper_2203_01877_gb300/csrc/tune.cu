@@ -25,12 +25,12 @@ int ht_scale(const tqp_ctx* ctx) {
     return 1;
 }
 
-int tuned_variant(const tqp_ctx* ctx) {
+int tuned_variant(const tqp_ctx* ctx, int built_in) {
     if (ctx->force_variant >= 0) return ctx->force_variant;
-    if (ctx->forced.tile_rows > 0) return std::max(ctx->forced.variant, 0);
+    if (ctx->forced.tile_rows > 0) return ctx->forced.variant >= 0 ? ctx->forced.variant : built_in;
     tqp_tuning t;
     if (ctx->tuner && ctx->cur_key[0] && ctx->tuner->lookup(ctx->cur_key, &t)) return t.variant;
-    return 0;
+    return built_in;
 }
 
 bool user_shape(const tqp_ctx* ctx) { return ctx->forced.tile_rows > 0 && ctx->forced.variant < 0; }
