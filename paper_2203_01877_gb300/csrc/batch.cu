@@ -166,9 +166,13 @@ struct ProbeJob {
     ProbeAggArgs A;
     long long first_block, nblocks;
 };
-constexpr long long kPaRowsPerBlock = 32768;     // 32 128-row steps per warp
 constexpr int kDirArgsBytes = (static_cast<int>(sizeof(GroupDirectArgs)) + 127) / 128 * 128;
-constexpr long long kDirRowsPerBlock = 32768;    // direct kernel: 32 128-row steps per warp
+// Rows of a block of the flat row launches: at most kFlatRowsMax (32 128-row
+// steps per warp; uneven jobs balance), fewer when the batch's rows would not
+// give every SM several blocks.
+constexpr long long kFlatRowsMax = 32768;
+constexpr long long kFlatRowsMin = 4096;
+constexpr long long kFlatBlocksPerSm = 12;
 constexpr long long kDirRangeRowsPerBlock = 65536;
 
 struct TopItem {
@@ -323,11 +327,13 @@ __global__ void __launch_bounds__(kDirThreads, kDirMinBlocks) k_b_gdirect(const 
     group_direct_block<false>(A, dsm, static_cast<long long>(blockIdx.x) - j.first_block, j.nblocks);
 }
 
+template <bool kTab>
 __global__ void __launch_bounds__(kPaThreads, kPaMinBlocks) k_b_probe_agg(const ProbeJob* J, const int32_t* bjob) {
+    extern __shared__ __align__(16) uint32_t ptab[];
     __shared__ __align__(16) unsigned char args[sizeof(ProbeAggArgs)];
     const ProbeJob& j = J[bjob[blockIdx.x]];
     const ProbeAggArgs& A = stage_args(j.A, args);
-    probe_agg_block(A, static_cast<long long>(blockIdx.x) - j.first_block, j.nblocks);
+    probe_agg_block<kTab>(A, ptab, static_cast<long long>(blockIdx.x) - j.first_block, j.nblocks);
 }
 
 __global__ void __launch_bounds__(kFinThreads) k_b_finalize(const FinJob* F) {
@@ -387,12 +393,13 @@ struct tqp_batch {
     std::vector<TopJob> top;
     std::vector<DirJob> gdir;
     std::vector<FoldJob> fold;
-    std::vector<ProbeJob> probe;
+    std::vector<ProbeJob> probe[2];  // [1]: with a table in shared memory
     std::vector<std::vector<TopItem>> levels;
     // block -> job maps, concatenated
     std::vector<int32_t> maps;
     long long fill_blocks = 0, row_blocks = 0, num_blocks = 0, slot_blocks = 0, compact_blocks = 0, top0_blocks = 0,
-              sel_blocks = 0, grange_blocks = 0, gdirect_blocks = 0, fold_blocks = 0, probe_blocks = 0;
+              sel_blocks = 0, grange_blocks = 0, gdirect_blocks = 0, fold_blocks = 0;
+    long long probe_blocks[2] = {0, 0};
     long long scan_chunks[kKinds] = {0, 0, 0, 0};
     // lookup tables and outputs of the shared scans (one blob; per job its offset)
     std::vector<unsigned char> mblob;
@@ -400,7 +407,8 @@ struct tqp_batch {
     unsigned char* d_mblob = nullptr;
     std::vector<long long> level_blocks;
     size_t off_fill = 0, off_row = 0, off_num = 0, off_slot = 0, off_compact = 0, off_top0 = 0, off_sel = 0,
-           off_grange = 0, off_gdirect = 0, off_fold = 0, off_probe = 0;
+           off_grange = 0, off_gdirect = 0, off_fold = 0;
+    size_t off_probe[2] = {0, 0};
     size_t off_scan[kKinds] = {0, 0, 0, 0};
     std::vector<size_t> off_level;
     // small zeroed counters share one slab (one fill range)
@@ -416,7 +424,7 @@ struct tqp_batch {
     TopJob* d_top = nullptr;
     DirJob* d_gdir = nullptr;
     FoldJob* d_fold = nullptr;
-    ProbeJob* d_probe = nullptr;
+    ProbeJob* d_probe[2] = {nullptr, nullptr};
     std::vector<TopItem*> d_levels;
     int32_t* d_maps = nullptr;
     unsigned long long* d_ticket[kKinds] = {nullptr, nullptr, nullptr, nullptr};
@@ -616,9 +624,6 @@ static tqp_status add_group_job(tqp_batch* b, const tqp_plan* p, const tqp_resul
             D.range_nblocks = (t->num_rows + kDirRangeRowsPerBlock - 1) / kDirRangeRowsPerBlock;
             b->grange_blocks += D.range_nblocks;
         }
-        D.first_block = b->gdirect_blocks;
-        D.nblocks = (t->num_rows + kDirRowsPerBlock - 1) / kDirRowsPerBlock;
-        b->gdirect_blocks += D.nblocks;
         b->gdir.push_back(D);
         return TQP_OK;
     }
@@ -789,10 +794,7 @@ static tqp_status add_join_job(tqp_batch* b, const tqp_plan* p, const tqp_result
     }
     ProbeJob P;
     if (A.G.ntiles > 0 && lower_probe_agg(A, F, &P.A)) {
-        P.first_block = b->probe_blocks;
-        P.nblocks = (F->num_rows + kPaRowsPerBlock - 1) / kPaRowsPerBlock;
-        b->probe_blocks += P.nblocks;
-        b->probe.push_back(P);
+        b->probe[probe_agg_tab(P.A, A.S.cap, ndr) ? 1 : 0].push_back(P);
     } else if (A.G.ntiles > 0) {
         b->scan[kJobJoin - 1].push_back(J);
     } else {
@@ -1089,8 +1091,26 @@ static void plan_top_levels(tqp_batch* b) {
     }
 }
 
+// Blocks of the flat row launches, a contiguous range per job.
+template <class Job>
+static long long assign_blocks(const tqp_batch* b, std::vector<Job>& jobs) {
+    long long rows = 0;
+    for (const Job& j : jobs) rows += j.A.n;
+    const long long want = rows / (kFlatBlocksPerSm * b->ctx->num_sms);
+    const long long per = std::min(kFlatRowsMax, std::max(kFlatRowsMin, want / 1024 * 1024));
+    long long first = 0;
+    for (Job& j : jobs) {
+        j.first_block = first;
+        j.nblocks = (j.A.n + per - 1) / per;
+        first += j.nblocks;
+    }
+    return first;
+}
+
 // Block -> job maps of every flattened phase, in one array.
 static void build_maps(tqp_batch* b) {
+    b->gdirect_blocks = assign_blocks(b, b->gdir);
+    for (int k = 0; k < 2; ++k) b->probe_blocks[k] = assign_blocks(b, b->probe[k]);
     auto& M = b->maps;
     auto push = [&M](size_t j, long long nblocks) {
         for (long long k = 0; k < nblocks; ++k) M.push_back(static_cast<int32_t>(j));
@@ -1119,8 +1139,10 @@ static void build_maps(tqp_batch* b) {
     for (size_t j = 0; j < b->gdir.size(); ++j) push(j, b->gdir[j].nblocks);
     b->off_fold = M.size();
     for (size_t j = 0; j < b->fold.size(); ++j) push(j, b->fold[j].nblocks);
-    b->off_probe = M.size();
-    for (size_t j = 0; j < b->probe.size(); ++j) push(j, b->probe[j].nblocks);
+    for (int k = 0; k < 2; ++k) {
+        b->off_probe[k] = M.size();
+        for (size_t j = 0; j < b->probe[k].size(); ++j) push(j, b->probe[k][j].nblocks);
+    }
     b->off_compact = M.size();
     for (size_t j = 0; j < b->compact.size(); ++j) push(j, (b->compact[j].n + kCompactRows - 1) / kCompactRows);
     b->off_sel = M.size();
@@ -1188,8 +1210,12 @@ static tqp_status batch_launch(tqp_batch* b, cudaStream_t st) {
     if (b->gdirect_blocks)
         k_b_gdirect<<<static_cast<unsigned>(b->gdirect_blocks), kDirThreads, kDirSmemBytes + kDirArgsBytes, st>>>(
             b->d_gdir, M + b->off_gdirect);
-    if (b->probe_blocks)
-        k_b_probe_agg<<<static_cast<unsigned>(b->probe_blocks), kPaThreads, 0, st>>>(b->d_probe, M + b->off_probe);
+    if (b->probe_blocks[0])
+        k_b_probe_agg<false><<<static_cast<unsigned>(b->probe_blocks[0]), kPaThreads, 0, st>>>(b->d_probe[0],
+                                                                                              M + b->off_probe[0]);
+    if (b->probe_blocks[1])
+        k_b_probe_agg<true><<<static_cast<unsigned>(b->probe_blocks[1]), kPaThreads, kPaSmemBytes, st>>>(
+            b->d_probe[1], M + b->off_probe[1]);
     if (b->scan_chunks[0])
         k_b_scan<FilterBody><<<b->scan_grid[0], kEngineThreads, b->scan_smem[0], st>>>(
             b->d_scan[0], M + b->off_scan[0], b->d_ticket[0], b->scan_chunks[0]);
@@ -1248,9 +1274,10 @@ static tqp_status scan_shape(tqp_batch* b, int k) {
 // Lower, lay out and upload every batched job (no launch).
 static tqp_status batch_prepare(tqp_ctx* ctx, const tqp_plan* plans, const tqp_result* res, int32_t n, tqp_batch* b,
                                 cudaStream_t st) {
-    static SmemFlags attr_fin, attr_dir;
+    static SmemFlags attr_fin, attr_dir, attr_probe;
     TQP_TRY(allow_smem(ctx, reinterpret_cast<const void*>(k_b_finalize), attr_fin));
     TQP_TRY(allow_smem(ctx, reinterpret_cast<const void*>(k_b_gdirect), attr_dir));
+    TQP_TRY(allow_smem(ctx, reinterpret_cast<const void*>(k_b_probe_agg<true>), attr_probe));
     TQP_TRY(lower_batch(b, plans, res, n));
     TQP_TRY(scan_shape<FilterBody>(b, 0));
     TQP_TRY(scan_shape<GroupBody>(b, 1));
@@ -1270,7 +1297,7 @@ static tqp_status batch_prepare(tqp_ctx* ctx, const tqp_plan* plans, const tqp_r
     TQP_TRY(upload(b, b->top, &b->d_top, st));
     TQP_TRY(upload(b, b->gdir, &b->d_gdir, st));
     TQP_TRY(upload(b, b->fold, &b->d_fold, st));
-    TQP_TRY(upload(b, b->probe, &b->d_probe, st));
+    for (int k = 0; k < 2; ++k) TQP_TRY(upload(b, b->probe[k], &b->d_probe[k], st));
     b->d_levels.resize(b->levels.size());
     for (size_t L = 0; L < b->levels.size(); ++L) TQP_TRY(upload(b, b->levels[L], &b->d_levels[L], st));
     TQP_TRY(upload(b, b->maps, &b->d_maps, st));

@@ -24,6 +24,7 @@
 #include "bodies.cuh"
 #include "finalize.cuh"
 #include "groupdirect.cuh"
+#include "grouprange.cuh"
 
 namespace tqp {
 
@@ -34,7 +35,9 @@ size_t radix_sort_scratch(long long n_max);
 
 
 
-__global__ void __launch_bounds__(kEngineThreads, GroupBody::kMinBlocks) k_groupby(const __grid_constant__ GroupArgs P) {
+__global__ void __launch_bounds__(kEngineThreads, GroupBody::kMinBlocks) k_groupby(const __grid_constant__ GroupArgs P,
+                                                                                       const GroupRangePlan* rp) {
+    if (rp && rp->on) return;  // aggregated by key range
     extern __shared__ __align__(128) unsigned char smem[];
     const GroupArgs& A = stage_args(P, smem + kHeaderBytes);
     GroupBody body(A, smem + kHeaderBytes + args_bytes<GroupArgs>());
@@ -58,17 +61,74 @@ __global__ void __launch_bounds__(kDirThreads) k_groupby_dprep(const __grid_cons
     group_direct_prep_block(A, kpart, blockIdx.x, gridDim.x);
 }
 
+// ---- group-by over key columns of small range (grouprange.cuh) --------------------
+
+__global__ void __launch_bounds__(kDirThreads) k_group_range(const __grid_constant__ GroupRangeArgs A) {
+    group_range_block(A);
+}
+
+// Clears the entries, or the hash path's table.
+__global__ void __launch_bounds__(256) k_group_clear(const __grid_constant__ GroupSpec S, const GroupRangePlan* plan) {
+    const bool on = plan->on;
+    const long long tid = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
+    const long long nth = static_cast<long long>(gridDim.x) * blockDim.x;
+    const long long words = (on ? plan->entries : S.cap + 1) * S.nacc + (on ? 0 : 1);  // (ndistinct follows the table)
+    ulonglong2* p = reinterpret_cast<ulonglong2*>(S.acc);
+    for (long long i = tid; i < words / 2; i += nth) p[i] = make_ulonglong2(0, 0);
+    if (tid == 0 && words % 2) S.acc[words - 1] = 0;
+    if (on) return;
+    for (long long i = tid; i <= S.cap; i += nth) S.keys[i] = kEmptyKey;
+}
+
+__global__ void __launch_bounds__(kPaThreads, kPaMinBlocks) k_group_l2(const __grid_constant__ GroupRangeArgs A) {
+    const GroupRangePlan P = *A.plan;
+    if (!P.on || P.smem) return;
+    switch (A.nval) {
+        case 0: gr_l2_loop<1>(A, P); break;
+        case 1: gr_l2_loop<2>(A, P); break;
+        case 2: gr_l2_loop<3>(A, P); break;
+        default: gr_l2_loop<4>(A, P); break;
+    }
+}
+
+__global__ void __launch_bounds__(kGrSmemThreads, 1) k_group_smem(const __grid_constant__ GroupRangeArgs A) {
+    extern __shared__ __align__(16) uint32_t gsm[];
+    group_smem_block(A, gsm);
+}
+
+__global__ void __launch_bounds__(kGrEmitThreads) k_group_count(const __grid_constant__ GroupSpec S,
+                                                                const GroupRangePlan* plan, uint32_t* counts) {
+    if (!plan->on) return;
+    const long long e0 = static_cast<long long>(blockIdx.x) * kGrEmitPer, D = plan->entries;
+    if (e0 >= D) return;
+    int c = 0;
+    for (int s = 0; s < kGrEmitPer / kGrEmitThreads; ++s) {
+        const long long e = e0 + s * kGrEmitThreads + threadIdx.x;
+        c += __syncthreads_count(e < D && S.acc[e * S.nacc] != 0);
+    }
+    if (threadIdx.x == 0) counts[blockIdx.x] = static_cast<uint32_t>(c);
+}
+
+__global__ void __launch_bounds__(kGrEmitThreads) k_group_rows(const __grid_constant__ GroupSpec S,
+                                                               const __grid_constant__ GroupOut O,
+                                                               const GroupRangePlan* plan, const uint32_t* counts) {
+    group_rows_block(plan, S, O, counts);
+}
+
 // ---- finalize ----------------------------------------------------------------
 
 __global__ void __launch_bounds__(kFinThreads) k_groupby_finalize_small(const __grid_constant__ GroupSpec S,
-                                                                        const __grid_constant__ GroupOut O) {
+                                                                        const __grid_constant__ GroupOut O,
+                                                                        const GroupRangePlan* rp) {
+    if (rp && rp->on) return;
     extern __shared__ __align__(16) unsigned char fsm[];
     finalize_small_block(S, O, fsm);
 }
 
 // Large tables: collect (key, slot) pairs, radix sort, emit.
 __global__ void k_groupby_collect(const __grid_constant__ GroupSpec S, uint64_t* pk, uint32_t* ps,
-                                  long long* n_out) {
+                                  long long* n_out, const GroupRangePlan* rp) {
+    if (rp && rp->on) return;
     // warp-uniform trip count: blockDim is a multiple of 32
     for (long long base = blockIdx.x * static_cast<long long>(blockDim.x); base <= S.cap;
          base += static_cast<long long>(gridDim.x) * blockDim.x) {
@@ -83,7 +143,9 @@ __global__ void k_groupby_collect(const __grid_constant__ GroupSpec S, uint64_t*
 }
 
 __global__ void k_groupby_emit(const __grid_constant__ GroupSpec S, const __grid_constant__ GroupOut O,
-                               const uint64_t* pk, const uint32_t* ps, const long long* n_in) {
+                               const uint64_t* pk, const uint32_t* ps, const long long* n_in,
+                               const GroupRangePlan* rp) {
+    if (rp && rp->on) return;
     const long long G = *n_in;
     const bool overflow = static_cast<long long>(*S.ndistinct) > S.max_groups || G > O.capacity;
     if (overflow) {
@@ -194,12 +256,13 @@ tqp_status group_table_init(GroupSpec* S, void* mem, long long cap, long long ma
 }
 
 // Finalize a filled table into the caller's output arrays.
-tqp_status group_finalize(tqp_ctx* ctx, const GroupSpec& S, const GroupOut& O, cudaStream_t stream) {
+tqp_status group_finalize(tqp_ctx* ctx, const GroupSpec& S, const GroupOut& O, cudaStream_t stream,
+                          const GroupRangePlan* rp) {
     if (S.cap <= kSmallCap) {
         const size_t smem = static_cast<size_t>(2 * kSmallCap) * (8 + 4);
         static SmemFlags attr_done;
         TQP_TRY(allow_smem(ctx, reinterpret_cast<const void*>(k_groupby_finalize_small), attr_done));
-        k_groupby_finalize_small<<<1, kFinThreads, smem, stream>>>(S, O);
+        k_groupby_finalize_small<<<1, kFinThreads, smem, stream>>>(S, O, rp);
         TQP_CUDA(cudaGetLastError());
         return TQP_OK;
     }
@@ -216,14 +279,14 @@ tqp_status group_finalize(tqp_ctx* ctx, const GroupSpec& S, const GroupOut& O, c
     TQP_CUDA(cudaMemsetAsync(d_n, 0, sizeof(long long), stream));
     const int threads = 256;
     const int blocks = static_cast<int>(std::min<long long>((nmax + threads - 1) / threads, ctx->num_sms * 8LL));
-    k_groupby_collect<<<blocks, threads, 0, stream>>>(S, k0, v0, d_n);
+    k_groupby_collect<<<blocks, threads, 0, stream>>>(S, k0, v0, d_n, rp);
     bool in1 = false;
     const int end_bit = (S.width + 7) / 8 * 8;
     TQP_TRY(radix_sort_pairs(k0, v0, k1, v1, d_n, nmax, 0, end_bit, rs, stream, &in1));
     const int eblocks = static_cast<int>(
         std::max<long long>(1, std::min<long long>((std::min(nmax, O.capacity) + threads - 1) / threads,
                                                    ctx->num_sms * 8LL)));
-    k_groupby_emit<<<eblocks, threads, 0, stream>>>(S, O, in1 ? k1 : k0, in1 ? v1 : v0, d_n);
+    k_groupby_emit<<<eblocks, threads, 0, stream>>>(S, O, in1 ? k1 : k0, in1 ? v1 : v0, d_n, rp);
     TQP_CUDA(cudaGetLastError());
     return TQP_OK;
 }
@@ -386,6 +449,72 @@ bool lower_group_direct(const tqp_table* t, const GroupArgs& A, long long max_gr
     return lane_bytes <= kDirLaneBytes;
 }
 
+// Lower the hash path's query to the form over key ranges: conditions, keys and
+// factors of at most kGrVals sums on plain columns.
+static bool lower_group_range(const tqp_table* t, const GroupArgs& A, GroupRangeArgs* R) {
+    const int nval = A.S.nacc - 1;
+    if (t->num_rows <= 0 || A.S.ngc < 1 || nval > kGrVals || A.S.minmax) return false;
+    ScanGeom G;
+    memset(&G, 0, sizeof(G));
+    G.n = t->num_rows;
+    G.ncols = t->num_cols;
+    for (int c = 0; c < t->num_cols; ++c) {
+        G.col[c].type = t->cols[c].type;
+        G.col[c].slot = 0;
+        G.col[c].soff = c;
+    }
+    auto ptr = [&](int c) { return static_cast<const unsigned char*>(t->cols[c].data); };
+    memset(R, 0, sizeof(*R));
+    R->n = t->num_rows;
+    CondFast cf[TQP_MAX_PREDS];
+    int32_t fast = 0;
+    lower_fast(A.cond, A.ncond, G, cf, &fast);
+    if (!fast) return false;
+    R->ncond = A.ncond;
+    for (int q = 0; q < A.ncond; ++q)
+        R->cond[q] = PjCond{ptr(cf[q].soff), cf[q].type, cf[q].negate, cf[q].lo, cf[q].span};
+    R->ngc = A.S.ngc;
+    for (int i = 0; i < A.S.ngc; ++i) {
+        const int c = A.S.key_col[i];
+        R->key[i] = PjCol{ptr(c), t->cols[c].type, 0};
+    }
+    R->nval = nval;
+    for (int a = 0; a < nval; ++a) {
+        ProdForm pf;
+        if (!lower_prod(A.S.acc_expr[a], G, &pf)) return false;
+        for (int k = 0; k < 2; ++k) {
+            const bool col = pf.kind[k] != kFacConst;
+            R->f[a][k] = PjFactor{col ? ptr(pf.soff[k]) : nullptr, col ? pf.type[k] : 0, pf.kind[k], pf.a[k], pf.b[k]};
+        }
+    }
+    return true;
+}
+
+// The kernels over key ranges; the hash path's that follow them return at once
+// when the plan turns out on.
+static tqp_status launch_group_range(tqp_ctx* ctx, const GroupSpec& S, const GroupOut& O, GroupRangeArgs& R,
+                                     GroupRangePlan* plan, uint32_t* counts, cudaStream_t stream) {
+    R.plan = plan;
+    R.acc = S.acc;
+    R.max_entries = std::min<long long>(S.cap + 1, kGrMaxEntries);
+    const long long n = R.n, sms = ctx->num_sms;
+    auto grid = [](long long work, long long per, long long most) {
+        return static_cast<unsigned>(std::max<long long>(1, std::min<long long>((work + per - 1) / per, most)));
+    };
+    TQP_CUDA(cudaMemsetAsync(plan, 0, sizeof(*plan), stream));
+    k_group_range<<<grid(n, 8192, 4 * sms), kDirThreads, 0, stream>>>(R);
+    k_group_clear<<<grid((S.cap + 1) * S.nacc, 4096, 8 * sms), 256, 0, stream>>>(S, plan);
+    static SmemFlags attr_done;
+    TQP_TRY(allow_smem(ctx, reinterpret_cast<const void*>(k_group_smem), attr_done));
+    k_group_smem<<<grid(n, kGrSmemThreads * 4, sms), kGrSmemThreads, kGrSmemBytes, stream>>>(R);
+    k_group_l2<<<grid(n, kPaThreads * 4, kPaMinBlocks * sms), kPaThreads, 0, stream>>>(R);
+    const unsigned eb = grid(R.max_entries, kGrEmitPer, kGrMaxEntries / kGrEmitPer + 1);
+    k_group_count<<<eb, kGrEmitThreads, 0, stream>>>(S, plan, counts);
+    k_group_rows<<<eb, kGrEmitThreads, 0, stream>>>(S, O, plan, counts);
+    TQP_CUDA(cudaGetLastError());
+    return TQP_OK;
+}
+
 tqp_status launch_sort_agg(tqp_ctx* ctx, const tqp_table* t, const Cond* cond, int ncond, GroupSpec* S,
                            long long cap_groups, cudaStream_t stream);
 
@@ -459,7 +588,22 @@ tqp_status launch_groupby(tqp_ctx* ctx, const tqp_table* t, const tqp_pred* pred
     unsigned long long* ticket = static_cast<unsigned long long*>(arena_alloc(ctx, 256));
     if (!tab || !ticket) return arena_oom(ctx, group_table_bytes(cap, A.S.nacc));
     GroupOut O{d_keys, d_ivals, d_fvals, capacity_groups, d_num_groups, ctx->d_err};
-    TQP_TRY(group_table_init(&A.S, tab, cap, max_groups, stream, !direct));
+    // over key ranges, if they turn out small (and the caller set no shape of the staged scans)
+    GroupRangeArgs R;
+    GroupRangePlan* rp = nullptr;
+    uint32_t* counts = nullptr;
+    if (!direct && topk == 0 && !user_shape(ctx) && lower_group_range(t, A, &R)) {
+        const size_t used = ctx->used;
+        rp = static_cast<GroupRangePlan*>(arena_alloc(ctx, sizeof(GroupRangePlan)));
+        const long long blocks = (std::min<long long>(cap + 1, kGrMaxEntries) + kGrEmitPer - 1) / kGrEmitPer;
+        counts = static_cast<uint32_t*>(arena_alloc(ctx, static_cast<size_t>(blocks) * 4));
+        if (!rp || !counts) {
+            rp = nullptr;
+            ctx->used = used;
+        }
+    }
+    TQP_TRY(group_table_init(&A.S, tab, cap, max_groups, stream, !direct && !rp));
+    if (rp) TQP_TRY(launch_group_range(ctx, A.S, O, R, rp, counts, stream));
     if (direct) {
         // two launches: the range pass (which also clears the table), then the
         // aggregation, whose last CTA finalizes the table unless top-k follows
@@ -519,11 +663,11 @@ tqp_status launch_groupby(tqp_ctx* ctx, const tqp_table* t, const tqp_pred* pred
         A.ctl.err = ctx->d_err;
         A.ctl.wait_cap = ctx->wait_cap;
         TQP_CUDA(cudaMemsetAsync(ticket, 0, 8, stream));
-        k_groupby<<<static_cast<int>(A.ctl.nchunks), kEngineThreads, smem, stream>>>(A);
+        k_groupby<<<static_cast<int>(A.ctl.nchunks), kEngineThreads, smem, stream>>>(A, rp);
         TQP_CUDA(cudaGetLastError());
     }
     if (topk > 0) return group_topk(ctx, A.S, O, topk, topk_agg, d_total_groups, stream);
-    return group_finalize(ctx, A.S, O, stream);
+    return group_finalize(ctx, A.S, O, stream, rp);
 }
 
 }  // namespace tqp

@@ -753,7 +753,8 @@ __device__ __forceinline__ void dir_enc_update(long long x, unsigned long long& 
     mn = ~e > mn ? ~e : mn;
 }
 
-__device__ __forceinline__ void group_direct_range_block(const GroupDirectArgs& A, unsigned long long* kmeta,
+template <class Args>  // (n rows, ngc key columns key[])
+__device__ __forceinline__ void group_direct_range_block(const Args& A, unsigned long long* kmeta,
                                                          unsigned long long* kpart, long long vb, long long vg) {
     __shared__ unsigned long long red[kDirThreads / 32][2];
     const int lane = threadIdx.x % 32, w = threadIdx.x / 32;

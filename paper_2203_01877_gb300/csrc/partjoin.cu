@@ -321,6 +321,7 @@ bool lower_probe_agg(const PlanJoinArgs& J, const tqp_table* F, ProbeAggArgs* A)
     A->H = J.H;
     A->next = J.next;
     A->dgs = J.dgs;
+    A->d_groups = J.S.d_dense_n;
     A->gacc = J.S.acc;
     A->kacc = J.kacc;
     A->nk = J.nk;

@@ -110,8 +110,10 @@ __global__ void __launch_bounds__(kEngineThreads, PlanJoinBody::kMinBlocks) k_pl
     run_engine(A.G, A.ctl, body, smem, args_bytes<PlanJoinArgs>());
 }
 
+template <bool kTab>
 __global__ void __launch_bounds__(kPaThreads, kPaMinBlocks) k_probe_agg(const __grid_constant__ ProbeAggArgs A) {
-    probe_agg_block(A, blockIdx.x, gridDim.x);
+    extern __shared__ __align__(16) uint32_t ptab[];
+    probe_agg_block<kTab>(A, ptab, blockIdx.x, gridDim.x);
 }
 
 void lower_join_fast(PlanJoinArgs* A) {
@@ -505,7 +507,13 @@ static tqp_status run_join_plan(tqp_ctx* ctx, const tqp_plan* p, const tqp_resul
         if (!user_shape(ctx) && lower_probe_agg(A, F, &P)) {
             const long long steps = (F->num_rows + kPaThreads * 4 - 1) / (kPaThreads * 4);
             const long long g = std::min<long long>(steps, static_cast<long long>(kPaMinBlocks) * ctx->num_sms);
-            k_probe_agg<<<static_cast<unsigned>(g), kPaThreads, 0, stream>>>(P);
+            if (probe_agg_tab(P, A.S.cap, D->num_rows)) {
+                static SmemFlags attr_done;
+                TQP_TRY(allow_smem(ctx, reinterpret_cast<const void*>(k_probe_agg<true>), attr_done));
+                k_probe_agg<true><<<static_cast<unsigned>(g), kPaThreads, kPaSmemBytes, stream>>>(P);
+            } else {
+                k_probe_agg<false><<<static_cast<unsigned>(g), kPaThreads, 0, stream>>>(P);
+            }
         } else {
             static SmemFlags attr_done;
             TQP_TRY(allow_smem(ctx, reinterpret_cast<const void*>(k_plan_join), attr_done));

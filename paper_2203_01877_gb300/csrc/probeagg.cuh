@@ -16,7 +16,10 @@
 //     instruction with neighbouring lanes holding neighbouring words: an L2
 //     reduction costs per 32-byte sector an instruction touches, not per word
 //     (60M random 16-byte entries: 585 us with a reduction per word, 291 us
-//     with a lane pair; 32-byte entries: 1166 against 464 us).
+//     with a lane pair; 32-byte entries: 1166 against 464 us);
+//   * reductions on one 128-byte line serialise (2.5 ns each), so entries that
+//     fit a CTA's shared memory are accumulated there and flushed once, and
+//     the rows of an entry that is hot in a warp are added up before they go.
 // Lane l of a step handles rows 2l, 2l + 1, 64 + 2l and 64 + 2l + 1: loads of
 // 1-, 4- and 8-byte columns are all contiguous across the warp.
 #pragma once
@@ -32,6 +35,7 @@ constexpr int kPaMinBlocks = 3;      // 24 warps per SM: 85 registers
 constexpr int kPaStep = 4 * kWarp;   // rows of a warp step
 constexpr int kPaVals = 2;           // group sums
 constexpr uint32_t kPaNone = 0xFFFFFFFFu;
+constexpr int kPaSmemBytes = 64 * 1024;  // the CTA's entries: a 32-bit count and 64-bit sums each
 
 struct ProbeAggArgs {
     long long n;              // fact rows
@@ -46,6 +50,7 @@ struct ProbeAggArgs {
     JoinHT H;                 // cap < 2^31
     const uint32_t* next;     // chained build: next dim row of the same key
     const uint32_t* dgs;      // dim row -> dense group id; nullptr: no aggregation
+    const long long* d_groups; // groups (entries of gacc)
     unsigned long long* gacc; // dense group accumulators, nval + 1 words each
     unsigned long long* kacc; // key-first entries (direct-mapped tables), nullptr: off
     unsigned long long* acc;  // [0] joined, [1] sum, [2] passing fact rows, [3] finished blocks (zeroed)
@@ -123,8 +128,8 @@ __device__ __forceinline__ void pa_prod(const PjFactor (&f)[2], long long r0, in
 }
 
 // Pass bits of the lane's rows (those in `in`).
-template <bool kFull>
-__device__ __forceinline__ uint32_t pa_conds(const ProbeAggArgs& A, long long r0, int lane, uint32_t in) {
+template <bool kFull, class Args>
+__device__ __forceinline__ uint32_t pa_conds(const Args& A, long long r0, int lane, uint32_t in) {
     uint32_t ok = in;
     for (int q = 0; q < A.ncond; ++q) {
         const PjCond& c = A.cond[q];
@@ -171,10 +176,79 @@ __device__ __forceinline__ void pa_red(unsigned long long* base, uint32_t stride
     }
 }
 
+// The step's rows of a hot entry, summed over the warp and added once. `hot` is
+// the entry last seen in several lanes of a step's first row; an entry that more
+// lanes hold takes its place. Absorbed rows are set to kPaNone. All lanes call it.
+template <int W>
+__device__ __forceinline__ void pa_combine(unsigned long long* base, uint32_t stride, uint32_t (&e)[4],
+                                           const int64_t (&x0)[4], const int64_t (&x1)[4], const int64_t (&x2)[4],
+                                           int lane, uint32_t& hot) {
+    const uint32_t c = __shfl_sync(0xffffffffu, e[0], 0);
+    const int m = c == kPaNone ? 0 : __popc(__ballot_sync(0xffffffffu, e[0] == c));
+    int h = hot == kPaNone ? 0 : __popc(__ballot_sync(0xffffffffu, e[0] == hot));
+    if (m > 1 && m > h) {
+        hot = c;
+        h = m;
+    }
+    if (h < 2) return;
+    unsigned long long t[W] = {};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (e[j] != hot) continue;
+        t[0] += 1;
+        if (W > 1) t[W > 1 ? 1 : 0] += static_cast<unsigned long long>(x0[j]);
+        if (W > 2) t[W > 2 ? 2 : 0] += static_cast<unsigned long long>(x1[j]);
+        if (W > 3) t[W > 3 ? 3 : 0] += static_cast<unsigned long long>(x2[j]);
+        e[j] = kPaNone;
+    }
+#pragma unroll
+    for (int a = 0; a < W; ++a) {
+        const unsigned long long s = static_cast<unsigned long long>(group_sum_i64(0xffffffffu, static_cast<long long>(t[a])));
+        if (lane == 0) red_add_u64(base + static_cast<unsigned long long>(hot) * stride + a, s);
+    }
+}
+
+// x added to entry e of a CTA's table of D entries: D counts, then per value D
+// low and D high words (the low word's atomic returns what the carry needs).
+__device__ __forceinline__ void pa_smem_add(uint32_t* tab, uint32_t D, uint32_t e, int nv,
+                                            const unsigned long long (&x)[3]) {
+    atomicAdd(&tab[e], 1u);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        if (a >= nv) break;
+        uint32_t* lo = tab + (1 + 2 * a) * D + e;
+        const uint32_t xl = static_cast<uint32_t>(x[a]);
+        const uint32_t old = atomicAdd(lo, xl);
+        const uint32_t xh = static_cast<uint32_t>(x[a] >> 32) + (old + xl < old ? 1u : 0u);
+        if (xh) atomicAdd(lo + D, xh);
+    }
+}
+
+// The table into global entries of nv + 1 words (neighbouring words on neighbouring lanes).
+__device__ __forceinline__ void pa_smem_flush(const uint32_t* tab, uint32_t D, int nv, unsigned long long* base,
+                                              uint32_t stride) {
+    const uint32_t W = nv + 1;
+    for (uint32_t i = threadIdx.x; i < D * W; i += blockDim.x) {
+        const uint32_t e = i / W, a = i % W;
+        unsigned long long x = tab[e];
+        if (a > 0 && x) {
+            const uint32_t* lo = tab + (2 * a - 1) * D + e;
+            x = static_cast<unsigned long long>(lo[0]) | (static_cast<unsigned long long>(lo[D]) << 32);
+        }
+        if (x) red_add_u64(base + static_cast<unsigned long long>(e) * stride + a, x);
+    }
+}
+
 // A joined row of a key with several build rows: added to each of their groups.
-static __device__ __noinline__ void pa_add_chain(const ProbeAggArgs& A, uint32_t d, uint32_t cnt,
-                                                 unsigned long long x0, unsigned long long x1) {
+static __device__ __noinline__ void pa_add_chain(const ProbeAggArgs& A, uint32_t* tab, uint32_t D, uint32_t d,
+                                                 uint32_t cnt, unsigned long long x0, unsigned long long x1) {
     for (uint32_t k = 0; k < cnt; ++k) {
+        if (tab) {
+            const unsigned long long x[3] = {x0, x1, 0};
+            pa_smem_add(tab, D, __ldg(&A.dgs[d]), A.nval, x);
+            if (k + 1 < cnt) d = __ldg(&A.next[d]);
+            continue;
+        }
         unsigned long long* a = A.gacc + static_cast<long long>(__ldg(&A.dgs[d])) * (A.nval + 1);
         red_add_u64(&a[0], 1ULL);
         if (A.nval > 0) red_add_u64(&a[1], x0);
@@ -191,9 +265,11 @@ struct PaTotals {
 // One warp step.  kKey: aggregate by join key (direct-mapped tables): W words
 // per entry of A.kacc, no slot load; otherwise look the key up and add to the
 // group of its build row(s), W = nval + 1 words (W = 0: no aggregation).
-template <bool kFull, bool kKey, int W>
+// kSmem: into the CTA's table `tab` of D entries.
+template <bool kFull, bool kKey, bool kSmem, int W>
 __device__ __forceinline__ void pa_step(const ProbeAggArgs& A, long long r0, int lane, bool direct, long long kmin,
-                                        unsigned long long krange, PaTotals& T) {
+                                        unsigned long long krange, uint32_t* tab, uint32_t D, PaTotals& T,
+                                        uint32_t& hot) {
     uint32_t in = 0xFu;
     if constexpr (!kFull) {
         in = 0;
@@ -213,15 +289,24 @@ __device__ __forceinline__ void pa_step(const ProbeAggArgs& A, long long r0, int
     if (!__any_sync(0xffffffffu, ok)) return;
     T.passed += __popc(ok);
     if constexpr (kKey) {
+        uint32_t e[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const unsigned long long d = static_cast<uint64_t>(key[j]) - static_cast<uint64_t>(kmin);
-            const uint32_t e = ((ok >> j) & 1u) && d < krange ? static_cast<uint32_t>(d) : kPaNone;
-            unsigned long long x[3] = {static_cast<unsigned long long>(v0[j]), static_cast<unsigned long long>(v1[j]),
-                                       static_cast<unsigned long long>(vs[j])};
-            if (A.nval < 1) x[0] = x[2];
-            if (A.nval < 2) x[1] = x[2];
-            pa_red<W>(A.kacc, static_cast<uint32_t>(A.nk), e, x, lane);
+            e[j] = ((ok >> j) & 1u) && d < krange ? static_cast<uint32_t>(d) : kPaNone;
+            if (A.nval < 1) v0[j] = vs[j];  // (the ungrouped sum follows the group sums)
+            if (A.nval < 2) v1[j] = vs[j];
+        }
+        if constexpr (!kSmem) pa_combine<W>(A.kacc, static_cast<uint32_t>(A.nk), e, v0, v1, vs, lane, hot);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const unsigned long long x[3] = {static_cast<unsigned long long>(v0[j]), static_cast<unsigned long long>(v1[j]),
+                                             static_cast<unsigned long long>(vs[j])};
+            if constexpr (kSmem) {
+                if (e[j] != kPaNone) pa_smem_add(tab, D, e[j], W - 1, x);
+            } else {
+                pa_red<W>(A.kacc, static_cast<uint32_t>(A.nk), e[j], x, lane);
+            }
         }
         return;
     }
@@ -258,61 +343,96 @@ __device__ __forceinline__ void pa_step(const ProbeAggArgs& A, long long r0, int
             if (sk != k) sl[j].w = 0;
         }
     }
+    uint32_t e[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        uint32_t e = kPaNone;
+        e[j] = kPaNone;
         const uint32_t cnt = sl[j].w;
         if (cnt) {
             T.joined += cnt;
             T.sum += vs[j] * static_cast<long long>(cnt);
             if (W > 0) {
-                if (sl[j].z & kDirectGroup) e = sl[j].z & ~kDirectGroup;
-                else pa_add_chain(A, sl[j].z, cnt, static_cast<unsigned long long>(v0[j]), static_cast<unsigned long long>(v1[j]));
+                if (sl[j].z & kDirectGroup) e[j] = sl[j].z & ~kDirectGroup;
+                else pa_add_chain(A, kSmem ? tab : nullptr, D, sl[j].z, cnt, static_cast<unsigned long long>(v0[j]),
+                                  static_cast<unsigned long long>(v1[j]));
             }
         }
-        if constexpr (W > 0) {
+    }
+    if constexpr (W > 0) {
+        if constexpr (!kSmem) {
             __syncwarp();
+            pa_combine<W>(A.gacc, W, e, v0, v1, vs, lane, hot);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
             const unsigned long long x[3] = {static_cast<unsigned long long>(v0[j]),
                                              static_cast<unsigned long long>(v1[j]), 0};
-            pa_red<W>(A.gacc, static_cast<uint32_t>(W), e, x, lane);
+            if constexpr (kSmem) {
+                if (e[j] != kPaNone) pa_smem_add(tab, D, e[j], W - 1, x);
+            } else {
+                pa_red<W>(A.gacc, static_cast<uint32_t>(W), e[j], x, lane);
+            }
         }
     }
 }
 
-template <bool kKey, int W>
+template <bool kKey, bool kSmem, int W>
 __device__ __forceinline__ void pa_loop(const ProbeAggArgs& A, bool direct, long long kmin, unsigned long long krange,
-                                        long long vb, long long vg, PaTotals& T) {
+                                        long long vb, long long vg, uint32_t* tab, uint32_t D, PaTotals& T) {
     const int lane = threadIdx.x % kWarp, w = threadIdx.x / kWarp;
     const long long stride = vg * (kPaThreads / kWarp) * kPaStep;
+    uint32_t hot = kPaNone;
     for (long long r0 = (vb * (kPaThreads / kWarp) + w) * kPaStep; r0 < A.n; r0 += stride) {
-        if (r0 + kPaStep <= A.n) pa_step<true, kKey, W>(A, r0, lane, direct, kmin, krange, T);
-        else pa_step<false, kKey, W>(A, r0, lane, direct, kmin, krange, T);
+        if (r0 + kPaStep <= A.n) pa_step<true, kKey, kSmem, W>(A, r0, lane, direct, kmin, krange, tab, D, T, hot);
+        else pa_step<false, kKey, kSmem, W>(A, r0, lane, direct, kmin, krange, tab, D, T, hot);
     }
 }
 
-// Block vb of vg working on this plan.
-static __device__ __forceinline__ void probe_agg_block(const ProbeAggArgs& A, long long vb, long long vg) {
+template <bool kSmem>
+__device__ __forceinline__ void pa_run(const ProbeAggArgs& A, bool bykey, bool direct, long long kmin,
+                                       unsigned long long krange, long long vb, long long vg, uint32_t* tab, uint32_t D,
+                                       PaTotals& T) {
+    if (bykey) {
+        switch (A.nval + 1 + (A.has_sum ? 1 : 0)) {
+            case 1: pa_loop<true, kSmem, 1>(A, direct, kmin, krange, vb, vg, tab, D, T); break;
+            case 2: pa_loop<true, kSmem, 2>(A, direct, kmin, krange, vb, vg, tab, D, T); break;
+            case 3: pa_loop<true, kSmem, 3>(A, direct, kmin, krange, vb, vg, tab, D, T); break;
+            default: pa_loop<true, kSmem, 4>(A, direct, kmin, krange, vb, vg, tab, D, T); break;
+        }
+    } else {
+        switch (A.dgs ? A.nval + 1 : 0) {
+            case 0: pa_loop<false, false, 0>(A, direct, kmin, 0, vb, vg, nullptr, 0, T); break;
+            case 1: pa_loop<false, kSmem, 1>(A, direct, kmin, 0, vb, vg, tab, D, T); break;
+            case 2: pa_loop<false, kSmem, 2>(A, direct, kmin, 0, vb, vg, tab, D, T); break;
+            default: pa_loop<false, kSmem, 3>(A, direct, kmin, 0, vb, vg, tab, D, T); break;
+        }
+    }
+}
+
+// Block vb of vg working on this plan. kTab: the launch gave it a table of
+// kPaSmemBytes (a plan whose entries cannot fit it leaves the memory to L1).
+template <bool kTab>
+__device__ __forceinline__ void probe_agg_block(const ProbeAggArgs& A, uint32_t* tab, long long vb, long long vg) {
     __shared__ unsigned long long red[3][kPaThreads / kWarp];
     const int lane = threadIdx.x % kWarp, w = threadIdx.x / kWarp;
     long long kmin = 0;
     const bool direct = ht_is_direct(A.H, &kmin);
     const bool bykey = direct && A.kacc != nullptr;
+    const unsigned long long krange = bykey ? static_cast<unsigned long long>(__ldg(&A.H.meta[1]) - kmin) + 1 : 0;
+    // the CTA's own table: it must fit, and be worth clearing and flushing
+    const int nv = A.nval + (bykey && A.has_sum ? 1 : 0);
+    const long long D = bykey ? static_cast<long long>(krange) : (A.dgs ? __ldg(A.d_groups) : 0);
+    const bool smem = kTab && D > 0 && D * (4 + 8 * nv) <= kPaSmemBytes && A.n / vg >= 4 * D;
     PaTotals T;
-    if (bykey) {
-        const unsigned long long krange = static_cast<unsigned long long>(__ldg(&A.H.meta[1]) - kmin) + 1;
-        switch (A.nval + 1 + (A.has_sum ? 1 : 0)) {
-            case 1: pa_loop<true, 1>(A, direct, kmin, krange, vb, vg, T); break;
-            case 2: pa_loop<true, 2>(A, direct, kmin, krange, vb, vg, T); break;
-            case 3: pa_loop<true, 3>(A, direct, kmin, krange, vb, vg, T); break;
-            default: pa_loop<true, 4>(A, direct, kmin, krange, vb, vg, T); break;
-        }
+    if (kTab && smem) {
+        for (int i = threadIdx.x; i < D * (1 + 2 * nv); i += kPaThreads) tab[i] = 0;
+        __syncthreads();
+        pa_run<kTab>(A, bykey, direct, kmin, krange, vb, vg, tab, static_cast<uint32_t>(D), T);
+        __syncthreads();
+        pa_smem_flush(tab, static_cast<uint32_t>(D), nv, bykey ? A.kacc : A.gacc,
+                      bykey ? static_cast<uint32_t>(A.nk) : static_cast<uint32_t>(nv + 1));
     } else {
-        switch (A.dgs ? A.nval + 1 : 0) {
-            case 0: pa_loop<false, 0>(A, direct, kmin, 0, vb, vg, T); break;
-            case 1: pa_loop<false, 1>(A, direct, kmin, 0, vb, vg, T); break;
-            case 2: pa_loop<false, 2>(A, direct, kmin, 0, vb, vg, T); break;
-            default: pa_loop<false, 3>(A, direct, kmin, 0, vb, vg, T); break;
-        }
+        pa_run<false>(A, bykey, direct, kmin, krange, vb, vg, nullptr, 0, T);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -339,6 +459,13 @@ static __device__ __forceinline__ void probe_agg_block(const ProbeAggArgs& A, lo
     if (A.d_num_joined && !bykey) *A.d_num_joined = static_cast<int64_t>(atomicAdd(&A.acc[0], 0ULL));
     if (A.d_sum && !bykey) *A.d_sum = static_cast<int64_t>(atomicAdd(&A.acc[1], 0ULL));
     if (A.d_num_rows) *A.d_num_rows = static_cast<int64_t>(atomicAdd(&A.acc[2], 0ULL));
+}
+
+// Host: whether the launch should give the plan a table of its own, from what
+// is known before the key range and the groups are: their upper bounds.
+inline bool probe_agg_tab(const ProbeAggArgs& A, long long max_groups, long long build_rows) {
+    const int per = 4 + 8 * (A.nval + (A.has_sum ? 1 : 0));
+    return A.dgs && (max_groups * (4 + 8 * A.nval) <= kPaSmemBytes || (A.kacc && build_rows * per <= kPaSmemBytes));
 }
 
 // Host (partjoin.cu): lower the staged probe's arguments (closed forms over

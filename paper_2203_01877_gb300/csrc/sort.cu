@@ -27,6 +27,7 @@ __global__ void __launch_bounds__(kSortThreads) k_rs_upsweep(const uint64_t* __r
                                                              unsigned long long* __restrict__ digit_tot) {
     __shared__ uint32_t cnt[256];
     const long long n = *n_ptr;
+    if (n == 0) return;
     const long long tile = blockIdx.x;
     const long long base = tile * kSortTile;
     cnt[threadIdx.x] = 0;
@@ -44,7 +45,9 @@ __global__ void __launch_bounds__(kSortThreads) k_rs_upsweep(const uint64_t* __r
 }
 
 __global__ void __launch_bounds__(1024) k_rs_scan(uint32_t* __restrict__ hist, long long ntiles,
-                                                  const unsigned long long* __restrict__ digit_tot) {
+                                                  const unsigned long long* __restrict__ digit_tot,
+                                                  const long long* __restrict__ n_ptr) {
+    if (*n_ptr == 0) return;
     __shared__ unsigned long long wsum[32];
     __shared__ unsigned long long carry_sm;
     const int d = blockIdx.x;
@@ -169,7 +172,7 @@ tqp_status radix_sort_pairs(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* 
         TQP_CUDA(cudaMemsetAsync(digit_tot, 0, 256 * sizeof(unsigned long long), stream));
         k_rs_upsweep<<<static_cast<unsigned>(ntiles), kSortThreads, 0, stream>>>(ki, d_n, shift, hist, ntiles,
                                                                                  digit_tot);
-        k_rs_scan<<<256, 1024, 0, stream>>>(hist, ntiles, digit_tot);
+        k_rs_scan<<<256, 1024, 0, stream>>>(hist, ntiles, digit_tot, d_n);
         k_rs_downsweep<<<static_cast<unsigned>(ntiles), kSortThreads, 0, stream>>>(ki, vi, ko, vo, d_n, shift, hist,
                                                                                    ntiles);
         TQP_CUDA(cudaGetLastError());
