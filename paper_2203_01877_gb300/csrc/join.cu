@@ -15,12 +15,17 @@
 //          remembered, matches are counted per chunk, a decoupled look-back
 //          over chunks gives each chunk's output offset, and each row's run
 //          is copied out as (build, probe) pairs.
+// That is the form for a caller's launch shape of the staged scans, and its
+// probe the one of the sort-based build; the built-in path is joinpairs.cuh
+// (a table of one sector per probe, the sort only when some key repeats, one
+// pass over the probe keys).
 // Keys compare by their int64 value; int32, int64 and uint8 key columns mix.
 #include <cstdio>
 
 #include "host.h"
 #include "join.cuh"
 #include "dimgroups.cuh"
+#include "joinpairs.cuh"
 
 namespace tqp {
 
@@ -497,11 +502,125 @@ __global__ void __launch_bounds__(kEngineThreads, 2) k_join_probe(const __grid_c
     run_engine(A.G, A.ctl, body, smem, args_bytes<ProbeArgs>());
 }
 
+// ---- one-pass pairs (joinpairs.cuh) -----------------------------------------------
+
+__global__ void k_pair_insert(PairTable T, const unsigned char* key_col, int key_type, long long n, uint64_t* sort_key,
+                              uint32_t* sort_val, long long* n_sort) {
+    unsigned long long lo = 0, range = 0;
+    const bool direct = pt_direct(T, &lo, &range);
+    bool dup = false;
+    for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n;
+         i += static_cast<long long>(gridDim.x) * blockDim.x) {
+        unsigned long long s;
+        dup |= pt_insert(T, direct, lo, static_cast<uint64_t>(ldg_typed(key_col, key_type, i)), static_cast<uint32_t>(i), &s);
+        sort_key[i] = s;
+        sort_val[i] = static_cast<uint32_t>(i);
+    }
+    if (dup) *n_sort = n;  // (every writer stores the same)
+}
+
+// After the sort, when some key repeats: the run starts into the value words
+// (a key of one row keeps its row), then each run's length at its start.
+__global__ void k_pair_runs(PairTable T, const uint64_t* skey, const long long* n_sort) {
+    const long long n = *n_sort;
+    unsigned long long lo = 0, range = 0;
+    const bool direct = pt_direct(T, &lo, &range);
+    for (long long p = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; p < n;
+         p += static_cast<long long>(gridDim.x) * blockDim.x) {
+        const uint64_t s = skey[p];
+        if ((p == 0 || skey[p - 1] != s) && p + 1 < n && skey[p + 1] == s)
+            *pt_value(T, direct, s) = static_cast<uint32_t>(p);
+    }
+}
+
+__global__ void k_pair_lens(PairTable T, const uint64_t* skey, const long long* n_sort, uint32_t* rlen) {
+    const long long n = *n_sort;
+    unsigned long long lo = 0, range = 0;
+    const bool direct = pt_direct(T, &lo, &range);
+    for (long long p = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; p < n;
+         p += static_cast<long long>(gridDim.x) * blockDim.x) {
+        const uint64_t s = skey[p];
+        if (p > 0 && skey[p - 1] == s && (p + 1 == n || skey[p + 1] != s)) {
+            const uint32_t start = *pt_value(T, direct, s);
+            rlen[start] = static_cast<uint32_t>(p) - start + 1;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kJpThreads, kJpMinBlocks) k_join_pairs(const __grid_constant__ PairArgs A) {
+    join_pairs_tile(A);
+}
+
+static tqp_status launch_join_pairs(tqp_ctx* ctx, const tqp_table* build, int32_t build_key, const tqp_table* probe,
+                                    int32_t probe_key, int32_t kind, int32_t* d_build_idx, int32_t* d_probe_idx,
+                                    int64_t capacity, int64_t* d_count, cudaStream_t stream) {
+    const tqp_column &bc = build->cols[build_key], &pc = probe->cols[probe_key];
+    const long long nb = build->num_rows, nn = nb > 0 ? nb : 1;
+    PairArgs A;
+    memset(&A, 0, sizeof(A));
+    PairTable& T = A.T;
+    T.wide = bc.type == TQP_I64;
+    T.cap = ht_cap(nb) * ht_scale(ctx);
+    A.n = probe->num_rows;
+    A.ntiles = (A.n + kJpTile - 1) / kJpTile;
+    const size_t tab = T.wide ? static_cast<size_t>(T.cap + 1) * 16 : static_cast<size_t>(T.cap) * 8;
+    const size_t words = static_cast<size_t>(A.ntiles) + 2;  // look-back words, ticket, rows to sort
+    T.mem = arena_alloc(ctx, tab);
+    uint64_t* k0 = static_cast<uint64_t*>(arena_alloc(ctx, static_cast<size_t>(nn) * 24));
+    void* rs = arena_alloc(ctx, radix_sort_scratch(nn));
+    long long* meta = static_cast<long long*>(arena_alloc(ctx, 64));
+    unsigned long long* sc = static_cast<unsigned long long*>(arena_alloc(ctx, words * 8));
+    if (!T.mem || !k0 || !rs || !meta || !sc)
+        return arena_oom(ctx, tab + static_cast<size_t>(nn) * 24 + radix_sort_scratch(nn) + words * 8);
+    T.meta = meta;
+    TQP_CUDA(cudaMemsetAsync(T.mem, 0xFF, tab, stream));
+    TQP_CUDA(cudaMemsetAsync(sc, 0, words * 8, stream));
+    TQP_TRY(ht_key_range_launch(ctx, build, build_key, meta, stream));
+    if (nb > 0) {
+        uint64_t* k1 = k0 + nn;
+        uint32_t* v0 = reinterpret_cast<uint32_t*>(k1 + nn);
+        uint32_t* v1 = v0 + nn;
+        long long* n_sort = reinterpret_cast<long long*>(sc + 1);
+        const int threads = 256;
+        const int blocks = static_cast<int>(std::min<long long>((nb + threads - 1) / threads, ctx->num_sms * 16LL));
+        k_pair_insert<<<blocks, threads, 0, stream>>>(T, static_cast<const unsigned char*>(bc.data), bc.type, nb, k0, v0,
+                                                      n_sort);
+        int bits = 1;
+        while ((1LL << bits) <= T.cap) ++bits;
+        bool in1 = false;
+        TQP_TRY(radix_sort_pairs(k0, v0, k1, v1, n_sort, nb, 0, (bits + 7) / 8 * 8, rs, stream, &in1));
+        const uint64_t* sk = in1 ? k1 : k0;
+        uint32_t* rlen = reinterpret_cast<uint32_t*>(in1 ? k0 : k1);  // (the sort's other key buffer)
+        T.bidx = in1 ? v1 : v0;
+        T.rlen = rlen;
+        k_pair_runs<<<blocks, threads, 0, stream>>>(T, sk, n_sort);
+        k_pair_lens<<<blocks, threads, 0, stream>>>(T, sk, n_sort, rlen);
+        TQP_CUDA(cudaGetLastError());
+    }
+    A.key = static_cast<const unsigned char*>(pc.data);
+    A.key_type = pc.type;
+    A.kind = kind;
+    A.out_build = d_build_idx;
+    A.out_probe = d_probe_idx;
+    A.capacity = capacity;
+    A.d_count = d_count;
+    A.ticket = sc;
+    A.status = sc + 2;
+    A.err = ctx->d_err;
+    A.wait_cap = ctx->wait_cap;
+    k_join_pairs<<<static_cast<unsigned>(A.ntiles), kJpThreads, 0, stream>>>(A);
+    TQP_CUDA(cudaGetLastError());
+    return TQP_OK;
+}
+
 tqp_status launch_hash_join(tqp_ctx* ctx, const tqp_table* build, int32_t build_key, const tqp_table* probe,
                             int32_t probe_key, int32_t kind, int32_t* d_build_idx, int32_t* d_probe_idx,
                             int64_t capacity, int64_t* d_count, cudaStream_t stream) {
-    JoinHT H{};
     // variant 1: the sort-based join; 0: the hash table (the autotuner times both)
+    if (tuned_variant(ctx) != 1 && !user_shape(ctx) && probe->num_rows > 0)
+        return launch_join_pairs(ctx, build, build_key, probe, probe_key, kind, d_build_idx, d_probe_idx, capacity,
+                                 d_count, stream);
+    JoinHT H{};
     if (tuned_variant(ctx) == 1) TQP_TRY(ht_build_sorted(ctx, build, build_key, &H, stream));
     else TQP_TRY(ht_build(ctx, build, build_key, &H, stream));
     if (probe->num_rows == 0) {
