@@ -15,8 +15,9 @@
 //   few-group group-bys (at most 64 groups, closed-form sums): the key-range
 //             pass, then the direct kernel (vector reads one warp step ahead,
 //             lane-private tables), each job a contiguous range of blocks
-//   joined aggregations of closed-form shapes: the plain-load probe
-//             (probeagg.cuh), each job a contiguous range of blocks
+//   joined aggregations and filters of closed-form shapes: the plain-load
+//             probe (probeagg.cuh) and scan (filterdirect.cuh), each job a
+//             contiguous range of blocks
 //   scan      one persistent launch of the staged scan engine per body kind
 //             (filter, shared filter, group-by, joined aggregation): CTAs draw chunk
 //             tickets across the tables of every job of that kind (uneven
@@ -44,6 +45,7 @@
 #include "bodies.cuh"
 #include "dimgroups.cuh"
 #include "dim.cuh"
+#include "filterdirect.cuh"
 #include "probeagg.cuh"
 #include "finalize.cuh"
 #include "groupdirect.cuh"
@@ -164,6 +166,12 @@ struct DirJob {
 // first_block + nblocks) of its launch.
 struct ProbeJob {
     ProbeAggArgs A;
+    long long first_block, nblocks;
+};
+// A filter run by the plain-load scan: blocks [first_block, first_block +
+// nblocks) of its launch.
+struct FiltJob {
+    FilterDirectArgs A;
     long long first_block, nblocks;
 };
 constexpr int kDirArgsBytes = (static_cast<int>(sizeof(GroupDirectArgs)) + 127) / 128 * 128;
@@ -336,6 +344,13 @@ __global__ void __launch_bounds__(kPaThreads, kPaMinBlocks) k_b_probe_agg(const 
     probe_agg_block<kTab>(A, ptab, static_cast<long long>(blockIdx.x) - j.first_block, j.nblocks);
 }
 
+__global__ void __launch_bounds__(kFdThreads, kFdMinBlocks) k_b_filter_direct(const FiltJob* J, const int32_t* bjob) {
+    __shared__ __align__(16) unsigned char args[sizeof(FilterDirectArgs)];
+    const FiltJob& j = J[bjob[blockIdx.x]];
+    const FilterDirectArgs& A = stage_args(j.A, args);
+    filter_direct_block(A, static_cast<long long>(blockIdx.x) - j.first_block, j.nblocks);
+}
+
 __global__ void __launch_bounds__(kFinThreads) k_b_finalize(const FinJob* F) {
     extern __shared__ __align__(16) unsigned char fsm[];
     const FinJob& f = F[blockIdx.x];
@@ -394,11 +409,12 @@ struct tqp_batch {
     std::vector<DirJob> gdir;
     std::vector<FoldJob> fold;
     std::vector<ProbeJob> probe[2];  // [1]: with a table in shared memory
+    std::vector<FiltJob> filt;
     std::vector<std::vector<TopItem>> levels;
     // block -> job maps, concatenated
     std::vector<int32_t> maps;
     long long fill_blocks = 0, row_blocks = 0, num_blocks = 0, slot_blocks = 0, compact_blocks = 0, top0_blocks = 0,
-              sel_blocks = 0, grange_blocks = 0, gdirect_blocks = 0, fold_blocks = 0;
+              sel_blocks = 0, grange_blocks = 0, gdirect_blocks = 0, fold_blocks = 0, filt_blocks = 0;
     long long probe_blocks[2] = {0, 0};
     long long scan_chunks[kKinds] = {0, 0, 0, 0};
     // lookup tables and outputs of the shared scans (one blob; per job its offset)
@@ -407,7 +423,7 @@ struct tqp_batch {
     unsigned char* d_mblob = nullptr;
     std::vector<long long> level_blocks;
     size_t off_fill = 0, off_row = 0, off_num = 0, off_slot = 0, off_compact = 0, off_top0 = 0, off_sel = 0,
-           off_grange = 0, off_gdirect = 0, off_fold = 0;
+           off_grange = 0, off_gdirect = 0, off_fold = 0, off_filt = 0;
     size_t off_probe[2] = {0, 0};
     size_t off_scan[kKinds] = {0, 0, 0, 0};
     std::vector<size_t> off_level;
@@ -425,6 +441,7 @@ struct tqp_batch {
     DirJob* d_gdir = nullptr;
     FoldJob* d_fold = nullptr;
     ProbeJob* d_probe[2] = {nullptr, nullptr};
+    FiltJob* d_filt = nullptr;
     std::vector<TopItem*> d_levels;
     int32_t* d_maps = nullptr;
     unsigned long long* d_ticket[kKinds] = {nullptr, nullptr, nullptr, nullptr};
@@ -528,6 +545,19 @@ static tqp_status add_filter_job(tqp_batch* b, const tqp_plan* p, const tqp_resu
         b->zero.push_back(d_count);
         if (d_count2) b->zero.push_back(d_count2);
         if (A.d_sum) b->zero.push_back(A.d_sum);
+        return TQP_OK;
+    }
+    FiltJob D;
+    if (lower_filter_direct(p->fact, A, &D.A)) {
+        D.A.mask = A.mask;
+        D.A.block_tot = A.block_tot;
+        D.A.acc = A.acc;
+        D.A.d_count = A.d_count;
+        D.A.d_count2 = A.d_count2;
+        D.A.d_sum = A.d_sum;
+        D.A.capacity = A.capacity;
+        D.A.err = ctx->d_err;
+        b->filt.push_back(D);
         return TQP_OK;
     }
     b->scan[kJobFilter - 1].push_back(J);
@@ -1111,6 +1141,7 @@ static long long assign_blocks(const tqp_batch* b, std::vector<Job>& jobs) {
 static void build_maps(tqp_batch* b) {
     b->gdirect_blocks = assign_blocks(b, b->gdir);
     for (int k = 0; k < 2; ++k) b->probe_blocks[k] = assign_blocks(b, b->probe[k]);
+    b->filt_blocks = assign_blocks(b, b->filt);
     auto& M = b->maps;
     auto push = [&M](size_t j, long long nblocks) {
         for (long long k = 0; k < nblocks; ++k) M.push_back(static_cast<int32_t>(j));
@@ -1143,6 +1174,8 @@ static void build_maps(tqp_batch* b) {
         b->off_probe[k] = M.size();
         for (size_t j = 0; j < b->probe[k].size(); ++j) push(j, b->probe[k][j].nblocks);
     }
+    b->off_filt = M.size();
+    for (size_t j = 0; j < b->filt.size(); ++j) push(j, b->filt[j].nblocks);
     b->off_compact = M.size();
     for (size_t j = 0; j < b->compact.size(); ++j) push(j, (b->compact[j].n + kCompactRows - 1) / kCompactRows);
     b->off_sel = M.size();
@@ -1216,6 +1249,8 @@ static tqp_status batch_launch(tqp_batch* b, cudaStream_t st) {
     if (b->probe_blocks[1])
         k_b_probe_agg<true><<<static_cast<unsigned>(b->probe_blocks[1]), kPaThreads, kPaSmemBytes, st>>>(
             b->d_probe[1], M + b->off_probe[1]);
+    if (b->filt_blocks)
+        k_b_filter_direct<<<static_cast<unsigned>(b->filt_blocks), kFdThreads, 0, st>>>(b->d_filt, M + b->off_filt);
     if (b->scan_chunks[0])
         k_b_scan<FilterBody><<<b->scan_grid[0], kEngineThreads, b->scan_smem[0], st>>>(
             b->d_scan[0], M + b->off_scan[0], b->d_ticket[0], b->scan_chunks[0]);
@@ -1298,6 +1333,7 @@ static tqp_status batch_prepare(tqp_ctx* ctx, const tqp_plan* plans, const tqp_r
     TQP_TRY(upload(b, b->gdir, &b->d_gdir, st));
     TQP_TRY(upload(b, b->fold, &b->d_fold, st));
     for (int k = 0; k < 2; ++k) TQP_TRY(upload(b, b->probe[k], &b->d_probe[k], st));
+    TQP_TRY(upload(b, b->filt, &b->d_filt, st));
     b->d_levels.resize(b->levels.size());
     for (size_t L = 0; L < b->levels.size(); ++L) TQP_TRY(upload(b, b->levels[L], &b->d_levels[L], st));
     TQP_TRY(upload(b, b->maps, &b->d_maps, st));

@@ -16,6 +16,7 @@ namespace tqp {
 constexpr int kCompactRows = 65536;                  // rows per compaction block of the selection mask
 constexpr int kCompactWords = kCompactRows / kWarp;  // 2048 mask words
 constexpr int kCompactThreads = 1024;
+constexpr uint32_t kCompactDense = 8 * kWarp;          // set bits of a warp's 2048 rows from which its lanes share each word
 
 // Count one (chunk, warp) completion; true for the very last one of the scan.
 __device__ __forceinline__ bool last_completion(unsigned long long* done, long long nchunks) {
@@ -992,8 +993,10 @@ __device__ __forceinline__ void keyfirst_fold_block(const JoinHT& H, const unsig
 // Expand the selection mask of rows [b * kCompactRows, ...) into row ids.
 // Called by a whole block of kCompactThreads threads for mask block b: each
 // thread takes two consecutive mask words (64 rows), one block-wide exclusive
-// scan of their bit counts gives every thread its output offset, and each
-// thread writes the ids of its own set bits (ascending, so the output is).
+// scan of their bit counts gives every thread its output offset. Few set bits:
+// each thread writes the ids of its own (ascending, so the output is); where a
+// warp's words hold many, its lanes take the bits of one word at a time, so that
+// the stores are contiguous (20M rows, 96% set: 155 us without that).
 __device__ __forceinline__ void compact_block(const uint32_t* __restrict__ mask, const uint32_t* __restrict__ block_tot,
                                               long long n, int32_t* __restrict__ row_ids, long long capacity,
                                               long long b) {
@@ -1031,6 +1034,23 @@ __device__ __forceinline__ void compact_block(const uint32_t* __restrict__ mask,
     }
     unsigned long long pos = base + before_warps + (incl - c);
     const long long row0 = wi * kWarp;
+    if (__shfl_sync(0xffffffffu, incl, kWarp - 1) >= kCompactDense) {  // (warp-uniform)
+        const uint32_t lt = lanemask_lt();
+        const unsigned long long p0 = __shfl_sync(0xffffffffu, pos, 0);  // of the warp's first word
+        const uint32_t off = incl - c;
+        const long long first = __shfl_sync(0xffffffffu, row0, 0) + lane;
+#pragma unroll 4
+        for (int k = 0; k < kWarp; ++k) {
+            const uint32_t x = __shfl_sync(0xffffffffu, m0, k), y = __shfl_sync(0xffffffffu, m1, k);
+            const unsigned long long px = p0 + __shfl_sync(0xffffffffu, off, k) + __popc(x & lt);
+            const unsigned long long py = p0 + __shfl_sync(0xffffffffu, off, k) + __popc(x) + __popc(y & lt);
+            const long long r = first + 2 * kWarp * k;
+            if (((x >> lane) & 1u) && px < static_cast<unsigned long long>(capacity)) __stcs(row_ids + px, static_cast<int32_t>(r));
+            if (((y >> lane) & 1u) && py < static_cast<unsigned long long>(capacity))
+                __stcs(row_ids + py, static_cast<int32_t>(r + kWarp));
+        }
+        return;
+    }
     uint32_t m = m0;
     while (m) {
         const int bit = __ffs(m) - 1;
