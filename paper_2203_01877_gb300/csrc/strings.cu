@@ -207,6 +207,313 @@ __global__ void __launch_bounds__(kStrThreads) k_str_prepass(const __grid_consta
     }
 }
 
+// ---- strings of at most 32 bytes: the words in registers ---------------------------
+// The general form above walks a string byte by byte through shared memory and
+// is bound by integer issue. Here a lane holds its string's 32-bit words; a
+// segment of a LIKE pattern is a list of 4-byte (value, mask) chunks (`_`: mask
+// 0), its match positions are one 32-bit mask -- the chunk compared with the
+// four-byte window at every position, later chunks ANDed in at their offset --
+// and the segments are placed leftmost-first with bit operations. IN compares
+// whole words against each of a short list. Still bound by issue (63% of the
+// slots, 333 warp instructions per 32 strings of 24 bytes before the length was
+// found with one bit scan). 20M rows, `%xy%` and a price bound: 476 -> 297 us;
+// a prefix 209, eight IN values 274. Longer lists are searched by the general
+// form, and patterns of more segments or wider strings matched by it.
+constexpr int kSfThreads = 256;
+constexpr int kSfMinBlocks = 4;
+constexpr int kSfMaxWords = 8;
+constexpr int kSfSegs = 8;           // LIKE segments
+constexpr int kSfValues = 32;        // IN values
+constexpr int kSfWords = 1024;       // program words of a launch
+
+struct StrFastPred {
+    const unsigned char* col;
+    int32_t type;
+    int32_t width;
+    int32_t op;
+    int32_t flags;             // kLike*
+    int32_t count;             // LIKE: segments; IN: values
+    int32_t off;               // first program word. LIKE: {length, chunks (value, mask)} per segment; IN: the values
+                               // (strings padded with zero to whole words; numbers as two words)
+};
+
+struct StrFast {
+    int64_t n;
+    unsigned char* out;
+    int32_t npred;
+    int32_t nwords;
+    int32_t stage_bytes;       // per warp, for widths that are not whole words
+    int32_t pad;
+    StrFastPred p[TQP_MAX_PREDS];
+    uint32_t words[kSfWords];
+};
+
+// Match positions of a segment of `len` bytes (len >= 1): bit p set when it matches at byte p.
+template <int NW>
+__device__ __forceinline__ uint32_t sf_find(const uint32_t (&w)[NW], const uint32_t* chunk, int len) {
+    uint32_t M = ~0u;
+    for (int c = 0; 4 * c < len && M; ++c) {
+        const uint32_t v = chunk[2 * c], m = chunk[2 * c + 1];
+        uint32_t hit = 0;
+#pragma unroll
+        for (int i = 0; i < NW; ++i) {
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const uint32_t x = __funnelshift_r(w[i], i + 1 < NW ? w[i + 1] : 0u, 8 * b);
+                if (((x ^ v) & m) == 0) hit |= 1u << (4 * i + b);
+            }
+        }
+        M &= hit >> (4 * c);
+    }
+    return M;
+}
+
+template <int NW>
+__device__ __forceinline__ bool sf_like(const uint32_t (&w)[NW], const StrFastPred& q, const uint32_t* prog) {
+    // the string's length: its first zero byte (the lowest set bit of the first word with one)
+    uint32_t z0 = 0x80u;
+    int n = 4 * NW;
+#pragma unroll
+    for (int i = NW - 1; i >= 0; --i) {
+        const uint32_t z = (w[i] - 0x01010101u) & ~w[i] & 0x80808080u;
+        if (z) {
+            z0 = z;
+            n = 4 * i;
+        }
+    }
+    n += (__ffs(z0) - 1) / 8;
+    n = n < q.width ? n : q.width;
+    int pos = 0;
+    for (int k = 0; k < q.count; ++k) {
+        const int len = static_cast<int>(*prog);
+        const uint32_t* chunk = prog + 1;
+        prog += 1 + 2 * ((len + 3) / 4);
+        if (len > n - pos) return false;
+        if (len == 0) return n == 0;  // (only the empty pattern has an empty segment)
+        if ((q.flags & kLikeExact) || (k == 0 && (q.flags & kLikeStart))) {
+            if ((q.flags & kLikeExact) && n != len) return false;
+            uint32_t d = 0;
+#pragma unroll
+            for (int i = 0; i < NW; ++i)
+                if (4 * i < len) d |= (w[i] ^ chunk[2 * i]) & chunk[2 * i + 1];
+            if (d) return false;
+            pos = len;
+            continue;
+        }
+        // starts from which the segment ends within the string
+        uint32_t M = sf_find<NW>(w, chunk, len) & (n - len >= 31 ? ~0u : (2u << (n - len)) - 1u);
+        if (k == q.count - 1 && (q.flags & kLikeEnd)) {
+            return (M >> (n - len)) & 1u;  // (n - len >= pos)
+        } else {
+            M &= ~0u << pos;
+            if (!M) return false;
+            pos = __ffs(M) - 1 + len;
+            if (pos >= 32 && k + 1 < q.count) return false;  // nothing is left for the next segment
+        }
+    }
+    return true;
+}
+
+// Two groups of 32 rows per warp step, their strings' loads in flight together.
+constexpr int kSfUnroll = 2;
+
+// The words of the lane's string in group g (zero past the width and where `pass` is false).
+template <int NW>
+__device__ __forceinline__ void sf_load(const StrFast& L, const StrFastPred& q, long long g, int lane, bool pass,
+                                        unsigned char* my, uint32_t (&w)[NW]) {
+    const int m = q.width;
+#pragma unroll
+    for (int i = 0; i < NW; ++i) w[i] = 0;
+    if ((m & 3) == 0) {
+        if (!pass) return;
+        const unsigned char* s = q.col + (g * kWarp + lane) * m;
+        if (m == 4 * NW) {
+#pragma unroll
+            for (int i = 0; i + 1 < NW; i += 2) {
+                const uint2 x = __ldcs(reinterpret_cast<const uint2*>(s) + i / 2);
+                w[i] = x.x;
+                w[i + 1] = x.y;
+            }
+        } else if ((m & 7) == 0) {
+#pragma unroll
+            for (int i = 0; i + 1 < NW; i += 2)
+                if (4 * i < m) {
+                    const uint2 x = __ldcs(reinterpret_cast<const uint2*>(s) + i / 2);
+                    w[i] = x.x;
+                    w[i + 1] = x.y;
+                }
+        } else {
+#pragma unroll
+            for (int i = 0; i < NW; ++i)
+                if (4 * i < m) w[i] = __ldcs(reinterpret_cast<const uint32_t*>(s) + i);
+        }
+        return;
+    }
+    // through shared memory: the group's strings from a 16-byte boundary, each cut out of whole words
+    const long long r0 = g * kWarp;
+    const int bytes = static_cast<int>(L.n - r0 < kWarp ? L.n - r0 : kWarp) * m;
+    const unsigned char* src = q.col + r0 * m;
+    __syncwarp();
+    for (int i = lane; i < bytes / 16; i += kWarp)
+        reinterpret_cast<uint4*>(my)[i] = __ldcs(reinterpret_cast<const uint4*>(src) + i);
+    for (int i = (bytes / 16) * 16 + lane; i < bytes; i += kWarp) my[i] = __ldg(src + i);
+    __syncwarp();
+    const int at = lane * m;
+    const uint32_t* sw = reinterpret_cast<const uint32_t*>(my) + at / 4;
+    uint32_t x = sw[0];
+#pragma unroll
+    for (int i = 0; i < NW; ++i) {
+        if (4 * i >= m) break;
+        const uint32_t y = sw[i + 1];
+        w[i] = __funnelshift_r(x, y, 8 * (at & 3));
+        x = y;
+        const int left = m - 4 * i;
+        if (left < 4) w[i] &= (1u << (8 * left)) - 1u;
+    }
+}
+
+template <int NW>
+__device__ __forceinline__ bool sf_test(const uint32_t (&w)[NW], const StrFastPred& q, const uint32_t* prog) {
+    if (q.op != TQP_IN) return sf_like<NW>(w, q, prog) == (q.op == TQP_LIKE);
+    const int nw = (q.width + 3) / 4;
+    for (int v = 0; v < q.count; ++v) {
+        uint32_t d = 0;
+#pragma unroll
+        for (int i = 0; i < NW; ++i)
+            if (i < nw) d |= w[i] ^ prog[v * nw + i];
+        if (d == 0) return true;
+    }
+    return false;
+}
+
+template <int NW>
+__global__ void __launch_bounds__(kSfThreads, kSfMinBlocks) k_str_fast(const __grid_constant__ StrFast L) {
+    extern __shared__ __align__(16) unsigned char ssm[];
+    uint32_t* words = reinterpret_cast<uint32_t*>(ssm);
+    for (int i = threadIdx.x; i < L.nwords; i += kSfThreads) words[i] = L.words[i];
+    __syncthreads();
+    const int lane = threadIdx.x % kWarp, warp = threadIdx.x / kWarp;
+    unsigned char* my = ssm + (L.nwords * 4 + 15) / 16 * 16 + warp * L.stage_bytes;
+    const long long groups = (L.n + kWarp - 1) / kWarp;
+    const long long step = static_cast<long long>(gridDim.x) * (kSfThreads / kWarp);
+    for (long long g = static_cast<long long>(blockIdx.x) * (kSfThreads / kWarp) + warp; g < groups; g += kSfUnroll * step) {
+        uint32_t pass = 0;
+#pragma unroll
+        for (int u = 0; u < kSfUnroll; ++u) pass |= static_cast<uint32_t>((g + u * step) * kWarp + lane < L.n) << u;
+        for (int k = 0; k < L.npred; ++k) {
+            if (!__any_sync(0xffffffffu, pass != 0)) break;
+            const StrFastPred& q = L.p[k];
+            const uint32_t* prog = words + q.off;
+            if (q.type != TQP_CHAR) {  // IN on a numeric column
+#pragma unroll
+                for (int u = 0; u < kSfUnroll; ++u) {
+                    if (!((pass >> u) & 1u)) continue;
+                    const uint64_t x = static_cast<uint64_t>(ldg_typed(q.col, q.type, (g + u * step) * kWarp + lane));
+                    bool hit = false;
+                    for (int v = 0; v < q.count; ++v)
+                        hit |= prog[2 * v] == static_cast<uint32_t>(x) && prog[2 * v + 1] == static_cast<uint32_t>(x >> 32);
+                    if (!hit) pass &= ~(1u << u);
+                }
+                continue;
+            }
+            uint32_t w[kSfUnroll][NW];
+#pragma unroll
+            for (int u = 0; u < kSfUnroll; ++u)
+                if (g + u * step < groups) sf_load<NW>(L, q, g + u * step, lane, (pass >> u) & 1u, my, w[u]);
+#pragma unroll
+            for (int u = 0; u < kSfUnroll; ++u)
+                if (((pass >> u) & 1u) && !sf_test<NW>(w[u], q, prog)) pass &= ~(1u << u);
+        }
+#pragma unroll
+        for (int u = 0; u < kSfUnroll; ++u) {
+            const long long row = (g + u * step) * kWarp + lane;
+            if (row < L.n) L.out[row] = (pass >> u) & 1u;
+        }
+    }
+}
+
+// The launch above from the general one; false outside its shapes.
+static bool lower_str_fast(const StrLaunch& L, StrFast* F, int* words_per_string) {
+    F->n = L.n;
+    F->out = L.out;
+    F->npred = L.npred;
+    int used = 0, maxw = 4;
+    bool stage = false;
+    auto push = [&](uint32_t x) {
+        if (used < kSfWords) F->words[used] = x;
+        ++used;
+    };
+    for (int k = 0; k < L.npred; ++k) {
+        const StrPred& q = L.p[k];
+        StrFastPred& f = F->p[k];
+        f = StrFastPred{q.col, q.type, q.width, q.op, q.flags, q.count, used};
+        const unsigned char* data = L.blob + q.off;
+        if (q.type == TQP_CHAR) {
+            if (q.width > 4 * kSfMaxWords) return false;
+            maxw = std::max(maxw, q.width);
+            stage = stage || q.width % 4 != 0;
+        }
+        if (q.op == TQP_IN) {
+            if (q.count > kSfValues) return false;
+            const int bytes = q.type == TQP_CHAR ? q.width : 8;
+            for (int v = 0; v < q.count; ++v)
+                for (int b = 0; b < bytes; b += 4) {
+                    uint32_t x = 0;
+                    for (int i = 0; i < 4 && b + i < bytes; ++i) x |= static_cast<uint32_t>(data[v * bytes + b + i]) << (8 * i);
+                    push(x);
+                }
+            continue;
+        }
+        if ((q.flags & kLikeGreedy) || q.nseg > kSfSegs) return false;
+        f.count = q.nseg;
+        // the segments again, from the pattern (split at `%`; without one, the whole pattern)
+        std::vector<std::string> segs;
+        if (q.flags & kLikeExact) {
+            segs.emplace_back(reinterpret_cast<const char*>(data), q.count);
+        } else {
+            std::string cur;
+            for (int i = 0; i <= q.count; ++i) {
+                if (i < q.count && data[i] != '%') {
+                    cur.push_back(static_cast<char>(data[i]));
+                } else {
+                    if (!cur.empty()) segs.push_back(cur);
+                    cur.clear();
+                }
+            }
+        }
+        for (const std::string& g : segs) {
+            push(static_cast<uint32_t>(g.size()));
+            for (size_t b = 0; b < g.size(); b += 4) {
+                uint32_t x = 0, m = 0;
+                for (size_t i = 0; i < 4 && b + i < g.size(); ++i) {
+                    if (g[b + i] == '_') continue;
+                    x |= static_cast<uint32_t>(static_cast<unsigned char>(g[b + i])) << (8 * i);
+                    m |= 0xFFu << (8 * i);
+                }
+                push(x);
+                push(m);
+            }
+        }
+    }
+    if (used > kSfWords) return false;
+    F->nwords = used;
+    F->stage_bytes = stage ? (kWarp * maxw + 4 + 15) / 16 * 16 : 0;
+    *words_per_string = maxw <= 8 ? 2 : (maxw <= 16 ? 4 : (maxw <= 24 ? 6 : 8));
+    return true;
+}
+
+template <int NW>
+static tqp_status launch_str_fast(const tqp_ctx* ctx, const StrFast& F, cudaStream_t st) {
+    const size_t smem = (static_cast<size_t>(F.nwords) * 4 + 15) / 16 * 16 +
+                        static_cast<size_t>(kSfThreads / kWarp) * F.stage_bytes;  // (below 16 KB)
+    const long long groups = (F.n + kWarp - 1) / kWarp;
+    const long long want = (groups + kSfThreads / kWarp - 1) / (kSfThreads / kWarp);
+    const long long grid = std::min<long long>(want, 1LL * kSfMinBlocks * ctx->num_sms);
+    k_str_fast<NW><<<static_cast<unsigned>(grid), kSfThreads, smem, st>>>(F);
+    TQP_CUDA(cudaGetLastError());
+    return TQP_OK;
+}
+
 static bool is_set_op(int op) { return op == TQP_IN || op == TQP_LIKE || op == TQP_NOT_LIKE; }
 
 bool has_set_preds(const tqp_table* t, const tqp_pred* preds, int32_t npreds) {
@@ -343,19 +650,27 @@ tqp_status str_prepass(tqp_ctx* ctx, const tqp_table* t, const tqp_pred* preds, 
         L->n = n;
         L->out = pass;
         L->blob_bytes = static_cast<int32_t>(used);
-        L->stage_bytes = (kWarp * maxw + 15) / 16 * 16;
-        static SmemFlags attr;
-        TQP_TRY(allow_smem(ctx, reinterpret_cast<const void*>(k_str_prepass), attr));
-        const size_t smem = (used + 15) / 16 * 16 + static_cast<size_t>(kStrWarps) * L->stage_bytes;
-        int occ = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_str_prepass, kStrThreads, smem) != cudaSuccess ||
-            occ < 1)
-            occ = 1;
-        const long long groups = (n + kWarp - 1) / kWarp;
-        const long long want = (groups + kStrWarps - 1) / kStrWarps;
-        const int grid = static_cast<int>(std::min<long long>(want, static_cast<long long>(ctx->num_sms) * occ));
-        k_str_prepass<<<grid, kStrThreads, smem, st>>>(*L);
-        TQP_CUDA(cudaGetLastError());
+        StrFast F;
+        int nw = 0;
+        if (lower_str_fast(*L, &F, &nw)) {
+            TQP_TRY(nw == 2 ? launch_str_fast<2>(ctx, F, st)
+                            : (nw == 4 ? launch_str_fast<4>(ctx, F, st)
+                                       : (nw == 6 ? launch_str_fast<6>(ctx, F, st) : launch_str_fast<8>(ctx, F, st))));
+        } else {
+            L->stage_bytes = (kWarp * maxw + 15) / 16 * 16;
+            static SmemFlags attr;
+            TQP_TRY(allow_smem(ctx, reinterpret_cast<const void*>(k_str_prepass), attr));
+            const size_t smem = (used + 15) / 16 * 16 + static_cast<size_t>(kStrWarps) * L->stage_bytes;
+            int occ = 0;
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_str_prepass, kStrThreads, smem) != cudaSuccess ||
+                occ < 1)
+                occ = 1;
+            const long long groups = (n + kWarp - 1) / kWarp;
+            const long long want = (groups + kStrWarps - 1) / kStrWarps;
+            const int grid = static_cast<int>(std::min<long long>(want, static_cast<long long>(ctx->num_sms) * occ));
+            k_str_prepass<<<grid, kStrThreads, smem, st>>>(*L);
+            TQP_CUDA(cudaGetLastError());
+        }
     }
     out->cols.assign(t->cols, t->cols + t->num_cols);
     tqp_column pc;
