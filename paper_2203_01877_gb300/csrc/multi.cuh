@@ -16,12 +16,14 @@
 //     breakpoints span at most kMqDirectMax values, else a branch-free binary
 //     search over the sorted breakpoints.  The cost per row grows with the
 //     number of condition columns, not with the number of queries;
-//   * accumulation: every consumer warp keeps a count and a sum per query in
-//     shared memory; each lane walks the set bits of its rows' pass masks and
-//     adds to those queries with shared-memory atomics (the work is the
-//     number of (row, passing query) pairs, spread over the lanes; rows that
-//     pass no query cost nothing).  At the end of a chunk lane q moves query
-//     q's totals of its warp to global memory;
+//   * accumulation: lane q keeps query q's count and sum in registers. Rows that
+//     pass some query join a queue of their warp (pass mask and values, in shared
+//     memory); for every 32 of them the masks are transposed (five exchange
+//     steps), so that lane q holds the rows that pass query q: its count is a bit
+//     count, and it adds their values. 60M rows and 32 queries of 2% each took 654
+//     us with a shared-memory atomic per (row, passing query) pair instead: the
+//     lanes wait for the one with most pairs, 244 warp instructions per 32 rows.
+//     At the end of a chunk lane q moves query q's totals to global memory;
 //   * per-query row ranges: a query may cover only rows [rlo, rhi) of the
 //     scan (queries over slices of one table).  Per tile a ballot splits the
 //     queries into those covering the whole tile and those touching part of
@@ -43,10 +45,12 @@ constexpr int kMqMinPack = 3;       // smaller packs run through the single-quer
 constexpr int kMqWords = 5120;      // mask words of all lookup tables (shared memory)
 constexpr int kMqBreaks = 512;      // breakpoints of the searched tables (shared memory)
 constexpr int kMqDirectMax = 4096;  // direct tables: at most this many entries per column
-// per-warp accumulators: 32 sums (8 bytes) and 32 counts (4 bytes) per consumer warp
-constexpr int kMqAccBytes = kConsumerWarps * kMqMax * 12;
+constexpr int kMqRows = 4;          // rows per lane of a step
+constexpr int kMqQueue = (kMqRows + 1) * kWarp;  // queued rows of a warp: a step's and fewer than kWarp before it
+// the queue of each consumer warp: per row a value for each sum expression, and its pass mask
+constexpr int kMqAccBytes = kConsumerWarps * kMqQueue * (kMqExprs * 8 + 4);
 
-// Shared memory of one launch's body: accumulators | mask words | breakpoints.
+// Shared memory of one launch's body: row queues | mask words | breakpoints.
 __host__ __device__ constexpr int mq_words_bytes(int nwords) { return (nwords * 4 + 15) / 16 * 16; }
 __host__ __device__ constexpr int mq_body_bytes(int nwords, int nbreaks) {
     return (kMqAccBytes + mq_words_bytes(nwords) + nbreaks * 8 + 127) / 128 * 128;
@@ -128,15 +132,19 @@ __device__ __forceinline__ int64_t mq_factor_row(const ScanGeom& G, const TileVi
     return static_cast<int64_t>(x * a + b);
 }
 
-// 64-bit add to shared memory as two 32-bit atomic adds (low word, then the
-// high word with the carry): measured faster than a 64-bit atomic add on
-// shared memory.  Readers see the sum only after the warp's adds are done.
-__device__ __forceinline__ void add_shared_u64(unsigned long long* p, unsigned long long x) {
-    unsigned int* w = reinterpret_cast<unsigned int*>(p);
-    const unsigned int lo = static_cast<unsigned int>(x);
-    const unsigned int old = atomicAdd(w, lo);
-    const unsigned int hi = static_cast<unsigned int>(x >> 32) + (old + lo < old ? 1u : 0u);
-    if (hi) atomicAdd(w + 1, hi);
+// The transpose of the 32 x 32 bit matrix whose row l is lane l's x (all lanes
+// call it): bit r of lane q's result is bit q of lane r's x.
+__device__ __forceinline__ uint32_t warp_transpose(uint32_t x, int lane) {
+    uint32_t m = 0x0000FFFFu;  // columns whose index has bit j clear
+#pragma unroll
+    for (int j = 16; j > 0; j >>= 1) {
+        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, j);
+        const bool up = lane & j;
+        const uint32_t keep = up ? ~m : m;
+        x = (x & keep) | (__funnelshift_l(y, y, up ? 32 - j : j) & ~keep);
+        m ^= m << (j >> 1);
+    }
+    return x;
 }
 
 // A direct-table condition column held in registers by the fast path: the
@@ -152,29 +160,29 @@ constexpr int kMqFastCols = 4;  // condition columns of the fast path
 struct MultiBody {
     static constexpr int kMinBlocks = 2;
     static constexpr int kSmemBytes = mq_body_bytes(kMqWords, kMqBreaks);  // the largest launch
-    static constexpr int kU = 4;  // rows per lane per step
+    static constexpr int kU = kMqRows;  // rows per lane per step
 
     const MultiArgs& A;
     const uint32_t* w;         // shared-memory copy of the masks
     const int64_t* bk;         // shared-memory copy of the breakpoints
-    unsigned long long* wsum;  // this warp's 32 sums
-    unsigned int* wcnt;        // this warp's 32 counts
+    unsigned long long* qval;  // this warp's queue: values [expression][row], and masks
+    uint32_t* qmask;
+    int qn = 0;                // queued rows (warp-uniform)
+    unsigned long long qsum = 0;  // lane q: query q's sum and count since the last chunk
+    unsigned int qcnt = 0;
     int64_t rlo = 0, rhi = 0;  // lane q: query q's row range
     MqHot hot[kMqFastCols];    // fast path: the condition columns
     bool fast = false;         // every condition column has a direct table (at most kMqFastCols)
 
     const MqOut* outp;         // the queries' outputs and row ranges
 
-    // Every thread of the CTA copies its share of the tables and each
-    // consumer warp clears its accumulators; the caller synchronises the CTA
-    // before the first tile.  The tables and outputs come from the argument
+    // Every thread of the CTA copies its share of the tables; the caller
+    // synchronises the CTA before the first tile.  The tables and outputs come from the argument
     // block's pointers, or from the explicit ones (kernel parameters).
     __device__ MultiBody(const MultiArgs& a, unsigned char* sm) : MultiBody(a, sm, a.words, a.breaks, a.out) {}
     __device__ MultiBody(const MultiArgs& a, unsigned char* sm, const uint32_t* words, const int64_t* breaks,
                          const MqOut* out)
         : A(a), outp(out) {
-        unsigned long long* acc = reinterpret_cast<unsigned long long*>(sm);
-        unsigned int* cnt = reinterpret_cast<unsigned int*>(sm + kConsumerWarps * kMqMax * 8);
         uint32_t* ws = reinterpret_cast<uint32_t*>(sm + kMqAccBytes);
         int64_t* bs = reinterpret_cast<int64_t*>(sm + kMqAccBytes + mq_words_bytes(a.nwords));
         for (int i = threadIdx.x; i < a.nwords; i += blockDim.x) ws[i] = words[i];
@@ -184,12 +192,8 @@ struct MultiBody {
         const int warp = threadIdx.x / kWarp;
         const int lane = threadIdx.x % kWarp;
         const int cw = warp < kConsumerWarps ? warp : 0;
-        wsum = acc + cw * kMqMax;
-        wcnt = cnt + cw * kMqMax;
-        if (warp < kConsumerWarps) {
-            wsum[lane] = 0;
-            wcnt[lane] = 0;
-        }
+        qval = reinterpret_cast<unsigned long long*>(sm) + cw * kMqExprs * kMqQueue;
+        qmask = reinterpret_cast<uint32_t*>(sm + kConsumerWarps * kMqExprs * kMqQueue * 8) + cw * kMqQueue;
         if (lane < a.nq) {
             rlo = out[lane].rlo;
             rhi = out[lane].rhi;
@@ -282,35 +286,36 @@ struct MultiBody {
         add_pairs<U>(m, v0, v1);
     }
 
-    // One work list per lane over its U rows: the warp iterates as often as
-    // its busiest lane has (row, passing query) pairs.
+    // The last up to kWarp queued rows (from `first` on) into the queries they pass.
+    __device__ __forceinline__ void flush(int first, int lane) {
+        __syncwarp();
+        uint32_t x = warp_transpose(first + lane < qn ? qmask[first + lane] : 0u, lane);  // the rows of this lane's query
+        qcnt += __popc(x);
+        if (A.nexpr > 0) {
+            const unsigned long long* v = qval + ((A.esel >> lane) & 1u) * kMqQueue + first;
+            for (; x; x &= x - 1) qsum += v[__ffs(x) - 1];
+        }
+        qn = first;
+        __syncwarp();  // (read before the next rows take their place)
+    }
+
+    // The step's rows that pass some query into the queue (every lane calls it).
     template <int U>
     __device__ __forceinline__ void add_pairs(const uint32_t (&m)[U], const int64_t (&v0)[U], const int64_t (&v1)[U]) {
-        const uint32_t esel = A.esel;
-        uint32_t mm[U];
+        static_assert(U == kMqRows, "the queue holds a step's rows");
+        const uint32_t lt = lanemask_lt();
 #pragma unroll
-        for (int j = 0; j < U; ++j) mm[j] = m[j];
-        while (true) {
-            int64_t a0 = v0[U - 1], a1 = v1[U - 1];
-            uint32_t cur = mm[U - 1];
-            int jj = U - 1;
-#pragma unroll
-            for (int j = U - 2; j >= 0; --j) {
-                if (mm[j]) {
-                    a0 = v0[j];
-                    a1 = v1[j];
-                    cur = mm[j];
-                    jj = j;
-                }
+        for (int j = 0; j < U; ++j) {
+            const uint32_t b = __ballot_sync(0xffffffffu, m[j] != 0);
+            if (m[j]) {
+                const int at = qn + __popc(b & lt);
+                qmask[at] = m[j];
+                if (A.nexpr > 0) qval[at] = static_cast<unsigned long long>(v0[j]);
+                if (A.nexpr > 1) qval[kMqQueue + at] = static_cast<unsigned long long>(v1[j]);
             }
-            if (!cur) break;
-            const int q = __ffs(cur) - 1;
-#pragma unroll
-            for (int j = 0; j < U; ++j)
-                if (j == jj) mm[j] = cur & (cur - 1);
-            add_shared_u64(&wsum[q], static_cast<unsigned long long>(((esel >> q) & 1u) ? a1 : a0));
-            atomicAdd(&wcnt[q], 1u);
+            qn += __popc(b);
         }
+        while (qn >= kWarp) flush(qn - kWarp, static_cast<int>(threadIdx.x % kWarp));
     }
 
     // General path (a ragged last tile, searched tables, more than
@@ -381,11 +386,11 @@ struct MultiBody {
     }
 
     __device__ void chunk_end(const ScanGeom&, long long, long long, long long, int, int lane) {
-        __syncwarp();
-        const unsigned long long ls = wsum[lane];
-        const unsigned long long lc = wcnt[lane];
-        wsum[lane] = 0;
-        wcnt[lane] = 0;
+        if (qn > 0) flush(0, lane);
+        const unsigned long long ls = qsum;
+        const unsigned long long lc = qcnt;
+        qsum = 0;
+        qcnt = 0;
         if (lane < A.nq) {
             if (ls) atomicAdd(&A.acc[2 * lane], ls);
             if (lc) atomicAdd(&A.acc[2 * lane + 1], lc);
