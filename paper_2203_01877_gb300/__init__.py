@@ -18,6 +18,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 import threading
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
@@ -159,12 +160,14 @@ def _check(status: int):
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
     if stream is None:
         import torch
+        if torch.cuda.is_initialized():  # (the raw handle: building a Stream object costs more than a launch)
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
         return C.c_void_p(torch.cuda.current_stream().cuda_stream)
     if isinstance(stream, int):
         return C.c_void_p(stream)
@@ -220,11 +223,40 @@ class TableRef:
         return C.byref(self.t)
 
 
-def make_expr(tokens) -> Expr:
-    e = Expr()
+# Structs are packed in one call: a ctypes field store costs about half a
+# microsecond, and a call on a small table takes twenty in all. Values that do
+# not fit their field go through the stores, which wrap them.
+_PRED = "iiqq"
+_EXPR = "i8i4x8q"
+assert struct.calcsize("=" + _PRED) == C.sizeof(Pred) and struct.calcsize("=" + _EXPR) == C.sizeof(Expr)
+
+
+def _expr_values(tokens):
     toks = list(tokens)
     if len(toks) > MAX_EXPR:
         raise ValueError("expression longer than 8 tokens")
+    op, v = [0] * MAX_EXPR, [0] * MAX_EXPR
+    for i, tk in enumerate(toks):
+        if isinstance(tk, str):
+            op[i] = _XOPS[tk]
+        else:
+            op[i], v[i] = _XOPS[tk[0]], int(tk[1])
+    return [len(toks), *op, *v]
+
+
+_NO_EXPR = [0] * (1 + 2 * MAX_EXPR)
+
+
+def make_expr(tokens) -> Expr:
+    try:
+        return Expr.from_buffer_copy(struct.pack("=" + _EXPR, *_expr_values(tokens)))
+    except struct.error:
+        return _store_expr(tokens)
+
+
+def _store_expr(tokens) -> Expr:
+    e = Expr()
+    toks = list(tokens)
     e.n = len(toks)
     for i, tk in enumerate(toks):
         if isinstance(tk, str):
@@ -278,6 +310,21 @@ def _fill_pred(dst, table, pred, keep):
 def make_preds(preds, table=None):
     """Predicates (col, op, lo[, hi]); op "in" takes a list of values, "like" / "not_like" a pattern (str or
     bytes).  The array keeps the value buffers alive (``_keep``)."""
+    flat, n = [], 0
+    for c, op, lo, *hi in preds:
+        code = _OPS[op]
+        if code >= _OPS["in"]:  # its values need a buffer
+            n = -1
+            break
+        flat += (int(c), code, int(lo), int(hi[0]) if hi else 0)
+        n += 1
+    if n > 0:
+        try:
+            arr = (Pred * n).from_buffer_copy(struct.pack("=" + _PRED * n, *flat))
+            arr._keep = []
+            return arr
+        except struct.error:
+            pass
     arr = (Pred * max(1, len(preds)))()
     keep = []
     for i, pr in enumerate(preds):
@@ -287,7 +334,16 @@ def make_preds(preds, table=None):
 
 
 def make_aggs(aggs):
-    arr = (Agg * max(1, len(aggs)))()
+    n, flat = len(aggs), []
+    for fn, ex in aggs:
+        flat += (_FNS[fn], 0)
+        flat += _NO_EXPR if ex is None else _expr_values(ex)
+    if n:
+        try:
+            return (Agg * n).from_buffer_copy(struct.pack("=" + ("ii" + _EXPR) * n, *flat))
+        except struct.error:
+            pass
+    arr = (Agg * max(1, n))()
     for i, (fn, ex) in enumerate(aggs):
         arr[i].fn = _FNS[fn]
         if ex is not None:

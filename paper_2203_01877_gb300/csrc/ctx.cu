@@ -436,10 +436,26 @@ tqp_status make_geom(const tqp_ctx* ctx, const tqp_table* t, std::vector<int> st
     return TQP_OK;
 }
 
-int engine_grid(const tqp_ctx* ctx, const void* kernel, size_t smem, int64_t ntiles, int ctas_per_sm) {
+// (The answer depends on the program alone, so it is asked for once: the query
+// costs about as much as a launch.)
+int resident_blocks(int device, const void* kernel, int threads, size_t smem) {
+    static std::mutex mu;
+    static std::map<std::tuple<int, const void*, int, size_t>, int> known;
+    const auto key = std::make_tuple(device, kernel, threads, smem);
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        const auto it = known.find(key);
+        if (it != known.end()) return it->second;
+    }
     int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, kEngineThreads, smem) != cudaSuccess || occ < 1)
-        occ = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, smem) != cudaSuccess || occ < 1) return 1;
+    std::lock_guard<std::mutex> lk(mu);
+    if (known.size() < 4096) known[key] = occ;
+    return occ;
+}
+
+int engine_grid(const tqp_ctx* ctx, const void* kernel, size_t smem, int64_t ntiles, int ctas_per_sm) {
+    int occ = resident_blocks(ctx->device, kernel, kEngineThreads, smem);
     if (ctas_per_sm > 0) occ = std::min(occ, ctas_per_sm);
     const int64_t g = std::min<int64_t>(static_cast<int64_t>(ctx->num_sms) * occ, ntiles);
     return static_cast<int>(std::max<int64_t>(g, 1));

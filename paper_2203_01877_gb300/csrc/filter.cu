@@ -41,12 +41,12 @@ struct FilterScratch {
     long long nblocks;
 };
 
-static FilterScratch filter_scratch_layout(const ScanGeom& G, bool ids) {
+static FilterScratch filter_scratch_layout(long long n, long long mask_rows, bool ids) {
     FilterScratch s;
-    s.nblocks = ids ? (G.n + kCompactRows - 1) / kCompactRows : 0;
+    s.nblocks = ids ? (n + kCompactRows - 1) / kCompactRows : 0;
     s.tot_off = 4 * sizeof(unsigned long long);
     s.mask_off = (s.tot_off + s.nblocks * sizeof(uint32_t) + 255) / 256 * 256;
-    s.bytes = s.mask_off + (ids ? static_cast<size_t>(G.ntiles) * (G.T / kWarp) * sizeof(uint32_t) : 0);
+    s.bytes = s.mask_off + (ids ? static_cast<size_t>(mask_rows / kWarp) * sizeof(uint32_t) : 0);
     return s;
 }
 
@@ -128,15 +128,15 @@ bool lower_filter_direct(const tqp_table* t, const FilterArgs& F, FilterDirectAr
     return true;
 }
 
-// Lower a filter call into kernel arguments and a launch shape.
-static tqp_status plan_filter(const tqp_ctx* ctx, const tqp_table* t, const tqp_pred* preds, int32_t npreds,
-                              const tqp_expr* sum_expr, bool ids, const tqp_tuning* force, FilterArgs* A,
-                              size_t* smem, int* grid, FilterScratch* lay) {
+// Lower a filter call's conditions and sum, and check its columns; *staged and
+// *staged_bytes: the columns a staged scan copies, and their bytes per row.
+static tqp_status lower_filter(const tqp_table* t, const tqp_pred* preds, int32_t npreds, const tqp_expr* sum_expr,
+                               FilterArgs* A, std::vector<int>* staged_cols, int* staged_bytes) {
     memset(A, 0, sizeof(*A));
     int ncond = 0;
     TQP_TRY(lower_preds(t, preds, npreds, A->cond, &ncond));
     A->ncond = ncond;
-    std::vector<int> staged;
+    std::vector<int>& staged = *staged_cols;
     for (int i = 0; i < ncond; ++i) staged.push_back(A->cond[i].col);
     if (sum_expr) {
         TQP_TRY(lower_expr(sum_expr, t->num_cols, &A->sum));
@@ -155,6 +155,13 @@ static tqp_status plan_filter(const tqp_ctx* ctx, const tqp_table* t, const tqp_
     }
     int bpr = 0;
     for (int c : u) bpr += t->cols[c].type == TQP_I64 ? 8 : (t->cols[c].type == TQP_I32 ? 4 : 1);
+    *staged_bytes = bpr;
+    return TQP_OK;
+}
+
+// The launch shape of a lowered filter as a staged scan.
+static tqp_status shape_filter(const tqp_ctx* ctx, const tqp_table* t, const std::vector<int>& staged, int bpr, bool ids,
+                               const tqp_tuning* force, FilterArgs* A, size_t* smem, int* grid, FilterScratch* lay) {
     const tqp_tuning tu = force ? *force : default_tuning(ctx, bpr, FilterBody::kSmemBytes + args_bytes<FilterArgs>());
     TQP_TRY(make_geom(ctx, t, staged, tu, FilterBody::kSmemBytes + args_bytes<FilterArgs>(), &A->G, smem));
     lower_fast(A->cond, A->ncond, A->G, A->cf, &A->fast);
@@ -164,7 +171,7 @@ static tqp_status plan_filter(const tqp_ctx* ctx, const tqp_table* t, const tqp_
     A->ctl.chunk_tiles = (A->G.ntiles + g - 1) / g;
     A->ctl.nchunks = (A->G.ntiles + A->ctl.chunk_tiles - 1) / A->ctl.chunk_tiles;
     *grid = static_cast<int>(A->ctl.nchunks);
-    *lay = filter_scratch_layout(A->G, ids);
+    *lay = filter_scratch_layout(A->G.n, A->G.ntiles * A->G.T, ids);
     return TQP_OK;
 }
 
@@ -220,22 +227,31 @@ tqp_status launch_filter(tqp_ctx* ctx, const tqp_table* t, const tqp_pred* preds
     size_t smem = 0;
     int grid = 0;
     FilterScratch lay;
-    TQP_TRY(plan_filter(ctx, t, preds, npreds, sum_expr, d_row_ids != nullptr, force, &A, &smem, &grid, &lay));
-    if (t->num_rows == 0) {
+    std::vector<int> staged;
+    int bpr = 0;
+    TQP_TRY(lower_filter(t, preds, npreds, sum_expr, &A, &staged, &bpr));
+    const long long n = t->num_rows;
+    if (n == 0) {
         TQP_CUDA(cudaMemsetAsync(d_count, 0, sizeof(int64_t), stream));
         if (d_sum) TQP_CUDA(cudaMemsetAsync(d_sum, 0, sizeof(int64_t), stream));
         return TQP_OK;
     }
-    void* scratch = arena_alloc(ctx, lay.bytes);
-    if (!scratch) return arena_oom(ctx, lay.bytes);
+    const bool ids = d_row_ids != nullptr;
     FilterDirectArgs D;
     if (!force && !user_shape(ctx) && tuned_variant(ctx, kFilterVariant) == 1 && lower_filter_direct(t, A, &D)) {
+        lay = filter_scratch_layout(n, (n + kFdStep - 1) / kFdStep * kFdStep, ids);
+        void* scratch = arena_alloc(ctx, lay.bytes);
+        if (!scratch) return arena_oom(ctx, lay.bytes);
         const long long step = kFdStep * (kFdThreads / kWarp), most = 1LL * kFdMinBlocks * ctx->num_sms;
-        while (D.steps > 1 && t->num_rows < most * step * D.steps) D.steps /= 2;  // every SM gets its blocks
-        const long long g = std::min<long long>((t->num_rows + step * D.steps - 1) / (step * D.steps), most);
+        while (D.steps > 1 && n < most * step * D.steps) D.steps /= 2;  // every SM gets its blocks
+        const long long g = std::min<long long>((n + step * D.steps - 1) / (step * D.steps), most);
+        A.G.n = n;
         return launch_filter_with(A, grid, smem, lay, scratch, ctx->d_err, ctx->wait_cap, d_row_ids, capacity, d_count,
                                   d_sum, stream, &D, static_cast<int>(g));
     }
+    TQP_TRY(shape_filter(ctx, t, staged, bpr, ids, force, &A, &smem, &grid, &lay));
+    void* scratch = arena_alloc(ctx, lay.bytes);
+    if (!scratch) return arena_oom(ctx, lay.bytes);
     return launch_filter_with(A, grid, smem, lay, scratch, ctx->d_err, ctx->wait_cap, d_row_ids, capacity, d_count,
                               d_sum, stream);
 }
@@ -338,8 +354,10 @@ extern "C" tqp_status tqp_filter_noalloc(int device, const tqp_table* t, const t
     size_t smem = 0;
     int grid = 0;
     FilterScratch lay;
-    TQP_TRY(plan_filter(&dev_info, t, preds, npreds, sum_expr, d_row_ids != nullptr, nullptr, &A, &smem, &grid,
-                        &lay));
+    std::vector<int> staged;
+    int bpr = 0;
+    TQP_TRY(lower_filter(t, preds, npreds, sum_expr, &A, &staged, &bpr));
+    TQP_TRY(shape_filter(&dev_info, t, staged, bpr, d_row_ids != nullptr, nullptr, &A, &smem, &grid, &lay));
     if (lay.bytes > kNoallocScratchBytes)
         return fail(TQP_ERR_INVALID_ARG, "tqp_filter_noalloc needs %zu scratch bytes, holds %zu", lay.bytes,
                     kNoallocScratchBytes);

@@ -12,6 +12,7 @@
 #include <map>
 #include <mutex>
 #include <string>
+#include <tuple>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -171,6 +172,8 @@ void expr_col_ids(const tqp_expr* e, std::vector<int>& cols);
 // floor(log2(max(n, 1))): the row-count part of a shape class.
 int rows_class(long long n);
 
+// Resident blocks per SM of a kernel (1 when the driver gives no answer).
+int resident_blocks(int device, const void* kernel, int threads, size_t smem);
 // Persistent grid size for an engine kernel.
 int engine_grid(const tqp_ctx* ctx, const void* kernel, size_t smem, int64_t ntiles, int ctas_per_sm);
 
