@@ -181,6 +181,7 @@ constexpr int kDirArgsBytes = (static_cast<int>(sizeof(GroupDirectArgs)) + 127) 
 constexpr long long kFlatRowsMax = 32768;
 constexpr long long kFlatRowsMin = 4096;
 constexpr long long kFlatBlocksPerSm = 12;
+constexpr long long kDirBlocksPerSm = 6;  // (the direct group-by's blocks clear and flush 64 KB of tables each)
 constexpr long long kDirRangeRowsPerBlock = 65536;
 
 struct TopItem {
@@ -1123,10 +1124,10 @@ static void plan_top_levels(tqp_batch* b) {
 
 // Blocks of the flat row launches, a contiguous range per job.
 template <class Job>
-static long long assign_blocks(const tqp_batch* b, std::vector<Job>& jobs) {
+static long long assign_blocks(const tqp_batch* b, std::vector<Job>& jobs, long long per_sm = kFlatBlocksPerSm) {
     long long rows = 0;
     for (const Job& j : jobs) rows += j.A.n;
-    const long long want = rows / (kFlatBlocksPerSm * b->ctx->num_sms);
+    const long long want = rows / (per_sm * b->ctx->num_sms);
     const long long per = std::min(kFlatRowsMax, std::max(kFlatRowsMin, want / 1024 * 1024));
     long long first = 0;
     for (Job& j : jobs) {
@@ -1139,7 +1140,7 @@ static long long assign_blocks(const tqp_batch* b, std::vector<Job>& jobs) {
 
 // Block -> job maps of every flattened phase, in one array.
 static void build_maps(tqp_batch* b) {
-    b->gdirect_blocks = assign_blocks(b, b->gdir);
+    b->gdirect_blocks = assign_blocks(b, b->gdir, kDirBlocksPerSm);
     for (int k = 0; k < 2; ++k) b->probe_blocks[k] = assign_blocks(b, b->probe[k]);
     b->filt_blocks = assign_blocks(b, b->filt);
     auto& M = b->maps;

@@ -29,7 +29,7 @@
 
 namespace tqp {
 
-tqp_status radix_sort_pairs(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, const long long* d_n,
+tqp_status radix_sort_pairs(const tqp_ctx* ctx, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, long long* d_n,
                             long long n_max, int begin_bit, int end_bit, void* scratch, cudaStream_t stream,
                             bool* result_in_1);
 size_t radix_sort_scratch(long long n_max);
@@ -148,6 +148,7 @@ __global__ void k_ht_runs(JoinHT H, const uint64_t* skey, const uint32_t* sval, 
     for (long long p = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; p < n;
          p += static_cast<long long>(gridDim.x) * blockDim.x) {
         const uint64_t s = skey[p];
+        if (s > static_cast<uint64_t>(H.cap)) continue;  // (a sort that gave up: the call reports it)
         if (p == 0 || skey[p - 1] != s) {
             const bool single = p + 1 == n || skey[p + 1] != s;
             H.slots[s].z = single ? (sval[p] | kRunRow) : static_cast<uint32_t>(p);
@@ -193,7 +194,7 @@ tqp_status ht_build(tqp_ctx* ctx, const tqp_table* build, int32_t key_col, JoinH
     int bits = 1;
     while ((1LL << bits) <= H->cap) ++bits;
     bool in1 = false;
-    TQP_TRY(radix_sort_pairs(k0, v0, k1, v1, d_n, n, 0, (bits + 7) / 8 * 8, rs, stream, &in1));
+    TQP_TRY(radix_sort_pairs(ctx, k0, v0, k1, v1, d_n, n, 0, (bits + 7) / 8 * 8, rs, stream, &in1));
     const uint64_t* sk = in1 ? k1 : k0;
     H->bidx = in1 ? v1 : v0;
     k_ht_runs<<<iblocks, threads, 0, stream>>>(*H, sk, H->bidx, n);
@@ -272,7 +273,7 @@ tqp_status ht_build_sorted(tqp_ctx* ctx, const tqp_table* build, int32_t key_col
     TQP_TRY(set_device_i64(d_n, n, stream));
     bool in1 = false;
     // key - min fits 32 bits for 32- and 8-bit key columns
-    TQP_TRY(radix_sort_pairs(k0, v0, k1, v1, d_n, n, 0, kc.type == TQP_I64 ? 64 : 32, rs, stream, &in1));
+    TQP_TRY(radix_sort_pairs(ctx, k0, v0, k1, v1, d_n, n, 0, kc.type == TQP_I64 ? 64 : 32, rs, stream, &in1));
     H->skeys = in1 ? k1 : k0;
     H->bidx = in1 ? v1 : v0;
     const int dblocks = static_cast<int>(std::min<long long>((n + threads) / threads, ctx->num_sms * 16LL));
@@ -588,7 +589,7 @@ static tqp_status launch_join_pairs(tqp_ctx* ctx, const tqp_table* build, int32_
         int bits = 1;
         while ((1LL << bits) <= T.cap) ++bits;
         bool in1 = false;
-        TQP_TRY(radix_sort_pairs(k0, v0, k1, v1, n_sort, nb, 0, (bits + 7) / 8 * 8, rs, stream, &in1));
+        TQP_TRY(radix_sort_pairs(ctx, k0, v0, k1, v1, n_sort, nb, 0, (bits + 7) / 8 * 8, rs, stream, &in1));
         const uint64_t* sk = in1 ? k1 : k0;
         uint32_t* rlen = reinterpret_cast<uint32_t*>(in1 ? k0 : k1);  // (the sort's other key buffer)
         T.bidx = in1 ? v1 : v0;

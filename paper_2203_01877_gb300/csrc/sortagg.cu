@@ -20,7 +20,7 @@
 
 namespace tqp {
 
-tqp_status radix_sort_pairs(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, const long long* d_n,
+tqp_status radix_sort_pairs(const tqp_ctx* ctx, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, long long* d_n,
                             long long n_max, int begin_bit, int end_bit, void* scratch, cudaStream_t stream,
                             bool* result_in_1);
 size_t radix_sort_scratch(long long n_max);
@@ -255,7 +255,7 @@ tqp_status launch_sort_agg(tqp_ctx* ctx, const tqp_table* t, const Cond* cond, i
     TQP_CUDA(cudaGetLastError());
     bool in1 = false;
     const int end_bit = std::max(8, (S->width + 7) / 8 * 8);
-    TQP_TRY(radix_sort_pairs(k0, v0, k1, v1, words, nn, 0, end_bit, rs, stream, &in1));
+    TQP_TRY(radix_sort_pairs(ctx, k0, v0, k1, v1, words, nn, 0, end_bit, rs, stream, &in1));
     A.skey = in1 ? k1 : k0;
     A.srow = in1 ? v1 : v0;
     k_sa_heads<<<static_cast<unsigned>(ntiles), kSaThreads, 0, stream>>>(A);
