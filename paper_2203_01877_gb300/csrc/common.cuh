@@ -57,6 +57,33 @@ __device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned l
 
 // ---- shared-memory addresses and mbarriers -------------------------------
 // Fire-and-forget 64-bit add to global memory (a RED, no value returned).
+// Barrier over the blocks of a cooperative launch (all resident): every thread
+// of every block calls it; `target` is the arrivals so far, blocks times
+// barriers. False after kGridWaitCap polls of 64 ns or more, or when a time-out
+// is already latched; the time-out is then latched.
+constexpr long long kGridWaitCap = 1LL << 24;
+__device__ __forceinline__ bool grid_barrier(unsigned int* bar, unsigned int target, int* err) {
+    __shared__ int ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(bar, 1u);
+        ok = 1;
+        long long polls = 0;
+        while (*reinterpret_cast<volatile unsigned int*>(bar) < target) {
+            if (++polls > kGridWaitCap || read_error(err) == TQP_ERR_TIMEOUT) {
+                ok = 0;
+                latch_error(err, TQP_ERR_TIMEOUT);
+                break;
+            }
+            __nanosleep(64);
+        }
+        __threadfence();
+    }
+    __syncthreads();
+    return ok != 0;
+}
+
 // Accumulator pointers often come from shared memory (staged kernel
 // arguments), where the compiler cannot tell that they address global memory
 // and would otherwise emit a generic atomic that returns the old value.

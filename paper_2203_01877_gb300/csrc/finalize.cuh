@@ -388,22 +388,25 @@ static __device__ void topsel_pass_block(const GroupSpec& S, int rank_acc, int k
             sel->done = 1;
             sel->empty = 1;
         } else {
+            // (volatile: an earlier pass of the same launch wrote these from another SM)
+            volatile TopSel* vs = sel;
             const int b = found_b;
             const long long hb = gh[b];
             int open;
             if (pass == 0) {
                 unsigned long long lo;
                 first_bin_interval(b, &lo, &open);
-                sel->thresh = lo;
+                vs->thresh = lo;
             } else {
                 open = shift;
-                sel->thresh |= static_cast<unsigned long long>(b) << shift;
+                vs->thresh = vs->thresh | static_cast<unsigned long long>(b) << shift;
             }
-            sel->known = open;
-            sel->above += found_above;
-            sel->need = need - found_above;
-            if (sel->above + hb <= kSelCand) sel->done = 1;
-            else if (open == 0) sel->fallback = 1;  // one value, too many ties
+            const long long above = vs->above + found_above;
+            vs->known = open;
+            vs->above = above;
+            vs->need = need - found_above;
+            if (above + hb <= kSelCand) vs->done = 1;
+            else if (open == 0) vs->fallback = 1;  // one value, too many ties
         }
         sel->blocks_done = 0;
     }

@@ -305,14 +305,22 @@ __global__ void __launch_bounds__(kTopThreads) k_topk_reduce(const __grid_consta
     topk_reduce_block(S, in, n_in, k, out, emit, O, total, total_out, blockIdx.x, run);
 }
 
-__global__ void __launch_bounds__(kSelThreads) k_topsel_pass(const __grid_constant__ GroupSpec S, int rank_acc, int k,
-                                                             TopSel* sel, int pass, long long nblocks) {
-    topsel_pass_block(S, rank_acc, k, sel, pass, blockIdx.x, nblocks);
-}
-
-__global__ void __launch_bounds__(kSelThreads) k_topsel_collect(const __grid_constant__ GroupSpec S, int rank_acc,
-                                                                TopSel* sel, TopBuf cand) {
-    topsel_collect_block(S, rank_acc, sel, cand, blockIdx.x);
+// Every pass and the collection of the candidates in one cooperative launch
+// (seven of about 2 us each otherwise; the passes after the deciding one are
+// skipped by all blocks alike).
+__global__ void __launch_bounds__(kSelThreads) k_topsel(const __grid_constant__ GroupSpec S, int rank_acc, int k, TopSel* sel,
+                                                        TopBuf cand, long long nblocks, unsigned int* bar, int* err) {
+    const volatile TopSel* vs = sel;
+    unsigned int arrivals = 0;
+    for (int pass = 0; pass < kSelPasses; ++pass) {
+        for (long long b = blockIdx.x; b < nblocks; b += gridDim.x) {
+            topsel_pass_block(S, rank_acc, k, sel, pass, b, nblocks);
+            __syncthreads();
+        }
+        if (!grid_barrier(bar, arrivals += gridDim.x, err)) return;
+        if (vs->done || vs->fallback) break;
+    }
+    for (long long b = blockIdx.x; b < nblocks; b += gridDim.x) topsel_collect_block(S, rank_acc, sel, cand, b);
 }
 
 __global__ void __launch_bounds__(kTopThreads) k_topsel_emit(const __grid_constant__ GroupSpec S, int k, const TopSel* sel,
@@ -342,13 +350,21 @@ tqp_status group_topk(tqp_ctx* ctx, const GroupSpec& S, const GroupOut& O, int k
     cand.slot = static_cast<uint32_t*>(arena_alloc(ctx, kSelCand * 4));
     if (!alloc_buf(&a) || !alloc_buf(&b) || !total || !sel || !cand.rank || !cand.key || !cand.slot)
         return arena_oom(ctx, ncand * 40 + sizeof(TopSel) + kSelCand * 20);
-    TQP_CUDA(cudaMemsetAsync(total, 0, 8, stream));
+    TQP_CUDA(cudaMemsetAsync(total, 0, 16, stream));
     TQP_CUDA(cudaMemsetAsync(sel, 0, sizeof(TopSel), stream));
     // radix select of the k-th largest, then one sort of the candidates
-    const long long nbs = (S.cap + 1 + kSelSlots - 1) / kSelSlots;
-    for (int pass = 0; pass < kSelPasses; ++pass)
-        k_topsel_pass<<<static_cast<unsigned>(nbs), kSelThreads, 0, stream>>>(S, rank_acc, k, sel, pass, nbs);
-    k_topsel_collect<<<static_cast<unsigned>(nbs), kSelThreads, 0, stream>>>(S, rank_acc, sel, cand);
+    long long nbs = (S.cap + 1 + kSelSlots - 1) / kSelSlots;
+    {
+        unsigned int* bar = reinterpret_cast<unsigned int*>(total + 1);
+        int* err = ctx->d_err;
+        const int most = resident_blocks(ctx->device, reinterpret_cast<const void*>(k_topsel), kSelThreads, 0) * ctx->num_sms;
+        GroupSpec Sc = S;
+        int ra = rank_acc, kk = k;
+        void* args[] = {&Sc, &ra, &kk, &sel, &cand, &nbs, &bar, &err};
+        TQP_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_topsel),
+                                             dim3(static_cast<unsigned>(std::min<long long>(nbs, most))), dim3(kSelThreads),
+                                             args, 0, stream));
+    }
     k_topsel_emit<<<1, kTopThreads, 0, stream>>>(S, k, sel, cand, O, total_groups);
     // the tournament, only when the select ended with too many ties (its blocks return early otherwise)
     const unsigned int* run = &sel->fallback;

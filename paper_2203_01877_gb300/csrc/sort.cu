@@ -21,7 +21,6 @@ constexpr int kSortItems = 16;                          // per thread
 constexpr int kSortTile = kSortThreads * kSortItems;    // 4096
 constexpr int kSortSlice = kSortTile / kSortWarps;      // 512 per warp
 constexpr int kSortBlocksPerSm = 4;
-constexpr long long kSortWaitCap = 1LL << 24;           // polls of a barrier, 64 ns or more each
 
 // Digit counts of tiles blockIdx.x, blockIdx.x + gridDim.x, ...
 __device__ __forceinline__ void rs_upsweep(const uint64_t* keys, long long n, int shift, uint32_t* hist, long long ntiles,
@@ -137,30 +136,6 @@ __device__ __forceinline__ void rs_downsweep(const uint64_t* kin, const uint32_t
     }
 }
 
-// Every block arrives (the launch is cooperative, so all are resident); false
-// after kSortWaitCap polls, with the time-out latched.
-__device__ __forceinline__ bool rs_barrier(unsigned int* bar, unsigned int target, int* err) {
-    __shared__ int ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(bar, 1u);
-        ok = 1;
-        long long polls = 0;
-        while (*reinterpret_cast<volatile unsigned int*>(bar) < target) {
-            if (++polls > kSortWaitCap || read_error(err) == TQP_ERR_TIMEOUT) {
-                ok = 0;
-                latch_error(err, TQP_ERR_TIMEOUT);
-                break;
-            }
-            __nanosleep(64);
-        }
-        __threadfence();
-    }
-    __syncthreads();
-    return ok != 0;
-}
-
 // All passes in one cooperative launch. An empty input (a build side of unique
 // keys, a group-by over key ranges) costs this one launch instead of four per
 // pass: 12 to 16 launches of about 2 us each.
@@ -176,12 +151,12 @@ __global__ void __launch_bounds__(kSortThreads, kSortBlocksPerSm) k_rs_sort(uint
     unsigned int arrivals = 0;
     for (int shift = begin_bit; shift < end_bit; shift += 8) {
         rs_upsweep(k0, n, shift, hist, ntiles, digit_tot, wcnt[0]);
-        if (!rs_barrier(bar, arrivals += gridDim.x, err)) break;
+        if (!grid_barrier(bar, arrivals += gridDim.x, err)) break;
         rs_scan(hist, ntiles, digit_tot, wsum);
-        if (!rs_barrier(bar, arrivals += gridDim.x, err)) break;
+        if (!grid_barrier(bar, arrivals += gridDim.x, err)) break;
         if (blockIdx.x == 0) digit_tot[threadIdx.x] = 0;  // (read by the scans only; the next barrier orders it)
         rs_downsweep(k0, v0, k1, v1, n, shift, hist, ntiles, wcnt);
-        if (!rs_barrier(bar, arrivals += gridDim.x, err)) break;
+        if (!grid_barrier(bar, arrivals += gridDim.x, err)) break;
         uint64_t* k = k0;
         k0 = k1;
         k1 = k;
