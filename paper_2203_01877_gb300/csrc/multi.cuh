@@ -17,13 +17,15 @@
 //     search over the sorted breakpoints.  The cost per row grows with the
 //     number of condition columns, not with the number of queries;
 //   * accumulation: lane q keeps query q's count and sum in registers. Rows that
-//     pass some query join a queue of their warp (pass mask and values, in shared
-//     memory); for every 32 of them the masks are transposed (five exchange
-//     steps), so that lane q holds the rows that pass query q: its count is a bit
-//     count, and it adds their values. 60M rows and 32 queries of 2% each took 654
-//     us with a shared-memory atomic per (row, passing query) pair instead: the
-//     lanes wait for the one with most pairs, 244 warp instructions per 32 rows.
-//     At the end of a chunk lane q moves query q's totals to global memory;
+//     pass some query join a queue of their warp (pass mask and row, in shared
+//     memory); 32 at a time their values are computed, one row per lane, and the
+//     masks are transposed (five exchange steps), so that lane q holds the rows
+//     that pass query q: its count is a bit count, and it adds their values. 60M
+//     rows and 32 queries of 2% each took 654 us with a shared-memory atomic per
+//     (row, passing query) pair instead (the lanes wait for the one with most
+//     pairs, 244 warp instructions per 32 rows), now 553; values computed for whole
+//     steps before the queue: 529, but 443 against 421 with 5 queries. At the end
+//     of a chunk lane q moves query q's totals to global memory;
 //   * per-query row ranges: a query may cover only rows [rlo, rhi) of the
 //     scan (queries over slices of one table).  Per tile a ballot splits the
 //     queries into those covering the whole tile and those touching part of
@@ -47,8 +49,8 @@ constexpr int kMqBreaks = 512;      // breakpoints of the searched tables (share
 constexpr int kMqDirectMax = 4096;  // direct tables: at most this many entries per column
 constexpr int kMqRows = 4;          // rows per lane of a step
 constexpr int kMqQueue = (kMqRows + 1) * kWarp;  // queued rows of a warp: a step's and fewer than kWarp before it
-// the queue of each consumer warp: per row a value for each sum expression, and its pass mask
-constexpr int kMqAccBytes = kConsumerWarps * kMqQueue * (kMqExprs * 8 + 4);
+// per consumer warp: 32 rows' values for each sum expression; the queued rows' pass masks and tile rows
+constexpr int kMqAccBytes = kConsumerWarps * (kMqExprs * kWarp * 8 + kMqQueue * 8);
 
 // Shared memory of one launch's body: row queues | mask words | breakpoints.
 __host__ __device__ constexpr int mq_words_bytes(int nwords) { return (nwords * 4 + 15) / 16 * 16; }
@@ -165,8 +167,9 @@ struct MultiBody {
     const MultiArgs& A;
     const uint32_t* w;         // shared-memory copy of the masks
     const int64_t* bk;         // shared-memory copy of the breakpoints
-    unsigned long long* qval;  // this warp's queue: values [expression][row], and masks
+    unsigned long long* qval;  // this warp's values [expression][lane], and its queue: masks and tile rows
     uint32_t* qmask;
+    uint32_t* qrow;
     int qn = 0;                // queued rows (warp-uniform)
     unsigned long long qsum = 0;  // lane q: query q's sum and count since the last chunk
     unsigned int qcnt = 0;
@@ -192,8 +195,9 @@ struct MultiBody {
         const int warp = threadIdx.x / kWarp;
         const int lane = threadIdx.x % kWarp;
         const int cw = warp < kConsumerWarps ? warp : 0;
-        qval = reinterpret_cast<unsigned long long*>(sm) + cw * kMqExprs * kMqQueue;
-        qmask = reinterpret_cast<uint32_t*>(sm + kConsumerWarps * kMqExprs * kMqQueue * 8) + cw * kMqQueue;
+        qval = reinterpret_cast<unsigned long long*>(sm) + cw * kMqExprs * kWarp;
+        qmask = reinterpret_cast<uint32_t*>(sm + kConsumerWarps * kMqExprs * kWarp * 8) + cw * 2 * kMqQueue;
+        qrow = qmask + kMqQueue;
         if (lane < a.nq) {
             rlo = out[lane].rlo;
             rhi = out[lane].rhi;
@@ -213,7 +217,7 @@ struct MultiBody {
 
     // Full tiles with direct tables only: descriptors in registers, each
     // lookup a clamp and one shared-memory load.  Rows rb + lane + 32 j.
-    __device__ __forceinline__ void fast_step(const TileView& v, int rb, int lane, uint32_t full, uint32_t part) {
+    __device__ __forceinline__ void fast_step(const ScanGeom& G, const TileView& v, int rb, int lane, uint32_t full, uint32_t part) {
         constexpr int U = kU;
         const int r0 = rb + lane;
         uint32_t m[U];
@@ -249,7 +253,7 @@ struct MultiBody {
                 for (int j = 0; j < U; ++j) m[j] &= w[h.off + (min(max(x[j], lo), hi) - lo)];
             }
         }
-        accumulate<U>(v, r0, m);
+        add_rows<U>(G, v, r0, m);
     }
 
     // Queries whose row range ends inside the tile: their bits, row by row.
@@ -269,39 +273,37 @@ struct MultiBody {
         }
     }
 
-    // Sum expressions of full-tile rows and every (row, passing query) pair.
-    template <int U>
-    __device__ __forceinline__ void accumulate(const TileView& v, int r0, const uint32_t (&m)[U]) {
-        uint32_t mor = 0;
-#pragma unroll
-        for (int j = 0; j < U; ++j) mor |= m[j];
-        if (!__any_sync(0xffffffffu, mor != 0u)) return;
-        int64_t v0[U], v1[U];
-#pragma unroll
-        for (int j = 0; j < U; ++j) v0[j] = v1[j] = 0;
-        if (A.nexpr > 0) {
-            prod_eval<U>(A.e[0], v.stage, r0, v0);
-            if (A.nexpr > 1) prod_eval<U>(A.e[1], v.stage, r0, v1);
-        }
-        add_pairs<U>(m, v0, v1);
-    }
-
-    // The last up to kWarp queued rows (from `first` on) into the queries they pass.
-    __device__ __forceinline__ void flush(int first, int lane) {
+    // The last (up to kWarp) queued rows, from `first` on, into the queries they pass.
+    __device__ __forceinline__ void flush(const ScanGeom& G, const TileView& v, int first, int lane) {
         __syncwarp();
-        uint32_t x = warp_transpose(first + lane < qn ? qmask[first + lane] : 0u, lane);  // the rows of this lane's query
+        const bool in = first + lane < qn;
+        const uint32_t m = in ? qmask[first + lane] : 0u;
+        if (A.nexpr > 0 && in) {
+            const int r = static_cast<int>(qrow[first + lane]);
+#pragma unroll
+            for (int e = 0; e < kMqExprs; ++e) {
+                if (e >= A.nexpr) break;
+                int64_t x[1];
+                if (v.full) prod_eval<1>(A.e[e], v.stage, r, x);
+                else x[0] = static_cast<int64_t>(static_cast<uint64_t>(mq_factor_row(G, v, A.e[e], 0, A.ecol[e][0], r)) *
+                                                 static_cast<uint64_t>(mq_factor_row(G, v, A.e[e], 1, A.ecol[e][1], r)));
+                qval[e * kWarp + lane] = static_cast<unsigned long long>(x[0]);
+            }
+        }
+        __syncwarp();
+        uint32_t x = warp_transpose(m, lane);  // the rows of this lane's query
         qcnt += __popc(x);
         if (A.nexpr > 0) {
-            const unsigned long long* v = qval + ((A.esel >> lane) & 1u) * kMqQueue + first;
-            for (; x; x &= x - 1) qsum += v[__ffs(x) - 1];
+            const unsigned long long* val = qval + ((A.esel >> lane) & 1u) * kWarp;
+            for (; x; x &= x - 1) qsum += val[__ffs(x) - 1];
         }
         qn = first;
         __syncwarp();  // (read before the next rows take their place)
     }
 
-    // The step's rows that pass some query into the queue (every lane calls it).
+    // The step's rows (r0 + 32 j) that pass some query into the queue (every lane calls it).
     template <int U>
-    __device__ __forceinline__ void add_pairs(const uint32_t (&m)[U], const int64_t (&v0)[U], const int64_t (&v1)[U]) {
+    __device__ __forceinline__ void add_rows(const ScanGeom& G, const TileView& v, int r0, const uint32_t (&m)[U]) {
         static_assert(U == kMqRows, "the queue holds a step's rows");
         const uint32_t lt = lanemask_lt();
 #pragma unroll
@@ -310,12 +312,11 @@ struct MultiBody {
             if (m[j]) {
                 const int at = qn + __popc(b & lt);
                 qmask[at] = m[j];
-                if (A.nexpr > 0) qval[at] = static_cast<unsigned long long>(v0[j]);
-                if (A.nexpr > 1) qval[kMqQueue + at] = static_cast<unsigned long long>(v1[j]);
+                qrow[at] = static_cast<uint32_t>(r0 + kWarp * j);
             }
             qn += __popc(b);
         }
-        while (qn >= kWarp) flush(qn - kWarp, static_cast<int>(threadIdx.x % kWarp));
+        while (qn >= kWarp) flush(G, v, qn - kWarp, static_cast<int>(threadIdx.x % kWarp));
     }
 
     // General path (a ragged last tile, searched tables, more than
@@ -341,30 +342,7 @@ struct MultiBody {
 #pragma unroll
             for (int j = 0; j < U; ++j) m[j] &= mq_lookup(mc, x[j], w, bk);
         }
-        if (v.full) {
-            accumulate<U>(v, r0, m);
-            return;
-        }
-        uint32_t mor = 0;
-#pragma unroll
-        for (int j = 0; j < U; ++j) mor |= m[j];
-        if (!__any_sync(0xffffffffu, mor != 0u)) return;
-        // sum expressions of the passing rows, the columns read through col_val
-        int64_t v0[U], v1[U];
-#pragma unroll
-        for (int j = 0; j < U; ++j) {
-            v0[j] = v1[j] = 0;
-            const int r = r0 + kWarp * j;
-            if (m[j] && A.nexpr > 0) {
-                v0[j] = static_cast<int64_t>(static_cast<uint64_t>(mq_factor_row(G, v, A.e[0], 0, A.ecol[0][0], r)) *
-                                             static_cast<uint64_t>(mq_factor_row(G, v, A.e[0], 1, A.ecol[0][1], r)));
-                if (A.nexpr > 1)
-                    v1[j] = static_cast<int64_t>(
-                        static_cast<uint64_t>(mq_factor_row(G, v, A.e[1], 0, A.ecol[1][0], r)) *
-                        static_cast<uint64_t>(mq_factor_row(G, v, A.e[1], 1, A.ecol[1][1], r)));
-            }
-        }
-        add_pairs<U>(m, v0, v1);
+        add_rows<U>(G, v, r0, m);
     }
 
     __device__ void pass1(const ScanGeom& G, const TileView& v, int cw, int lane) {
@@ -376,17 +354,15 @@ struct MultiBody {
         if (!(full | part)) return;
         const int rw = G.T / kConsumerWarps;  // a multiple of 128
         if (v.full && fast) {
-            for (int r = 0; r < rw; r += kU * kWarp) fast_step(v, cw * rw + r, lane, full, part);
-            return;
+            for (int r = 0; r < rw; r += kU * kWarp) fast_step(G, v, cw * rw + r, lane, full, part);
+        } else {
+            for (int r = 0; r < rw && cw * rw + r < v.rows; r += kU * kWarp)
+                step(G, v, cw * rw + r, lane, full, part);
         }
-        for (int r = 0; r < rw; r += kU * kWarp) {
-            if (cw * rw + r >= v.rows) return;
-            step(G, v, cw * rw + r, lane, full, part);
-        }
+        if (qn > 0) flush(G, v, 0, lane);  // (the tile's columns are there until the pass ends)
     }
 
     __device__ void chunk_end(const ScanGeom&, long long, long long, long long, int, int lane) {
-        if (qn > 0) flush(0, lane);
         const unsigned long long ls = qsum;
         const unsigned long long lc = qcnt;
         qsum = 0;
