@@ -268,6 +268,16 @@ __device__ __forceinline__ uint32_t sf_find(const uint32_t (&w)[NW], const uint3
     return M;
 }
 
+// Word i of the string (zero past its words).
+template <int NW>
+__device__ __forceinline__ uint32_t sf_word(const uint32_t (&w)[NW], int i) {
+    uint32_t x = 0;
+#pragma unroll
+    for (int j = 0; j < NW; ++j)
+        if (i == j) x = w[j];
+    return x;
+}
+
 template <int NW>
 __device__ __forceinline__ bool sf_like(const uint32_t (&w)[NW], const StrFastPred& q, const uint32_t* prog) {
     // the string's length: its first zero byte (the lowest set bit of the first word with one)
@@ -300,16 +310,22 @@ __device__ __forceinline__ bool sf_like(const uint32_t (&w)[NW], const StrFastPr
             pos = len;
             continue;
         }
+        if (k == q.count - 1 && (q.flags & kLikeEnd)) {  // at n - len (>= pos) only
+            const int at = n - len, i0 = at >> 2, sh = 8 * (at & 3);
+            uint32_t d = 0, lo = sf_word<NW>(w, i0);
+            for (int c = 0; 4 * c < len; ++c) {
+                const uint32_t hi = sf_word<NW>(w, i0 + c + 1);
+                d |= (__funnelshift_r(lo, hi, sh) ^ chunk[2 * c]) & chunk[2 * c + 1];
+                lo = hi;
+            }
+            return d == 0;
+        }
         // starts from which the segment ends within the string
         uint32_t M = sf_find<NW>(w, chunk, len) & (n - len >= 31 ? ~0u : (2u << (n - len)) - 1u);
-        if (k == q.count - 1 && (q.flags & kLikeEnd)) {
-            return (M >> (n - len)) & 1u;  // (n - len >= pos)
-        } else {
-            M &= ~0u << pos;
-            if (!M) return false;
-            pos = __ffs(M) - 1 + len;
-            if (pos >= 32 && k + 1 < q.count) return false;  // nothing is left for the next segment
-        }
+        M &= ~0u << pos;
+        if (!M) return false;
+        pos = __ffs(M) - 1 + len;
+        if (pos >= 32 && k + 1 < q.count) return false;  // nothing is left for the next segment
     }
     return true;
 }
