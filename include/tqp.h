@@ -201,12 +201,15 @@ TQP_API tqp_status tqp_ctx_set_tuning(tqp_ctx* ctx, int32_t tile_rows, int32_t s
  *     (paper Section 5.3's hash join), 1 = the sort-based join (Section 5.2,
  *     Algorithm 1: the build keys are radix-sorted with their rows and each
  *     probe key is bucketized into them);
+ *   tqp_filter: 0 = the staged scan, 1 = plain vector loads (one to four
+ *     conditions, a sum that is a product of two affine factors, or none);
  *   grouped join plans with at least 2^20 fact rows: 0 = the radix-partitioned
  *     aggregation (the probe side partitioned by group, each partition
  *     aggregated in shared memory), 1 = the fused probe (every joined row
  *     added to its key's or group's accumulators with L2 reductions).
  * -1 restores the default (the autotuner's choice, which times both; else 0 for
- * tqp_hash_join and 1, the fused probe, for grouped join plans).
+ * tqp_hash_join, 1 for tqp_filter and 1, the fused probe, for grouped join
+ * plans).
  * Errors: TQP_ERR_INVALID_ARG. */
 TQP_API tqp_status tqp_ctx_set_variant(tqp_ctx* ctx, int32_t variant);
 
