@@ -31,7 +31,9 @@ constexpr int kFdWord = 3;
 constexpr int kFdByte = 2;
 constexpr int kFdConds = 4;                        // in all
 constexpr int kFdStep = 4 * kWarp;                 // rows of a warp step
-constexpr int kFdSteps = 8;                        // consecutive steps of a warp (a power of two)
+constexpr int kFdSteps = 4;                        // consecutive steps of a warp (a power of two): 60M rows take 222
+                                                   // us a call, with 8 or 16 (a last wave mostly empty) 224 and 252,
+                                                   // with 2 (an atomic per 256 rows) 234
 constexpr int kFdDense = kFdStep / 4;              // passing rows of a step from which its lanes read their factors
 constexpr int kFdQueue = kFdDense + kWarp;         // queued rows of a warp
 constexpr int32_t kFdI64A32 = 16;                  // int64 column on a 32-byte boundary
