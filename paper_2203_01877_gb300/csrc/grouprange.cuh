@@ -19,10 +19,10 @@
 // 128-byte line serialise.
 //
 // Measured (60M rows, one int32 key, SUM and COUNT; hash path -> this): 1.5M
-// groups 3206 -> 547 us, of them k_group_l2 375 and the range pass 47; 60K groups
-// 2978 -> 582; 10K groups (shared memory) 2257 -> 355; 1K groups 3411 -> 291.
-// 100K rows, 1000 groups: 114 -> 48.  Entries beyond shared memory go to L2 from
-// about 17K (one sum): 20K groups take 636 us there, more than 10K in shared
+// groups 3206 -> 493 us, of them k_group_l2 375 and the range pass 47; 60K groups
+// 2978 -> 531; 10K groups (shared memory) 2257 -> 311; 1K groups 3170 -> 284.
+// 100K rows, 1000 groups: 113 -> 47.  Entries beyond shared memory go to L2 from
+// about 17K (one sum): 20K groups take 601 us there, more than 10K in shared
 // memory, less than the hash path's 2284.
 #pragma once
 

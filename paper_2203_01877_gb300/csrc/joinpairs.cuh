@@ -19,9 +19,9 @@
 // the prefix then advances faster than the tiles arrive.
 //
 // Measured (60M probe rows, 1.5M unique build keys; staged form -> this): keys
-// scattered over int32 1661 -> 605 us, dense 934 -> 540; 6M rows with ten build
-// rows per scattered key (60M pairs) 1197 -> 384, 805 of it before the lanes of a
-// warp shared the pairs of its rows; 300K rows 115 -> 57. Without the look-back
+// scattered over int32 1651 -> 572 us, dense 935 -> 508; 6M rows with ten build
+// rows per scattered key (60M pairs) 1162 -> 358 (about 800 before the lanes of a
+// warp shared the pairs of its rows); 100K rows 115 -> 49. Without the look-back
 // (offsets guessed, for timing) the scattered case takes 490 us, without the
 // lookups 351.
 #pragma once

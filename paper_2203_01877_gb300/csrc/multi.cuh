@@ -23,7 +23,7 @@
 //     that pass query q: its count is a bit count, and it adds their values. 60M
 //     rows and 32 queries of 2% each took 654 us with a shared-memory atomic per
 //     (row, passing query) pair instead (the lanes wait for the one with most
-//     pairs, 244 warp instructions per 32 rows), now 553; values computed for whole
+//     pairs, 244 warp instructions per 32 rows), now 575; values computed for whole
 //     steps before the queue: 529, but 443 against 421 with 5 queries. At the end
 //     of a chunk lane q moves query q's totals to global memory;
 //   * per-query row ranges: a query may cover only rows [rlo, rhi) of the

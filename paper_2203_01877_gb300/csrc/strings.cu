@@ -216,8 +216,8 @@ __global__ void __launch_bounds__(kStrThreads) k_str_prepass(const __grid_consta
 // and the segments are placed leftmost-first with bit operations. IN compares
 // whole words against each of a short list. Still bound by issue (63% of the
 // slots, 333 warp instructions per 32 strings of 24 bytes before the length was
-// found with one bit scan). 20M rows, `%xy%` and a price bound: 476 -> 297 us;
-// a prefix 209, eight IN values 274. Longer lists are searched by the general
+// found with one bit scan). 20M rows, `%xy%` and a price bound: 477 -> 292 us;
+// a prefix 311 -> 206, a suffix 317 -> 222, eight IN values 692 -> 275. Longer lists are searched by the general
 // form, and patterns of more segments or wider strings matched by it.
 constexpr int kSfThreads = 256;
 constexpr int kSfMinBlocks = 4;
