@@ -210,9 +210,11 @@ __device__ __forceinline__ void pa_combine(unsigned long long* base, uint32_t st
 
 // x added to entry e of a CTA's table of D entries: D counts, then per value D
 // low and D high words (the low word's atomic returns what the carry needs).
-__device__ __forceinline__ void pa_smem_add(uint32_t* tab, uint32_t D, uint32_t e, int nv,
+// True when the 32-bit count wrapped: the CTA's own rows (below 2^31) cannot,
+// the joined rows of keys with many build rows can.
+__device__ __forceinline__ bool pa_smem_add(uint32_t* tab, uint32_t D, uint32_t e, int nv,
                                             const unsigned long long (&x)[3]) {
-    atomicAdd(&tab[e], 1u);
+    const uint32_t c = atomicAdd(&tab[e], 1u);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         if (a >= nv) break;
@@ -222,6 +224,7 @@ __device__ __forceinline__ void pa_smem_add(uint32_t* tab, uint32_t D, uint32_t 
         const uint32_t xh = static_cast<uint32_t>(x[a] >> 32) + (old + xl < old ? 1u : 0u);
         if (xh) atomicAdd(lo + D, xh);
     }
+    return c == ~0u;
 }
 
 // The table into global entries of nv + 1 words (neighbouring words on neighbouring lanes).
@@ -231,7 +234,7 @@ __device__ __forceinline__ void pa_smem_flush(const uint32_t* tab, uint32_t D, i
     for (uint32_t i = threadIdx.x; i < D * W; i += blockDim.x) {
         const uint32_t e = i / W, a = i % W;
         unsigned long long x = tab[e];
-        if (a > 0 && x) {
+        if (a > 0) {  // (also of an entry whose count wrapped to 0)
             const uint32_t* lo = tab + (2 * a - 1) * D + e;
             x = static_cast<unsigned long long>(lo[0]) | (static_cast<unsigned long long>(lo[D]) << 32);
         }
@@ -245,7 +248,9 @@ static __device__ __noinline__ void pa_add_chain(const ProbeAggArgs& A, uint32_t
     for (uint32_t k = 0; k < cnt; ++k) {
         if (tab) {
             const unsigned long long x[3] = {x0, x1, 0};
-            pa_smem_add(tab, D, __ldg(&A.dgs[d]), A.nval, x);
+            const uint32_t g = __ldg(&A.dgs[d]);
+            if (pa_smem_add(tab, D, g, A.nval, x))  // the count's carry
+                red_add_u64(A.gacc + static_cast<long long>(g) * (A.nval + 1), 1ULL << 32);
             if (k + 1 < cnt) d = __ldg(&A.next[d]);
             continue;
         }
