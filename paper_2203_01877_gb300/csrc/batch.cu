@@ -374,13 +374,14 @@ __global__ void __launch_bounds__(kTopThreads) k_b_topk(const TopJob* T, const T
 }
 
 // Passes [first, last) of every plan's radix select, then (collect) its
-// candidates. Blocks up to what the chip holds take all of it in one cooperative
+// candidates. Blocks up to half of what the chip holds take all of it in one cooperative
 // launch with grid barriers instead of seven launches (4 plans over 200K-row
 // dimensions: 170 -> 155 us per call); beyond, each pass has its own launch, whose
 // blocks need not queue behind one another (64 plans, 1500 blocks: 689 against
 // 701 us).
 __global__ void __launch_bounds__(kSelThreads) k_b_sel(const TopJob* T, const int32_t* bjob, long long nblocks, int first,
-                                                       int last, int collect, unsigned int* bar, int* err) {
+                                                       int last, int collect, unsigned int* bar, int* err,
+                                                       long long wait_cap) {
     unsigned int arrivals = 0;
     for (int pass = first; pass < last; ++pass) {
         for (long long b = blockIdx.x; b < nblocks; b += gridDim.x) {
@@ -388,7 +389,7 @@ __global__ void __launch_bounds__(kSelThreads) k_b_sel(const TopJob* T, const in
             topsel_pass_block(t.S, t.rank_acc, t.k, t.sel, pass, b - t.sel_block, t.sel_nblocks);
             __syncthreads();
         }
-        if (bar && !grid_barrier(bar, arrivals += gridDim.x, err)) return;
+        if (bar && !grid_barrier(bar, arrivals += gridDim.x, err, wait_cap)) return;
     }
     if (!collect) return;
     for (long long b = blockIdx.x; b < nblocks; b += gridDim.x) {
@@ -1292,16 +1293,17 @@ static tqp_status batch_launch(tqp_batch* b, cudaStream_t st) {
         long long nblocks = b->sel_blocks;
         unsigned int* bar = reinterpret_cast<unsigned int*>(b->selbar);
         int* err = ctx->d_err;
+        long long cap = ctx->wait_cap;
         int first = 0, last = kSelPasses, collect = 1;
         const dim3 grid(static_cast<unsigned>(nblocks));
         if (nblocks <= resident_blocks(ctx->device, reinterpret_cast<const void*>(k_b_sel), kSelThreads, 0) * 1LL *
                            ctx->num_sms / 2) {
-            void* args[] = {&top, &map, &nblocks, &first, &last, &collect, &bar, &err};
+            void* args[] = {&top, &map, &nblocks, &first, &last, &collect, &bar, &err, &cap};
             TQP_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_b_sel), grid, dim3(kSelThreads), args, 0, st));
         } else {
             for (int pass = 0; pass < kSelPasses; ++pass)
-                k_b_sel<<<grid, kSelThreads, 0, st>>>(top, map, nblocks, pass, pass + 1, 0, nullptr, err);
-            k_b_sel<<<grid, kSelThreads, 0, st>>>(top, map, nblocks, 0, 0, 1, nullptr, err);
+                k_b_sel<<<grid, kSelThreads, 0, st>>>(top, map, nblocks, pass, pass + 1, 0, nullptr, err, cap);
+            k_b_sel<<<grid, kSelThreads, 0, st>>>(top, map, nblocks, 0, 0, 1, nullptr, err, cap);
         }
         k_b_selemit<<<static_cast<unsigned>(b->top.size()), kTopThreads, 0, st>>>(b->d_top);
     }

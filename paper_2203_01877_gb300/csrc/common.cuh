@@ -55,35 +55,38 @@ __device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned l
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-// ---- shared-memory addresses and mbarriers -------------------------------
-// Fire-and-forget 64-bit add to global memory (a RED, no value returned).
+// ---- barrier over a cooperative grid ---------------------------------------
 // Barrier over the blocks of a cooperative launch (all resident): every thread
-// of every block calls it; `target` is the arrivals so far, blocks times
-// barriers. False after kGridWaitCap polls of 64 ns or more, or when a time-out
-// is already latched; the time-out is then latched.
-constexpr long long kGridWaitCap = 1LL << 24;
-__device__ __forceinline__ bool grid_barrier(unsigned int* bar, unsigned int target, int* err) {
+// of every block calls it; `bar` starts at 0, `target` is the arrivals so far,
+// blocks times barriers. A block that has polled `cap` times (with back-off)
+// gives up: it latches the time-out and marks `bar`, and every block that finds
+// the mark gives up as well. False for those.
+constexpr unsigned int kGridGaveUp = 0x80000000u;  // (above any number of arrivals)
+__device__ __forceinline__ bool grid_barrier(unsigned int* bar, unsigned int target, int* err, long long cap) {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         atomicAdd(bar, 1u);
-        ok = 1;
+        unsigned int v;
         long long polls = 0;
-        while (*reinterpret_cast<volatile unsigned int*>(bar) < target) {
-            if (++polls > kGridWaitCap || read_error(err) == TQP_ERR_TIMEOUT) {
-                ok = 0;
+        while ((v = *reinterpret_cast<volatile unsigned int*>(bar)) < target) {
+            if (++polls > cap) {
                 latch_error(err, TQP_ERR_TIMEOUT);
+                v = atomicOr(bar, kGridGaveUp) | kGridGaveUp;
                 break;
             }
             __nanosleep(64);
         }
+        ok = (v & kGridGaveUp) == 0;
         __threadfence();
     }
     __syncthreads();
     return ok != 0;
 }
 
+// ---- shared-memory addresses and mbarriers -------------------------------
+// Fire-and-forget 64-bit add to global memory (a RED, no value returned).
 // Accumulator pointers often come from shared memory (staged kernel
 // arguments), where the compiler cannot tell that they address global memory
 // and would otherwise emit a generic atomic that returns the old value.

@@ -440,7 +440,10 @@ static __device__ void topsel_emit_block(const GroupSpec& S, int k, const TopSel
     __shared__ uint64_t kk[kTopBlock];
     __shared__ uint32_t ss[kTopBlock];
     const volatile TopSel* vs = sel;
-    if (!vs->done) return;
+    if (!vs->done) {
+        if (!vs->fallback && threadIdx.x == 0) *O.num_groups = -1;  // the select gave up (the call reports it)
+        return;
+    }
     const long long total = vs->total;
     const int n = vs->empty ? 0 : static_cast<int>(vs->ncand < static_cast<unsigned int>(kSelCand) ? vs->ncand
                                                                                                   : kSelCand);
@@ -457,9 +460,13 @@ static __device__ void topsel_emit_block(const GroupSpec& S, int k, const TopSel
             ss[i] = 0xFFFFFFFFu;
         }
     }
+    const long long m = total < k ? total : k;
+    if (m > n) {  // the select gave up before every candidate was collected
+        if (threadIdx.x == 0) *O.num_groups = -1;
+        return;
+    }
     __syncthreads();
     top_sort_block(r, kk, ss, n2);
-    const long long m = total < k ? total : k;
     if (m > O.capacity) {
         if (threadIdx.x == 0) {
             *O.num_groups = -1;

@@ -309,7 +309,8 @@ __global__ void __launch_bounds__(kTopThreads) k_topk_reduce(const __grid_consta
 // (seven of about 2 us each otherwise; the passes after the deciding one are
 // skipped by all blocks alike).
 __global__ void __launch_bounds__(kSelThreads) k_topsel(const __grid_constant__ GroupSpec S, int rank_acc, int k, TopSel* sel,
-                                                        TopBuf cand, long long nblocks, unsigned int* bar, int* err) {
+                                                        TopBuf cand, long long nblocks, unsigned int* bar, int* err,
+                                                        long long wait_cap) {
     const volatile TopSel* vs = sel;
     unsigned int arrivals = 0;
     for (int pass = 0; pass < kSelPasses; ++pass) {
@@ -317,7 +318,7 @@ __global__ void __launch_bounds__(kSelThreads) k_topsel(const __grid_constant__ 
             topsel_pass_block(S, rank_acc, k, sel, pass, b, nblocks);
             __syncthreads();
         }
-        if (!grid_barrier(bar, arrivals += gridDim.x, err)) return;
+        if (!grid_barrier(bar, arrivals += gridDim.x, err, wait_cap)) return;
         if (vs->done || vs->fallback) break;
     }
     for (long long b = blockIdx.x; b < nblocks; b += gridDim.x) topsel_collect_block(S, rank_acc, sel, cand, b);
@@ -360,7 +361,8 @@ tqp_status group_topk(tqp_ctx* ctx, const GroupSpec& S, const GroupOut& O, int k
         const int most = resident_blocks(ctx->device, reinterpret_cast<const void*>(k_topsel), kSelThreads, 0) * ctx->num_sms;
         GroupSpec Sc = S;
         int ra = rank_acc, kk = k;
-        void* args[] = {&Sc, &ra, &kk, &sel, &cand, &nbs, &bar, &err};
+        long long wait_cap = ctx->wait_cap;
+        void* args[] = {&Sc, &ra, &kk, &sel, &cand, &nbs, &bar, &err, &wait_cap};
         TQP_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_topsel),
                                              dim3(static_cast<unsigned>(std::min<long long>(nbs, most))), dim3(kSelThreads),
                                              args, 0, stream));

@@ -144,11 +144,11 @@ constexpr uint32_t kRunRow = 0x80000000u;
 // below 2^31 - 1, so no flagged row collides with it.)
 constexpr uint32_t kRunNone = 0xFFFFFFFFu;
 
-__global__ void k_ht_runs(JoinHT H, const uint64_t* skey, const uint32_t* sval, long long n) {
+__global__ void k_ht_runs(JoinHT H, const uint64_t* skey, const uint32_t* sval, const long long* n_sort) {
+    const long long n = *n_sort;  // 0: the sort gave up, and the slots keep no row (kNoRow)
     for (long long p = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; p < n;
          p += static_cast<long long>(gridDim.x) * blockDim.x) {
         const uint64_t s = skey[p];
-        if (s > static_cast<uint64_t>(H.cap)) continue;  // (a sort that gave up: the call reports it)
         if (p == 0 || skey[p - 1] != s) {
             const bool single = p + 1 == n || skey[p + 1] != s;
             H.slots[s].z = single ? (sval[p] | kRunRow) : static_cast<uint32_t>(p);
@@ -197,7 +197,7 @@ tqp_status ht_build(tqp_ctx* ctx, const tqp_table* build, int32_t key_col, JoinH
     TQP_TRY(radix_sort_pairs(ctx, k0, v0, k1, v1, d_n, n, 0, (bits + 7) / 8 * 8, rs, stream, &in1));
     const uint64_t* sk = in1 ? k1 : k0;
     H->bidx = in1 ? v1 : v0;
-    k_ht_runs<<<iblocks, threads, 0, stream>>>(*H, sk, H->bidx, n);
+    k_ht_runs<<<iblocks, threads, 0, stream>>>(*H, sk, H->bidx, d_n);
     TQP_CUDA(cudaGetLastError());
     return TQP_OK;
 }
@@ -227,8 +227,15 @@ __global__ void k_sj_shift(long long* meta, int dir_bits) {
 }
 
 // sdir[b] = the first sorted index whose key lies in bucket >= b.
-__global__ void k_sj_dir(const long long* meta, const uint64_t* skey, long long n, uint32_t* sdir, long long nb) {
+__global__ void k_sj_dir(const long long* meta, const uint64_t* skey, const long long* n_sort, uint32_t* sdir, long long nb) {
     const int sh = static_cast<int>(__ldg(&meta[2]));
+    const long long n = *n_sort;
+    if (n == 0) {  // the sort gave up: no key has a run
+        for (long long b = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; b <= nb;
+             b += static_cast<long long>(gridDim.x) * blockDim.x)
+            sdir[b] = 0;
+        return;
+    }
     for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i <= n;
          i += static_cast<long long>(gridDim.x) * blockDim.x) {
         const long long b_i = i < n ? static_cast<long long>(skey[i] >> sh) : nb;
@@ -277,7 +284,7 @@ tqp_status ht_build_sorted(tqp_ctx* ctx, const tqp_table* build, int32_t key_col
     H->skeys = in1 ? k1 : k0;
     H->bidx = in1 ? v1 : v0;
     const int dblocks = static_cast<int>(std::min<long long>((n + threads) / threads, ctx->num_sms * 16LL));
-    k_sj_dir<<<dblocks, threads, 0, stream>>>(meta, H->skeys, n, sdir, nb);
+    k_sj_dir<<<dblocks, threads, 0, stream>>>(meta, H->skeys, d_n, sdir, nb);
     TQP_CUDA(cudaGetLastError());
     return TQP_OK;
 }

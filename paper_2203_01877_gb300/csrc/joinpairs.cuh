@@ -218,9 +218,12 @@ static __device__ __noinline__ uint32_t jp_lookup_wide(const PairArgs& A, long l
     return slot_key(s) == key ? s.z : kJpNone;  // (a free slot's value is kJpNone)
 }
 
-// Exclusive prefix of `tile` (see lookback()), 128 predecessors per step.
+// Exclusive prefix of `tile` (see lookback()), 128 predecessors per step. A tile
+// whose wait expired publishes its prefix marked kJpBad, and so do the tiles that
+// build on it; *bad is then set.
+constexpr unsigned long long kJpBad = 3ULL << 62;
 __device__ __forceinline__ unsigned long long jp_lookback(unsigned long long* status, long long tile, unsigned long long agg,
-                                                          int lane, int* err, long long cap) {
+                                                          int lane, int* err, long long cap, bool* bad) {
     if (lane == 0) st_relaxed_u64(&status[tile], (tile == 0 ? kFlagP : kFlagA) | agg);
     if (tile == 0) return 0;
     unsigned long long excl = 0;
@@ -252,13 +255,17 @@ __device__ __forceinline__ unsigned long long jp_lookback(unsigned long long* st
         }
         if (gave_up) break;
         unsigned long long sum = 0;
-        bool found = false;
+        bool found = false, marked = false;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            if (!found) sum += x[k] & kValMask;
-            found |= (x[k] >> 62) == 2;
+            if (!found) {
+                sum += x[k] & kValMask;
+                marked = (x[k] >> 62) == 3;
+            }
+            found |= (x[k] >> 62) >= 2;
         }
         const uint32_t pmask = __ballot_sync(0xffffffffu, found);
+        if (pmask) *bad = __shfl_sync(0xffffffffu, marked, __ffs(pmask) - 1);
         if (pmask && lane > __ffs(pmask) - 1) sum = 0;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
@@ -266,7 +273,8 @@ __device__ __forceinline__ unsigned long long jp_lookback(unsigned long long* st
         if (pmask) break;
     }
     if (gave_up && lane == 0) latch_error(err, TQP_ERR_TIMEOUT);
-    if (lane == 0) st_relaxed_u64(&status[tile], kFlagP | ((excl + agg) & kValMask));
+    *bad |= gave_up;
+    if (lane == 0) st_relaxed_u64(&status[tile], (*bad ? kJpBad : kFlagP) | ((excl + agg) & kValMask));
     return excl;
 }
 
@@ -328,12 +336,13 @@ static __device__ __forceinline__ void join_pairs_tile(const PairArgs& A) {
         }
         if (lane < kJpWarps) wtot[lane] = incl - c;
         const unsigned long long agg = __shfl_sync(0xffffffffu, incl, kWarp - 1);
-        const unsigned long long ex = jp_lookback(A.status, tile, agg, lane, A.err, A.wait_cap);
+        bool bad = false;
+        const unsigned long long ex = jp_lookback(A.status, tile, agg, lane, A.err, A.wait_cap, &bad);
         if (lane == 0) {
             excl_sm = ex;
             if (tile == A.ntiles - 1) {
-                *A.d_count = static_cast<int64_t>(ex + agg);
-                if (static_cast<long long>(ex + agg) > A.capacity) latch_error(A.err, TQP_ERR_CAPACITY);
+                *A.d_count = bad ? -1 : static_cast<int64_t>(ex + agg);
+                if (!bad && static_cast<long long>(ex + agg) > A.capacity) latch_error(A.err, TQP_ERR_CAPACITY);
             }
         }
     }

@@ -143,20 +143,21 @@ __global__ void __launch_bounds__(kSortThreads, kSortBlocksPerSm) k_rs_sort(uint
                                                                             uint32_t* v1, long long* n_ptr, int begin_bit,
                                                                             int end_bit, unsigned long long* digit_tot,
                                                                             uint32_t* hist, long long ntiles,
-                                                                            unsigned int* bar, int* err) {
+                                                                            unsigned int* bar, int* err, long long wait_cap) {
     __shared__ uint32_t wcnt[kSortWarps][256];
     __shared__ unsigned long long wsum[kSortWarps];
     const long long n = *n_ptr;
     if (n == 0) return;
     unsigned int arrivals = 0;
-    for (int shift = begin_bit; shift < end_bit; shift += 8) {
+    bool ok = true;
+    for (int shift = begin_bit; ok && shift < end_bit; shift += 8) {
         rs_upsweep(k0, n, shift, hist, ntiles, digit_tot, wcnt[0]);
-        if (!grid_barrier(bar, arrivals += gridDim.x, err)) break;
+        if (!(ok = grid_barrier(bar, arrivals += gridDim.x, err, wait_cap))) break;
         rs_scan(hist, ntiles, digit_tot, wsum);
-        if (!grid_barrier(bar, arrivals += gridDim.x, err)) break;
+        if (!(ok = grid_barrier(bar, arrivals += gridDim.x, err, wait_cap))) break;
         if (blockIdx.x == 0) digit_tot[threadIdx.x] = 0;  // (read by the scans only; the next barrier orders it)
         rs_downsweep(k0, v0, k1, v1, n, shift, hist, ntiles, wcnt);
-        if (!grid_barrier(bar, arrivals += gridDim.x, err)) break;
+        ok = grid_barrier(bar, arrivals += gridDim.x, err, wait_cap);
         uint64_t* k = k0;
         k0 = k1;
         k1 = k;
@@ -164,8 +165,8 @@ __global__ void __launch_bounds__(kSortThreads, kSortBlocksPerSm) k_rs_sort(uint
         v0 = v1;
         v1 = v;
     }
-    // (a sort that gave up leaves no items: what follows reads the count again)
-    if (threadIdx.x == 0 && read_error(err) == TQP_ERR_TIMEOUT) *n_ptr = 0;
+    // a sort that gave up leaves no items: what follows takes its number from here
+    if (!ok && threadIdx.x == 0) *n_ptr = 0;
 }
 
 // Scratch needed by radix_sort_pairs for up to n_max items.
@@ -176,7 +177,8 @@ size_t radix_sort_scratch(long long n_max) {
 
 // Sort bits [begin_bit, end_bit) of the keys.  Buffers (k0, v0) hold the
 // input; (k1, v1) are a second buffer of the same size.  *result_in_1 tells
-// which buffer holds the sorted output.
+// which buffer holds the sorted output.  *d_n is 0 afterwards when a wait of the
+// sort expired, so kernels that read the output take the count from there.
 tqp_status radix_sort_pairs(const tqp_ctx* ctx, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, long long* d_n,
                             long long n_max, int begin_bit, int end_bit, void* scratch, cudaStream_t stream,
                             bool* result_in_1) {
@@ -191,7 +193,8 @@ tqp_status radix_sort_pairs(const tqp_ctx* ctx, uint64_t* k0, uint32_t* v0, uint
                               kSortBlocksPerSm) * ctx->num_sms;
     const int grid = static_cast<int>(std::min<long long>(most, std::max<long long>(ntiles, 32)));
     int* err = ctx->d_err;
-    void* args[] = {&k0, &v0, &k1, &v1, &d_n, &begin_bit, &end_bit, &digit_tot, &hist, &ntiles, &bar, &err};
+    long long cap = ctx->wait_cap;
+    void* args[] = {&k0, &v0, &k1, &v1, &d_n, &begin_bit, &end_bit, &digit_tot, &hist, &ntiles, &bar, &err, &cap};
     TQP_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_rs_sort), dim3(grid), dim3(kSortThreads), args, 0,
                                          stream));
     *result_in_1 = ((end_bit - begin_bit + 7) / 8) % 2 != 0;
