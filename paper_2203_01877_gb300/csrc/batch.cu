@@ -411,6 +411,9 @@ struct tqp_batch {
     tqp_ctx* ctx = nullptr;
     bool persistent = false;  // scratch from the arena's long-lived top region
     int tile = tqp::kBatchTile;  // rows per tile of the scans (clamped per job to what fits)
+    // Short of scratch: no padded key entries, and the staged scans, whose maps
+    // are the smaller ones, in place of the flat row launches.
+    bool lean = false;
     size_t top_before = 0;
     size_t top_after = 0;
     // lowered jobs
@@ -564,7 +567,7 @@ static tqp_status add_filter_job(tqp_batch* b, const tqp_plan* p, const tqp_resu
         return TQP_OK;
     }
     FiltJob D;
-    if (lower_filter_direct(p->fact, A, &D.A)) {
+    if (!b->lean && lower_filter_direct(p->fact, A, &D.A)) {
         D.A.mask = A.mask;
         D.A.block_tot = A.block_tot;
         D.A.acc = A.acc;
@@ -814,7 +817,8 @@ static tqp_status add_join_job(tqp_batch* b, const tqp_plan* p, const tqp_result
     // aggregation by join key first (used on the device only if the table is
     // direct-mapped), as in the single-plan path
     if (grouped && A.pjfast && A.fast && A.H.meta && A.G.ntiles > 0 && F->num_rows >= 2 * std::max<long long>(1, ndr)) {
-        A.nk = keyfirst_words(A.S.nacc + (A.has_sum ? 1 : 0));
+        A.nk = A.S.nacc + (A.has_sum ? 1 : 0);
+        if (!b->lean) A.nk = keyfirst_words(A.nk);
         const size_t kbytes = static_cast<size_t>(A.H.cap) * A.nk * 8;
         A.kacc = static_cast<unsigned long long*>(balloc(b, kbytes));
         if (!A.kacc) return arena_oom(ctx, kbytes);
@@ -839,7 +843,7 @@ static tqp_status add_join_job(tqp_batch* b, const tqp_plan* p, const tqp_result
         b->fold.push_back(Fo);
     }
     ProbeJob P;
-    if (A.G.ntiles > 0 && lower_probe_agg(A, F, &P.A)) {
+    if (!b->lean && A.G.ntiles > 0 && lower_probe_agg(A, F, &P.A)) {
         b->probe[probe_agg_tab(P.A, A.S.cap, ndr) ? 1 : 0].push_back(P);
     } else if (A.G.ntiles > 0) {
         b->scan[kJobJoin - 1].push_back(J);
@@ -1032,7 +1036,7 @@ static tqp_status add_shared_jobs(tqp_batch* b, const std::vector<SharedCand>& c
 static tqp_status lower_batch(tqp_batch* b, const tqp_plan* plans, const tqp_result* res, int32_t n) {
     // per plan at most 6 counters (group table, key ranges, top-k, filter, a
     // count, spare), the tickets and the radix select's barrier
-    b->slab_bytes = static_cast<size_t>(kCounterBytes) * (6 * static_cast<size_t>(n) + kKinds + 2);
+    b->slab_bytes = static_cast<size_t>(kCounterBytes) * (6 * static_cast<size_t>(n) + kKinds + 1);
     b->slab = static_cast<unsigned char*>(balloc(b, b->slab_bytes));
     if (!b->slab) return arena_oom(b->ctx, b->slab_bytes);
     add_fill(b, b->slab, b->slab_bytes, kZero16);
@@ -1144,7 +1148,7 @@ static long long assign_blocks(const tqp_batch* b, std::vector<Job>& jobs, long 
     long long rows = 0;
     for (const Job& j : jobs) rows += j.A.n;
     const long long want = rows / (per_sm * b->ctx->num_sms);
-    const long long per = std::min(kFlatRowsMax, std::max(kFlatRowsMin, want / 1024 * 1024));
+    const long long per = b->lean ? kFlatRowsMax : std::min(kFlatRowsMax, std::max(kFlatRowsMin, want / 1024 * 1024));
     long long first = 0;
     for (Job& j : jobs) {
         j.first_block = first;
@@ -1418,17 +1422,26 @@ static tqp_status batch_create(tqp_ctx* ctx, const tqp_plan* plans, const tqp_re
     return TQP_OK;
 }
 
-tqp_status run_plans_on(tqp_ctx* ctx, const tqp_plan* plans, const tqp_result* res, int32_t n, cudaStream_t st) {
+static tqp_status run_plans_once(tqp_ctx* ctx, const tqp_plan* plans, const tqp_result* res, int32_t n, bool lean,
+                                 cudaStream_t st) {
     arena_reset(ctx);
     tqp_batch b;
     b.ctx = ctx;
     b.persistent = false;
+    b.lean = lean;
     TQP_TRY(batch_prepare(ctx, plans, res, n, &b, st));
     TQP_TRY(batch_launch(&b, st));
     if (b.fb_plans.empty()) return TQP_OK;
     const size_t lo = (ctx->used + 255) / 256 * 256;
     if (lo >= ctx->top) return arena_oom(ctx, lo + kPersistentBytes);
     return run_fallbacks(&b, st, ctx->arena + lo, ctx->top - lo, nullptr);
+}
+
+tqp_status run_plans_on(tqp_ctx* ctx, const tqp_plan* plans, const tqp_result* res, int32_t n, cudaStream_t st) {
+    const tqp_status s = run_plans_once(ctx, plans, res, n, false, st);
+    if (s != TQP_ERR_OUT_OF_MEMORY) return s;
+    clear_error();
+    return run_plans_once(ctx, plans, res, n, true, st);
 }
 
 static void release(tqp_batch* b) {
@@ -1491,19 +1504,25 @@ tqp_status tqp_batch_create(tqp_ctx* ctx, const tqp_plan* plans, const tqp_resul
     if (!g.ok) return fail(TQP_ERR_CUDA, "cannot select device %d", ctx->device);
     int tile = kBatchTile;
     if (ctx->tuner && ctx->tuner->enabled) TQP_TRY(tune_batch_tile(ctx, plans, res, n, &tile));
-    tqp_batch* b = new (std::nothrow) tqp_batch();
-    if (!b) return fail(TQP_ERR_OUT_OF_MEMORY, "host allocation failed");
-    b->tile = tile;
-    top_open(ctx);
-    const tqp_status s = batch_create(ctx, plans, res, n, b);
-    b->top_after = ctx->top;
-    if (s != TQP_OK) {
+    tqp_status s = TQP_OK;
+    for (const bool lean : {false, true}) {
+        tqp_batch* b = new (std::nothrow) tqp_batch();
+        if (!b) return fail(TQP_ERR_OUT_OF_MEMORY, "host allocation failed");
+        b->tile = tile;
+        b->lean = lean;
+        top_open(ctx);
+        s = batch_create(ctx, plans, res, n, b);
+        b->top_after = ctx->top;
+        if (s == TQP_OK) {
+            clear_error();
+            *out = b;
+            return TQP_OK;
+        }
         release(b);
         delete b;
-        return s;
+        if (s != TQP_ERR_OUT_OF_MEMORY) break;
     }
-    *out = b;
-    return TQP_OK;
+    return s;
 }
 
 tqp_status tqp_batch_run(tqp_batch* b, void* stream) {

@@ -49,6 +49,11 @@ void* arena_alloc(tqp_ctx* ctx, size_t bytes, size_t align) {
     return ctx->arena + off;
 }
 
+size_t arena_after(size_t off, std::initializer_list<size_t> sizes) {
+    for (const size_t s : sizes) off = (off + 255) / 256 * 256 + s;
+    return off;
+}
+
 void* arena_alloc_top(tqp_ctx* ctx, size_t bytes, size_t align) {
     if (bytes > ctx->top) return nullptr;
     const size_t start = (ctx->top - bytes) / align * align;

@@ -173,6 +173,8 @@ tqp_status group_table_init(GroupSpec* S, void* mem, long long cap, long long ma
 struct GroupRangePlan;
 tqp_status group_finalize(tqp_ctx* ctx, const GroupSpec& S, const GroupOut& O, cudaStream_t stream,
                           const GroupRangePlan* ranged = nullptr);
+// The arena's end after group_finalize (k = 0) or group_topk (k > 0) of S from offset `off` on.
+size_t group_output_end(const GroupSpec& S, int k, size_t off);
 // Top-k groups by accumulator of aggregate `agg` (descending; ties: key
 // ascending); writes min(k, G) rows in rank order and *total_groups = G.
 tqp_status group_topk(tqp_ctx* ctx, const GroupSpec& S, const GroupOut& O, int k, int agg,

@@ -255,6 +255,17 @@ tqp_status group_table_init(GroupSpec* S, void* mem, long long cap, long long ma
     return TQP_OK;
 }
 
+size_t group_output_end(const GroupSpec& S, int k, size_t off) {
+    const long long nmax = S.cap + 1;
+    if (k > 0) {
+        const size_t ncand = static_cast<size_t>((nmax + kTopBlock - 1) / kTopBlock) * k;
+        return arena_after(off, {256, sizeof(TopSel), kSelCand * 8, kSelCand * 8, kSelCand * 4, ncand * 8, ncand * 8,
+                                 ncand * 4, ncand * 8, ncand * 8, ncand * 4});
+    }
+    if (S.cap <= kSmallCap) return off;
+    return arena_after(off, {2 * (static_cast<size_t>(nmax) * 12 + 512) + 256, radix_sort_scratch(nmax)});
+}
+
 // Finalize a filled table into the caller's output arrays.
 tqp_status group_finalize(tqp_ctx* ctx, const GroupSpec& S, const GroupOut& O, cudaStream_t stream,
                           const GroupRangePlan* rp) {
@@ -611,14 +622,11 @@ tqp_status launch_groupby(tqp_ctx* ctx, const tqp_table* t, const tqp_pred* pred
     GroupRangePlan* rp = nullptr;
     uint32_t* counts = nullptr;
     if (!direct && topk == 0 && !user_shape(ctx) && lower_group_range(t, A, &R)) {
-        const size_t used = ctx->used;
-        rp = static_cast<GroupRangePlan*>(arena_alloc(ctx, sizeof(GroupRangePlan)));
-        const long long blocks = (std::min<long long>(cap + 1, kGrMaxEntries) + kGrEmitPer - 1) / kGrEmitPer;
-        counts = static_cast<uint32_t*>(arena_alloc(ctx, static_cast<size_t>(blocks) * 4));
-        if (!rp || !counts) {
-            rp = nullptr;
-            ctx->used = used;
-        }
+        // no scratch of its own: the plan lies beside the scan's ticket, the blocks' counts in the
+        // hash table's keys (unused when the plan is on; one word per kGrEmitPer entries)
+        static_assert(sizeof(GroupRangePlan) <= 192, "beside the ticket");
+        rp = reinterpret_cast<GroupRangePlan*>(ticket + 8);
+        counts = static_cast<uint32_t*>(tab);
     }
     TQP_TRY(group_table_init(&A.S, tab, cap, max_groups, stream, !direct && !rp));
     if (rp) TQP_TRY(launch_group_range(ctx, A.S, O, R, rp, counts, stream));
@@ -647,14 +655,11 @@ tqp_status launch_groupby(tqp_ctx* ctx, const tqp_table* t, const tqp_pred* pred
         const size_t part_bytes = 2 * kDirKeys * 8;
         int nparts = static_cast<int>(
             std::max<long long>(1, std::min<long long>((t->num_rows + 8191) / 8192, 4LL * ctx->num_sms)));
-        const size_t used = ctx->used;
+        // one per SM where scratch is short (the flag and a top-k's follow)
+        const size_t end = arena_after(ctx->used, {static_cast<size_t>(nparts) * part_bytes, 16});
+        if ((topk > 0 ? group_output_end(A.S, topk, end) : end) > ctx->top) nparts = std::min(nparts, ctx->num_sms);
         unsigned long long* kpart =
             static_cast<unsigned long long*>(arena_alloc(ctx, static_cast<size_t>(nparts) * part_bytes));
-        if (!kpart && nparts > ctx->num_sms) {
-            ctx->used = used;
-            nparts = ctx->num_sms;
-            kpart = static_cast<unsigned long long*>(arena_alloc(ctx, static_cast<size_t>(nparts) * part_bytes));
-        }
         unsigned int* done = static_cast<unsigned int*>(arena_alloc(ctx, 16));
         if (!kpart || !done) return arena_oom(ctx, static_cast<size_t>(nparts) * part_bytes + 16);
         D.done = done;

@@ -9,6 +9,7 @@
 #include <cstddef>
 #include <cstdint>
 #include <cstring>
+#include <initializer_list>
 #include <map>
 #include <mutex>
 #include <string>
@@ -90,6 +91,8 @@ void clear_error();
 void arena_reset(tqp_ctx* ctx);
 // Returns nullptr (and records the shortfall) when the arena is exhausted.
 void* arena_alloc(tqp_ctx* ctx, size_t bytes, size_t align = 256);
+// Offset of the arena's end after allocations of `sizes` from offset `off` on (256-byte aligned, as arena_alloc).
+size_t arena_after(size_t off, std::initializer_list<size_t> sizes);
 // Long-lived allocation from the arena's end (survives arena_reset; freed by
 // moving ctx->top back, newest first).
 void* arena_alloc_top(tqp_ctx* ctx, size_t bytes, size_t align = 256);

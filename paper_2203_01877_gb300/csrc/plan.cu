@@ -488,6 +488,9 @@ static tqp_status run_join_plan(tqp_ctx* ctx, const tqp_plan* p, const tqp_resul
     // Used only if the table turns out direct-mapped; off when scratch is short.
     if (!parted && grouped && A.pjfast && A.fast && H.meta && F->num_rows >= 2 * std::max<long long>(1, D->num_rows)) {
         A.nk = keyfirst_words(A.S.nacc + (A.has_sum ? 1 : 0));
+        // without the padding where scratch is short of it (the groups' output follows)
+        const size_t end = arena_after(ctx->used, {static_cast<size_t>(H.cap) * A.nk * 8});
+        if (group_output_end(A.S, p->topk, end) > ctx->top) A.nk = A.S.nacc + (A.has_sum ? 1 : 0);
         const size_t used = ctx->used;
         A.kacc = static_cast<unsigned long long*>(arena_alloc(ctx, static_cast<size_t>(H.cap) * A.nk * 8));
         if (!A.kacc) ctx->used = used;
