@@ -58,8 +58,8 @@ bool lower_group_direct(const tqp_table* t, const GroupArgs& A, long long max_gr
 
 constexpr int kBatchTile = 1024;
 constexpr int kBatchStages = 3;
-constexpr int kJobFilter = 1, kJobGroup = 2, kJobJoin = 3, kJobMulti = 4;
-constexpr int kKinds = 4;  // scan bodies: filter, group-by, joined aggregation, shared filter
+constexpr int kJobFilter = 1, kJobGroup = 2, kJobJoin = 3, kJobMulti = 4, kJobFew = 5;
+constexpr int kKinds = 5;  // scan bodies: filter, group-by, joined aggregation, shared filter of many and of few queries
 constexpr int kFlatThreads = 256;
 constexpr int kFillPer = 4096;  // 16-byte units per fill block
 constexpr int kRowsPer = 2048;  // elements per block of the element-wise phases
@@ -263,7 +263,7 @@ template <> struct BodyArgs<GroupBody> {
 template <> struct BodyArgs<PlanJoinBody> {
     static __device__ __forceinline__ const PlanJoinArgs& of(const ScanJob& j) { return j.u.j; }
 };
-template <> struct BodyArgs<MultiBody> {
+template <bool kFew> struct BodyArgs<MultiBody<kFew>> {
     static __device__ __forceinline__ const MultiArgs& of(const ScanJob& j) { return j.u.m; }
 };
 
@@ -275,12 +275,13 @@ constexpr int body_bytes() { return (Body::kSmemBytes + 127) / 128 * 128; }
 // tables of every job of that kind.
 template <class Body>
 __global__ void __launch_bounds__(kEngineThreads, Body::kMinBlocks) k_b_scan(const ScanJob* J, const int32_t* cjob,
-                                                              unsigned long long* ticket, long long total_chunks) {
+                                                              unsigned long long* ticket, long long total_chunks,
+                                                              int body_size) {
     extern __shared__ __align__(128) unsigned char smem[];
     EngineHeader* h = reinterpret_cast<EngineHeader*>(smem);
     ScanJob* sj = reinterpret_cast<ScanJob*>(smem + kHeaderBytes);
     unsigned char* body_smem = smem + kHeaderBytes + kJobBytes;
-    unsigned char* stages = body_smem + body_bytes<Body>();
+    unsigned char* stages = body_smem + body_size;
     __shared__ int job_sm;
     const int warp = threadIdx.x / kWarp;
     const int lane = threadIdx.x % kWarp;
@@ -434,16 +435,16 @@ struct tqp_batch {
     long long fill_blocks = 0, row_blocks = 0, num_blocks = 0, slot_blocks = 0, compact_blocks = 0, top0_blocks = 0,
               sel_blocks = 0, grange_blocks = 0, gdirect_blocks = 0, fold_blocks = 0, filt_blocks = 0;
     long long probe_blocks[2] = {0, 0};
-    long long scan_chunks[kKinds] = {0, 0, 0, 0};
+    long long scan_chunks[kKinds] = {};
     // lookup tables and outputs of the shared scans (one blob; per job its offset)
     std::vector<unsigned char> mblob;
-    std::vector<size_t> mblob_off;
+    std::vector<size_t> mblob_off[2];  // [1]: of few queries
     unsigned char* d_mblob = nullptr;
     std::vector<long long> level_blocks;
     size_t off_fill = 0, off_row = 0, off_num = 0, off_slot = 0, off_compact = 0, off_top0 = 0, off_sel = 0,
            off_grange = 0, off_gdirect = 0, off_fold = 0, off_filt = 0;
     size_t off_probe[2] = {0, 0};
-    size_t off_scan[kKinds] = {0, 0, 0, 0};
+    size_t off_scan[kKinds] = {};
     std::vector<size_t> off_level;
     unsigned long long* selbar = nullptr;  // arrivals at the radix select's grid barriers
     // small zeroed counters share one slab (one fill range)
@@ -453,7 +454,7 @@ struct tqp_batch {
     FillRange* d_fill = nullptr;
     int64_t** d_zero = nullptr;
     BuildJob* d_build = nullptr;
-    ScanJob* d_scan[kKinds] = {nullptr, nullptr, nullptr, nullptr};
+    ScanJob* d_scan[kKinds] = {};
     CompactJob* d_compact = nullptr;
     FinJob* d_fin = nullptr;
     TopJob* d_top = nullptr;
@@ -463,9 +464,10 @@ struct tqp_batch {
     FiltJob* d_filt = nullptr;
     std::vector<TopItem*> d_levels;
     int32_t* d_maps = nullptr;
-    unsigned long long* d_ticket[kKinds] = {nullptr, nullptr, nullptr, nullptr};
-    size_t scan_smem[kKinds] = {0, 0, 0, 0};
-    int scan_grid[kKinds] = {0, 0, 0, 0};
+    unsigned long long* d_ticket[kKinds] = {};
+    size_t scan_smem[kKinds] = {};
+    int scan_grid[kKinds] = {};
+    int scan_body[kKinds] = {};  // the bodies' shared memory: the most any job of the kind needs
     // plans run through the single-plan path, and their scratch
     std::vector<tqp_plan> fb_plans;
     std::vector<tqp_result> fb_res;
@@ -626,7 +628,7 @@ static tqp_status add_group_job(tqp_batch* b, const tqp_plan* p, const tqp_resul
     int ncond = 0;
     TQP_TRY(lower_preds(t, p->preds, p->npreds, A.cond, &ncond));
     A.ncond = ncond;
-    int32_t types[TQP_MAX_GROUP_COLS] = {0, 0, 0, 0};
+    int32_t types[TQP_MAX_GROUP_COLS] = {};
     for (int i = 0; i < p->ngc; ++i) types[i] = t->cols[p->group_cols[i]].type;
     TQP_TRY(lower_group(p->group_cols, types, p->ngc, p->aggs, p->naggs, t->num_cols, &A.S));
     std::vector<int> staged;
@@ -952,8 +954,8 @@ static tqp_status add_multi_job(tqp_batch* b, const tqp_table* t, const std::vec
     cols.erase(std::unique(cols.begin(), cols.end()), cols.end());
     int stage_row = 0;
     for (int c : cols) stage_row += t->cols[c].type == TQP_I64 ? 8 : (t->cols[c].type == TQP_I32 ? 4 : 1);
-    const long long room =
-        static_cast<long long>(ctx->smem_optin) - 1024 - kHeaderBytes - kJobBytes - body_bytes<MultiBody>();
+    const long long room = static_cast<long long>(ctx->smem_optin) - 1024 - kHeaderBytes - kJobBytes -
+                           body_bytes<MultiBody<false>>();
     int T = b->tile;
     while (T > kBatchTile &&
            static_cast<long long>(kBatchStages) * (static_cast<long long>(T) * stage_row + 128LL * kMaxStaged) > room)
@@ -961,12 +963,13 @@ static tqp_status add_multi_job(tqp_batch* b, const tqp_table* t, const std::vec
     const tqp_tuning tu{T, kBatchStages, 2, 1};
     ScanJob J;
     memset(&J, 0, sizeof(J));
-    J.kind = kJobMulti;
     MultiArgs& A = J.u.m;
     std::vector<unsigned char> blob;
     size_t smem = 0;
     int per_sm = 0;
-    TQP_TRY(mq_lower_group(ctx, t, qs, members, &tu, kJobBytes, true, &A, &blob, &smem, &per_sm));
+    TQP_TRY(mq_lower_group(ctx, t, qs, members, &tu, kJobBytes, &A, &blob, &smem, &per_sm));
+    const bool few = mq_few(members.size(), A.nexpr);
+    J.kind = few ? kJobFew : kJobMulti;
     if (A.G.ntiles == 0) {  // an empty table: every output is zero
         for (int m : members) {
             const MqOut& o = qs[m].out;
@@ -984,8 +987,8 @@ static tqp_status add_multi_job(tqp_batch* b, const tqp_table* t, const std::vec
     const size_t off = (b->mblob.size() + 15) / 16 * 16;
     b->mblob.resize(off + blob.size());
     memcpy(b->mblob.data() + off, blob.data(), blob.size());
-    b->mblob_off.push_back(off);
-    b->scan[kJobMulti - 1].push_back(J);
+    b->mblob_off[few].push_back(off);
+    b->scan[J.kind - 1].push_back(J);
     return TQP_OK;
 }
 
@@ -1034,14 +1037,14 @@ static tqp_status add_shared_jobs(tqp_batch* b, const std::vector<SharedCand>& c
 }
 
 static tqp_status lower_batch(tqp_batch* b, const tqp_plan* plans, const tqp_result* res, int32_t n) {
-    // per plan at most 6 counters (group table, key ranges, top-k, filter, a
-    // count, spare), the tickets and the radix select's barrier
-    b->slab_bytes = static_cast<size_t>(kCounterBytes) * (6 * static_cast<size_t>(n) + kKinds + 1);
+    // the tickets, and per plan at most 6 counters (group table, key ranges,
+    // top-k, filter, a count, a spare one: the radix select's barrier)
+    static_assert(kKinds == 5, "a ticket each");
+    b->slab_bytes = static_cast<size_t>(kCounterBytes) * (6 * static_cast<size_t>(n) + 5);
     b->slab = static_cast<unsigned char*>(balloc(b, b->slab_bytes));
     if (!b->slab) return arena_oom(b->ctx, b->slab_bytes);
     add_fill(b, b->slab, b->slab_bytes, kZero16);
     for (int k = 0; k < kKinds; ++k) b->d_ticket[k] = counter(b);
-    b->selbar = counter(b);
     std::vector<SharedCand> shared;
     for (int32_t i = 0; i < n; ++i) {
         const tqp_plan* p = &plans[i];
@@ -1070,7 +1073,9 @@ static tqp_status lower_batch(tqp_batch* b, const tqp_plan* plans, const tqp_res
             else shared.push_back(SharedCand{p, r, sum, cnt, cnt2});
         }
     }
-    return add_shared_jobs(b, shared);
+    TQP_TRY(add_shared_jobs(b, shared));
+    if (!b->top.empty()) b->selbar = counter(b);  // (a plan's spare)
+    return TQP_OK;
 }
 
 static const ScanGeom& job_geom(const ScanJob& j) {
@@ -1274,16 +1279,19 @@ static tqp_status batch_launch(tqp_batch* b, cudaStream_t st) {
         k_b_filter_direct<<<static_cast<unsigned>(b->filt_blocks), kFdThreads, 0, st>>>(b->d_filt, M + b->off_filt);
     if (b->scan_chunks[0])
         k_b_scan<FilterBody><<<b->scan_grid[0], kEngineThreads, b->scan_smem[0], st>>>(
-            b->d_scan[0], M + b->off_scan[0], b->d_ticket[0], b->scan_chunks[0]);
+            b->d_scan[0], M + b->off_scan[0], b->d_ticket[0], b->scan_chunks[0], b->scan_body[0]);
     if (b->scan_chunks[1])
         k_b_scan<GroupBody><<<b->scan_grid[1], kEngineThreads, b->scan_smem[1], st>>>(
-            b->d_scan[1], M + b->off_scan[1], b->d_ticket[1], b->scan_chunks[1]);
+            b->d_scan[1], M + b->off_scan[1], b->d_ticket[1], b->scan_chunks[1], b->scan_body[1]);
     if (b->scan_chunks[2])
         k_b_scan<PlanJoinBody><<<b->scan_grid[2], kEngineThreads, b->scan_smem[2], st>>>(
-            b->d_scan[2], M + b->off_scan[2], b->d_ticket[2], b->scan_chunks[2]);
+            b->d_scan[2], M + b->off_scan[2], b->d_ticket[2], b->scan_chunks[2], b->scan_body[2]);
     if (b->scan_chunks[3])
-        k_b_scan<MultiBody><<<b->scan_grid[3], kEngineThreads, b->scan_smem[3], st>>>(
-            b->d_scan[3], M + b->off_scan[3], b->d_ticket[3], b->scan_chunks[3]);
+        k_b_scan<MultiBody<false>><<<b->scan_grid[3], kEngineThreads, b->scan_smem[3], st>>>(
+            b->d_scan[3], M + b->off_scan[3], b->d_ticket[3], b->scan_chunks[3], b->scan_body[3]);
+    if (b->scan_chunks[4])
+        k_b_scan<MultiBody<true>><<<b->scan_grid[4], kEngineThreads, b->scan_smem[4], st>>>(
+            b->d_scan[4], M + b->off_scan[4], b->d_ticket[4], b->scan_chunks[4], b->scan_body[4]);
     if (b->fold_blocks)
         k_b_fold<<<static_cast<unsigned>(b->fold_blocks), kFoldThreads, 0, st>>>(b->d_fold, M + b->off_fold);
     if (b->compact_blocks)
@@ -1331,7 +1339,13 @@ static tqp_status scan_shape(tqp_batch* b, int k) {
     TQP_TRY(allow_smem(ctx, reinterpret_cast<const void*>(k_b_scan<Body>), attr));
     int max_stage = 128;
     for (auto& j : b->scan[k]) max_stage = std::max(max_stage, job_stage_bytes(j));
-    b->scan_smem[k] = kHeaderBytes + kJobBytes + body_bytes<Body>() + static_cast<size_t>(kBatchStages) * max_stage;
+    int body = body_bytes<Body>();
+    if (k >= kJobMulti - 1) {  // shared scans: what their tables need
+        body = 0;
+        for (auto& j : b->scan[k]) body = std::max(body, (j.u.m.body_bytes + 127) / 128 * 128);
+    }
+    b->scan_body[k] = body;
+    b->scan_smem[k] = kHeaderBytes + kJobBytes + body + static_cast<size_t>(kBatchStages) * max_stage;
     if (b->scan_smem[k] + 1024 > static_cast<size_t>(ctx->smem_optin))
         return fail(TQP_ERR_UNSUPPORTED, "batched scan needs %zu bytes of shared memory", b->scan_smem[k]);
     int occ = 0;
@@ -1352,15 +1366,17 @@ static tqp_status batch_prepare(tqp_ctx* ctx, const tqp_plan* plans, const tqp_r
     TQP_TRY(scan_shape<FilterBody>(b, 0));
     TQP_TRY(scan_shape<GroupBody>(b, 1));
     TQP_TRY(scan_shape<PlanJoinBody>(b, 2));
-    TQP_TRY(scan_shape<MultiBody>(b, 3));
+    TQP_TRY(scan_shape<MultiBody<false>>(b, 3));
+    TQP_TRY(scan_shape<MultiBody<true>>(b, 4));
     plan_top_levels(b);
     build_maps(b);
     TQP_TRY(upload(b, b->fill, &b->d_fill, st));
     TQP_TRY(upload(b, b->zero, &b->d_zero, st));
     TQP_TRY(upload(b, b->build, &b->d_build, st));
     TQP_TRY(upload(b, b->mblob, &b->d_mblob, st));
-    for (size_t i = 0; i < b->scan[kJobMulti - 1].size(); ++i)
-        mq_bind(&b->scan[kJobMulti - 1][i].u.m, b->d_mblob + b->mblob_off[i]);
+    for (const int kind : {kJobMulti, kJobFew})
+        for (size_t i = 0; i < b->scan[kind - 1].size(); ++i)
+            mq_bind(&b->scan[kind - 1][i].u.m, b->d_mblob + b->mblob_off[kind == kJobFew][i]);
     for (int k = 0; k < kKinds; ++k) TQP_TRY(upload(b, b->scan[k], &b->d_scan[k], st));
     TQP_TRY(upload(b, b->compact, &b->d_compact, st));
     TQP_TRY(upload(b, b->fin, &b->d_fin, st));

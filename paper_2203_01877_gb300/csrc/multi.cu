@@ -391,15 +391,17 @@ void mq_pack(const tqp_table* t, const std::vector<MqQuery>& qs, std::vector<std
 }
 
 tqp_status mq_lower_group(const tqp_ctx* ctx, const tqp_table* t, const std::vector<MqQuery>& qs,
-                          const std::vector<int>& members, const tqp_tuning* tu_in, int extra_smem, bool fixed_body,
+                          const std::vector<int>& members, const tqp_tuning* tu_in, int extra_smem,
                           MultiArgs* A, std::vector<unsigned char>* blob, size_t* smem, int* ctas_per_sm) {
     memset(A, 0, sizeof(*A));
     std::vector<uint32_t> words;
     std::vector<int64_t> breaks;
     if (!mq_tables(t, qs, members, A, &words, &breaks))
         return fail(TQP_ERR_UNSUPPORTED, "shared scan: lookup tables exceed the shared-memory budget");
-    A->body_bytes = fixed_body ? MultiBody::kSmemBytes
-                               : mq_body_bytes(static_cast<int>(words.size()), static_cast<int>(breaks.size()));
+    const std::vector<DExpr> ex = mq_exprs(qs, members);
+    const bool few = mq_few(members.size(), ex.size());
+    A->body_bytes = mq_body_bytes(few, static_cast<int>(ex.size()), static_cast<int>(words.size()),
+                                  static_cast<int>(breaks.size()));
     const int body_smem = extra_smem + A->body_bytes;
     const std::vector<int> staged = mq_staged(qs, members, *A);
     if (staged.size() > static_cast<size_t>(kMaxStaged))
@@ -407,11 +409,24 @@ tqp_status mq_lower_group(const tqp_ctx* ctx, const tqp_table* t, const std::vec
     TQP_TRY(check_device_cols(t, staged, "tqp_filter_shared"));
     int bpr = 0;
     for (int c : staged) bpr += t->cols[c].type == TQP_I64 ? 8 : (t->cols[c].type == TQP_I32 ? 4 : 1);
-    const tqp_tuning tu = tu_in ? *tu_in : default_tuning(ctx, bpr, body_smem);
-    TQP_TRY(make_geom(ctx, t, staged, tu, body_smem, &A->G, smem));
+    tqp_tuning tu = tu_in ? *tu_in : default_tuning(ctx, bpr, body_smem);
+    // A shape set by the caller or the tuner is refused where it does not fit
+    // beside the tables and kMqShapeBytes; one that only the row queues push
+    // over is narrowed (results do not depend on it).
+    tqp_status gs = make_geom(ctx, t, staged, tu, body_smem, &A->G, smem);
+    const long long shape = static_cast<long long>(*smem) - mq_queue_bytes(few, static_cast<int>(ex.size())) + kMqShapeBytes;
+    if (shape > ctx->smem_optin)
+        gs = fail(TQP_ERR_UNSUPPORTED, "scan needs %lld bytes of shared memory (device allows %d)", shape, ctx->smem_optin);
+    else
+        while (gs == TQP_ERR_UNSUPPORTED && (tu.stages > 2 || tu.tile_rows > kRowQuantum)) {
+            if (tu.stages > 2) --tu.stages;
+            else tu.tile_rows -= kRowQuantum;
+            clear_error();
+            gs = make_geom(ctx, t, staged, tu, body_smem, &A->G, smem);
+        }
+    TQP_TRY(gs);
     *ctas_per_sm = tu.ctas_per_sm;
     for (int k = 0; k < A->ncols; ++k) A->c[k].soff = A->G.col[A->c[k].col].soff;
-    const std::vector<DExpr> ex = mq_exprs(qs, members);
     A->nexpr = static_cast<int32_t>(ex.size());
     for (size_t e = 0; e < ex.size(); ++e) {
         if (!lower_prod(ex[e], A->G, &A->e[e]))
@@ -453,11 +468,12 @@ void mq_bind(MultiArgs* A, const unsigned char* d_blob) {
     A->out = reinterpret_cast<const MqOut*>(d_blob + reinterpret_cast<uintptr_t>(A->out));
 }
 
-__global__ void __launch_bounds__(kEngineThreads, MultiBody::kMinBlocks)
+template <bool kFew>
+__global__ void __launch_bounds__(kEngineThreads, MultiBody<kFew>::kMinBlocks)
     k_filter_multi(const __grid_constant__ MultiLaunch P) {
     extern __shared__ __align__(128) unsigned char smem[];
     const MultiArgs& A = stage_args(P.A, smem + kHeaderBytes);
-    MultiBody body(A, smem + kHeaderBytes + args_bytes<MultiArgs>(), P.words, P.breaks, P.out);
+    MultiBody<kFew> body(A, smem + kHeaderBytes + args_bytes<MultiArgs>(), P.words, P.breaks, P.out);
     run_engine(A.G, A.ctl, body, smem, args_bytes<MultiArgs>(), A.body_bytes);
 }
 
@@ -510,14 +526,15 @@ static tqp_status shared_run(tqp_ctx* ctx, const tqp_table* t, const tqp_scan_qu
         for (size_t g = 0; g < groups.size(); ++g)
             for (int m : groups[g]) launch_of[m] = static_cast<int32_t>(g);
     }
-    static SmemFlags attr;
-    TQP_TRY(allow_smem(ctx, reinterpret_cast<const void*>(k_filter_multi), attr));
+    static SmemFlags attr[2];
+    TQP_TRY(allow_smem(ctx, reinterpret_cast<const void*>(k_filter_multi<false>), attr[0]));
+    TQP_TRY(allow_smem(ctx, reinterpret_cast<const void*>(k_filter_multi<true>), attr[1]));
     for (const auto& g : groups) {
         MultiArgs A;
         std::vector<unsigned char> blob;
         size_t smem = 0;
         int per_sm = 0;
-        TQP_TRY(mq_lower_group(ctx, t, qs, g, nullptr, args_bytes<MultiArgs>(), false, &A, &blob, &smem, &per_sm));
+        TQP_TRY(mq_lower_group(ctx, t, qs, g, nullptr, args_bytes<MultiArgs>(), &A, &blob, &smem, &per_sm));
         if (A.G.ntiles == 0) {
             for (int m : g) TQP_TRY(mq_zero(qs[m].out, st));
             continue;
@@ -538,11 +555,12 @@ static tqp_status shared_run(tqp_ctx* ctx, const tqp_table* t, const tqp_scan_qu
         A.acc = reinterpret_cast<unsigned long long*>(d) + 1;
         A.ctl.err = ctx->d_err;
         A.ctl.wait_cap = ctx->wait_cap;
-        const int grid = engine_grid(ctx, reinterpret_cast<const void*>(k_filter_multi), smem, A.G.ntiles, per_sm);
+        const auto kern = mq_few(A.nq, A.nexpr) ? k_filter_multi<true> : k_filter_multi<false>;
+        const int grid = engine_grid(ctx, reinterpret_cast<const void*>(kern), smem, A.G.ntiles, per_sm);
         A.ctl.chunk_tiles = (A.G.ntiles + grid - 1) / grid;
         A.ctl.nchunks = (A.G.ntiles + A.ctl.chunk_tiles - 1) / A.ctl.chunk_tiles;
         L[0].A = A;
-        k_filter_multi<<<static_cast<unsigned>(A.ctl.nchunks), kEngineThreads, smem, st>>>(L[0]);
+        kern<<<static_cast<unsigned>(A.ctl.nchunks), kEngineThreads, smem, st>>>(L[0]);
         TQP_CUDA(cudaGetLastError());
     }
     for (int i : singles)

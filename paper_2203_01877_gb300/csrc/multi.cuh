@@ -16,16 +16,25 @@
 //     breakpoints span at most kMqDirectMax values, else a branch-free binary
 //     search over the sorted breakpoints.  The cost per row grows with the
 //     number of condition columns, not with the number of queries;
-//   * accumulation: lane q keeps query q's count and sum in registers. Rows that
-//     pass some query join a queue of their warp (pass mask and row, in shared
-//     memory); 32 at a time their values are computed, one row per lane, and the
-//     masks are transposed (five exchange steps), so that lane q holds the rows
-//     that pass query q: its count is a bit count, and it adds their values. 60M
-//     rows and 32 queries of 2% each took 654 us with a shared-memory atomic per
-//     (row, passing query) pair instead (the lanes wait for the one with most
-//     pairs, 244 warp instructions per 32 rows), now 575; values computed for whole
-//     steps before the queue: 529, but 443 against 421 with 5 queries. At the end
-//     of a chunk lane q moves query q's totals to global memory;
+//   * accumulation, many queries: lane q keeps query q's count and sum in
+//     registers. Rows that pass some query join a queue of their warp (pass mask
+//     and row, in shared memory); 32 at a time their values are computed, one row
+//     per lane, and the masks are transposed (five exchange steps), so that lane q
+//     holds the rows that pass query q: its count is a bit count, and it adds their
+//     values;
+//   * accumulation, few queries (up to kMqFew; kMqFewCounts without sums): each
+//     lane keeps its own rows' totals of every query in registers. A step with more
+//     than 32 passing rows adds each lane's rows at once, the rest goes through the
+//     queue, so that the adds of 32 rows share their instructions;
+//     20M rows of four int32 columns, us, with a shared-memory atomic per (row,
+//     passing query) pair / the transposed queue for any number of queries / this:
+//     3 queries of 2% each 114 / 103 / 90, of 20% 193 / 258 / 114; 5 of 20% 295 /
+//     291 / 137; 8 of 2% 147 / 129 / 114, of 20% 462 / 299 / 154, of 80% 566 / 559 /
+//     176; 12 of 20% 657 / 314 / 293; 32 of 2% 212 / 209 / 188. Eight counts without
+//     sums over two columns: 99 transposed, 118 per row.
+//     The queues' shared memory is kept small because a launch shape has to fit
+//     beside it: with 160 rows per warp twelve queries over six int64 columns lose a
+//     resident CTA (519 -> 919 us);
 //   * per-query row ranges: a query may cover only rows [rlo, rhi) of the
 //     scan (queries over slices of one table).  Per tile a ballot splits the
 //     queries into those covering the whole tile and those touching part of
@@ -48,14 +57,28 @@ constexpr int kMqWords = 5120;      // mask words of all lookup tables (shared m
 constexpr int kMqBreaks = 512;      // breakpoints of the searched tables (shared memory)
 constexpr int kMqDirectMax = 4096;  // direct tables: at most this many entries per column
 constexpr int kMqRows = 4;          // rows per lane of a step
-constexpr int kMqQueue = (kMqRows + 1) * kWarp;  // queued rows of a warp: a step's and fewer than kWarp before it
-// per consumer warp: 32 rows' values for each sum expression; the queued rows' pass masks and tile rows
-constexpr int kMqAccBytes = kConsumerWarps * (kMqExprs * kWarp * 8 + kMqQueue * 8);
+constexpr int kMqFew = 8;           // launches of at most this many queries keep their totals per row, in registers
+
+// Count-only launches: a transposed mask's bit count costs less than their rows' adds from here on.
+constexpr int kMqFewCounts = 4;
+inline bool mq_few(size_t nq, size_t nexpr) { return nq <= static_cast<size_t>(nexpr ? kMqFew : kMqFewCounts); }
+
+// Queued rows (pass mask and tile row) of a consumer warp: fewer than kWarp, then
+// a step's where it has at most kWarp (few queries), or half a step's.
+__host__ __device__ constexpr int mq_queue(bool few) { return (few ? 2 : 1 + kMqRows / 2) * kWarp; }
+
+// The queues; many queries: and 32 values of a second expression per warp (the
+// first one's take the place of the rows they belong to).
+__host__ __device__ constexpr int mq_queue_bytes(bool few, int nexpr) {
+    return kConsumerWarps * (mq_queue(few) + (!few && nexpr > 1 ? kWarp : 0)) * 8;
+}
+// Shared memory of the queues that a launch shape has to leave room for.
+constexpr int kMqShapeBytes = 3072;
 
 // Shared memory of one launch's body: row queues | mask words | breakpoints.
 __host__ __device__ constexpr int mq_words_bytes(int nwords) { return (nwords * 4 + 15) / 16 * 16; }
-__host__ __device__ constexpr int mq_body_bytes(int nwords, int nbreaks) {
-    return (kMqAccBytes + mq_words_bytes(nwords) + nbreaks * 8 + 127) / 128 * 128;
+__host__ __device__ constexpr int mq_body_bytes(bool few, int nexpr, int nwords, int nbreaks) {
+    return (mq_queue_bytes(few, nexpr) + mq_words_bytes(nwords) + nbreaks * 8 + 127) / 128 * 128;
 }
 
 // One condition column of a launch.
@@ -159,20 +182,22 @@ struct MqHot {
 };
 constexpr int kMqFastCols = 4;  // condition columns of the fast path
 
+template <bool kFew>
 struct MultiBody {
     static constexpr int kMinBlocks = 2;
-    static constexpr int kSmemBytes = mq_body_bytes(kMqWords, kMqBreaks);  // the largest launch
+    static constexpr int kSmemBytes = mq_body_bytes(kFew, kMqExprs, kMqWords, kMqBreaks);  // the largest launch
     static constexpr int kU = kMqRows;  // rows per lane per step
 
     const MultiArgs& A;
     const uint32_t* w;         // shared-memory copy of the masks
     const int64_t* bk;         // shared-memory copy of the breakpoints
-    unsigned long long* qval;  // this warp's values [expression][lane], and its queue: masks and tile rows
-    uint32_t* qmask;
-    uint32_t* qrow;
+    unsigned long long* queue; // this warp's queued rows (pass mask, tile row << 32), and a second expression's values
+    unsigned long long* val1;
     int qn = 0;                // queued rows (warp-uniform)
     unsigned long long qsum = 0;  // lane q: query q's sum and count since the last chunk
     unsigned int qcnt = 0;
+    unsigned long long fsum[kMqFew] = {};  // (few queries) this lane's rows' share of them
+    unsigned int fcnt[kMqFew] = {};
     int64_t rlo = 0, rhi = 0;  // lane q: query q's row range
     MqHot hot[kMqFastCols];    // fast path: the condition columns
     bool fast = false;         // every condition column has a direct table (at most kMqFastCols)
@@ -186,8 +211,9 @@ struct MultiBody {
     __device__ MultiBody(const MultiArgs& a, unsigned char* sm, const uint32_t* words, const int64_t* breaks,
                          const MqOut* out)
         : A(a), outp(out) {
-        uint32_t* ws = reinterpret_cast<uint32_t*>(sm + kMqAccBytes);
-        int64_t* bs = reinterpret_cast<int64_t*>(sm + kMqAccBytes + mq_words_bytes(a.nwords));
+        const int qbytes = mq_queue_bytes(kFew, a.nexpr);
+        uint32_t* ws = reinterpret_cast<uint32_t*>(sm + qbytes);
+        int64_t* bs = reinterpret_cast<int64_t*>(sm + qbytes + mq_words_bytes(a.nwords));
         for (int i = threadIdx.x; i < a.nwords; i += blockDim.x) ws[i] = words[i];
         for (int i = threadIdx.x; i < a.nbreaks; i += blockDim.x) bs[i] = breaks[i];
         w = ws;
@@ -195,9 +221,8 @@ struct MultiBody {
         const int warp = threadIdx.x / kWarp;
         const int lane = threadIdx.x % kWarp;
         const int cw = warp < kConsumerWarps ? warp : 0;
-        qval = reinterpret_cast<unsigned long long*>(sm) + cw * kMqExprs * kWarp;
-        qmask = reinterpret_cast<uint32_t*>(sm + kConsumerWarps * kMqExprs * kWarp * 8) + cw * 2 * kMqQueue;
-        qrow = qmask + kMqQueue;
+        queue = reinterpret_cast<unsigned long long*>(sm) + cw * mq_queue(kFew);
+        val1 = reinterpret_cast<unsigned long long*>(sm) + kConsumerWarps * mq_queue(kFew) + cw * kWarp;
         if (lane < a.nq) {
             rlo = out[lane].rlo;
             rhi = out[lane].rhi;
@@ -273,50 +298,108 @@ struct MultiBody {
         }
     }
 
+    // Expression e at tile row r.
+    __device__ __forceinline__ unsigned long long value(const ScanGeom& G, const TileView& v, int e, int r) {
+        if (!v.full)
+            return static_cast<unsigned long long>(mq_factor_row(G, v, A.e[e], 0, A.ecol[e][0], r)) *
+                   static_cast<unsigned long long>(mq_factor_row(G, v, A.e[e], 1, A.ecol[e][1], r));
+        int64_t x[1];
+        prod_eval<1>(A.e[e], v.stage, r, x);
+        return static_cast<unsigned long long>(x[0]);
+    }
+
+    // The same at rows r0 + 32 j.
+    template <int U>
+    __device__ __forceinline__ void values(const ScanGeom& G, const TileView& v, int e, int r0, int64_t (&x)[U]) {
+        if (v.full) {
+            prod_eval<U>(A.e[e], v.stage, r0, x);
+            return;
+        }
+#pragma unroll
+        for (int j = 0; j < U; ++j)
+            if (r0 + kWarp * j < v.rows) x[j] = static_cast<int64_t>(value(G, v, e, r0 + kWarp * j));
+    }
+
+    // (few queries) One row into the queries it passes.
+    __device__ __forceinline__ void add_row(uint32_t m, unsigned long long x0, unsigned long long x1) {
+#pragma unroll
+        for (int q = 0; q < kMqFew; ++q) {
+            if (q >= A.nq) break;
+            if (!((m >> q) & 1u)) continue;
+            fsum[q] += (A.esel >> q) & 1u ? x1 : x0;
+            ++fcnt[q];
+        }
+    }
+
     // The last (up to kWarp) queued rows, from `first` on, into the queries they pass.
     __device__ __forceinline__ void flush(const ScanGeom& G, const TileView& v, int first, int lane) {
         __syncwarp();
         const bool in = first + lane < qn;
-        const uint32_t m = in ? qmask[first + lane] : 0u;
+        const unsigned long long t = in ? queue[first + lane] : 0ULL;
+        unsigned long long x0 = 0, x1 = 0;
         if (A.nexpr > 0 && in) {
-            const int r = static_cast<int>(qrow[first + lane]);
-#pragma unroll
-            for (int e = 0; e < kMqExprs; ++e) {
-                if (e >= A.nexpr) break;
-                int64_t x[1];
-                if (v.full) prod_eval<1>(A.e[e], v.stage, r, x);
-                else x[0] = static_cast<int64_t>(static_cast<uint64_t>(mq_factor_row(G, v, A.e[e], 0, A.ecol[e][0], r)) *
-                                                 static_cast<uint64_t>(mq_factor_row(G, v, A.e[e], 1, A.ecol[e][1], r)));
-                qval[e * kWarp + lane] = static_cast<unsigned long long>(x[0]);
-            }
-        }
-        __syncwarp();
-        uint32_t x = warp_transpose(m, lane);  // the rows of this lane's query
-        qcnt += __popc(x);
-        if (A.nexpr > 0) {
-            const unsigned long long* val = qval + ((A.esel >> lane) & 1u) * kWarp;
-            for (; x; x &= x - 1) qsum += val[__ffs(x) - 1];
+            x0 = value(G, v, 0, static_cast<int>(t >> 32));
+            if (A.nexpr > 1) x1 = value(G, v, 1, static_cast<int>(t >> 32));
         }
         qn = first;
+        if constexpr (kFew) {
+            add_row(static_cast<uint32_t>(t), x0, x1);
+            __syncwarp();  // (read before the next rows take their place)
+            return;
+        }
+        unsigned long long* val0 = queue + first;
+        __syncwarp();  // (read before the values take their place)
+        val0[lane] = x0;
+        if (A.nexpr > 1) val1[lane] = x1;
+        __syncwarp();
+        uint32_t x = warp_transpose(static_cast<uint32_t>(t), lane);  // the rows of this lane's query
+        qcnt += __popc(x);
+        if (A.nexpr > 0) {
+            const unsigned long long* val = (A.esel >> lane) & 1u ? val1 : val0;
+            for (; x; x &= x - 1) qsum += val[__ffs(x) - 1];
+        }
         __syncwarp();  // (read before the next rows take their place)
     }
 
-    // The step's rows (r0 + 32 j) that pass some query into the queue (every lane calls it).
+    // The step's rows (r0 + 32 j) into the queries they pass (every lane calls it).
     template <int U>
     __device__ __forceinline__ void add_rows(const ScanGeom& G, const TileView& v, int r0, const uint32_t (&m)[U]) {
-        static_assert(U == kMqRows, "the queue holds a step's rows");
+        static_assert(U == kMqRows && U % 2 == 0, "the queue holds half a step's rows");
+        const int lane = static_cast<int>(threadIdx.x % kWarp);
         const uint32_t lt = lanemask_lt();
+        uint32_t b[U];
+        int n = 0;
 #pragma unroll
         for (int j = 0; j < U; ++j) {
-            const uint32_t b = __ballot_sync(0xffffffffu, m[j] != 0);
-            if (m[j]) {
-                const int at = qn + __popc(b & lt);
-                qmask[at] = m[j];
-                qrow[at] = static_cast<uint32_t>(r0 + kWarp * j);
-            }
-            qn += __popc(b);
+            b[j] = __ballot_sync(0xffffffffu, m[j] != 0);
+            n += __popc(b[j]);
         }
-        while (qn >= kWarp) flush(G, v, qn - kWarp, static_cast<int>(threadIdx.x % kWarp));
+        if (n == 0) return;
+        if constexpr (kFew) {
+            if (n > kWarp) {  // many passing rows: each lane its own
+                int64_t x0[U], x1[U];
+#pragma unroll
+                for (int j = 0; j < U; ++j) x0[j] = x1[j] = 0;
+                if (A.nexpr > 0) values<U>(G, v, 0, r0, x0);
+                if (A.nexpr > 1) values<U>(G, v, 1, r0, x1);
+#pragma unroll
+                for (int j = 0; j < U; ++j)
+                    add_row(m[j], static_cast<unsigned long long>(x0[j]), static_cast<unsigned long long>(x1[j]));
+                return;
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < U; h += U / 2) {
+#pragma unroll
+            for (int j = h; j < h + U / 2; ++j) {
+                if (m[j])
+                    queue[qn + __popc(b[j] & lt)] = m[j] | (static_cast<unsigned long long>(r0 + kWarp * j) << 32);
+                qn += __popc(b[j]);
+            }
+            if (!kFew)
+                while (qn >= kWarp) flush(G, v, qn - kWarp, lane);
+        }
+        if (kFew && qn >= kWarp) flush(G, v, qn - kWarp, lane);
     }
 
     // General path (a ragged last tile, searched tables, more than
@@ -363,6 +446,20 @@ struct MultiBody {
     }
 
     __device__ void chunk_end(const ScanGeom&, long long, long long, long long, int, int lane) {
+        if constexpr (kFew) {
+#pragma unroll
+            for (int q = 0; q < kMqFew; ++q) {
+                const unsigned long long s = static_cast<unsigned long long>(
+                    group_sum_i64(0xffffffffu, static_cast<long long>(fsum[q])));
+                const unsigned int c = __reduce_add_sync(0xffffffffu, fcnt[q]);
+                if (lane == q) {
+                    qsum = s;
+                    qcnt = c;
+                }
+                fsum[q] = 0;
+                fcnt[q] = 0;
+            }
+        }
         const unsigned long long ls = qsum;
         const unsigned long long lc = qcnt;
         qsum = 0;
@@ -437,10 +534,9 @@ void mq_pack(const tqp_table* t, const std::vector<MqQuery>& qs, std::vector<std
 // resolved by mq_bind once the blob is in device memory), the blob itself
 // (lookup tables and per-query outputs) and the launch's shared memory.
 // extra_smem: shared memory before the body (staged arguments, a batch job);
-// fixed_body: the body takes MultiBody::kSmemBytes (a batch's common layout)
-// instead of what this launch's tables need.  tu: NULL for the default tuning.
+// tu: NULL for the default tuning.
 tqp_status mq_lower_group(const tqp_ctx* ctx, const tqp_table* t, const std::vector<MqQuery>& qs,
-                          const std::vector<int>& members, const tqp_tuning* tu, int extra_smem, bool fixed_body,
+                          const std::vector<int>& members, const tqp_tuning* tu, int extra_smem,
                           MultiArgs* A, std::vector<unsigned char>* blob, size_t* smem, int* ctas_per_sm);
 void mq_bind(MultiArgs* A, const unsigned char* d_blob);
 
