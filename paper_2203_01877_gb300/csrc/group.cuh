@@ -169,7 +169,7 @@ long long group_table_cap(long long max_groups);
 size_t group_table_bytes(long long cap, int nacc);
 tqp_status group_table_init(GroupSpec* S, void* mem, long long cap, long long max_groups, cudaStream_t stream,
                             bool clear = true);
-// With `ranged`, the kernels return at once when that plan is on (grouprange.cuh).
+// With `ranged` on, the groups are that plan's entries (grouprange.cuh).
 struct GroupRangePlan;
 tqp_status group_finalize(tqp_ctx* ctx, const GroupSpec& S, const GroupOut& O, cudaStream_t stream,
                           const GroupRangePlan* ranged = nullptr);

@@ -63,56 +63,31 @@ __global__ void __launch_bounds__(kDirThreads) k_groupby_dprep(const __grid_cons
 
 // ---- group-by over key columns of small range (grouprange.cuh) --------------------
 
-__global__ void __launch_bounds__(kDirThreads) k_group_range(const __grid_constant__ GroupRangeArgs A) {
+__global__ void __launch_bounds__(kDirThreads) k_group_range(const __grid_constant__ GroupRangeArgs A,
+                                                             const __grid_constant__ GroupSpec S, int clear) {
+    if (clear) group_clear(S, (S.cap + 1) * S.nacc + 1, true);
     group_range_block(A);
 }
 
-// Clears the entries, or the hash path's table.
 __global__ void __launch_bounds__(256) k_group_clear(const __grid_constant__ GroupSpec S, const GroupRangePlan* plan) {
-    const bool on = plan->on;
-    const long long tid = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
-    const long long nth = static_cast<long long>(gridDim.x) * blockDim.x;
-    const long long words = (on ? plan->entries : S.cap + 1) * S.nacc + (on ? 0 : 1);  // (ndistinct follows the table)
-    ulonglong2* p = reinterpret_cast<ulonglong2*>(S.acc);
-    for (long long i = tid; i < words / 2; i += nth) p[i] = make_ulonglong2(0, 0);
-    if (tid == 0 && words % 2) S.acc[words - 1] = 0;
-    if (on) return;
-    for (long long i = tid; i <= S.cap; i += nth) S.keys[i] = kEmptyKey;
+    if (plan->on) group_clear(S, plan->entries * S.nacc, false);
+    else group_clear(S, (S.cap + 1) * S.nacc + 1, true);
+}
+
+// kL2: the entries in L2 too; without it they have a kernel of their own.
+template <bool kL2>
+__global__ void __launch_bounds__(kGrThreads, 1) k_group_agg(const __grid_constant__ GroupRangeArgs A) {
+    extern __shared__ __align__(16) uint32_t gsm[];
+    if (!A.plan->on || (!kL2 && !A.plan->smem)) return;
+    const GroupRangePlan P = *A.plan;
+    if (P.smem) group_smem_block(A, P, gsm);
+    else if (kL2) group_l2_block<kGrThreads>(A, P);
 }
 
 __global__ void __launch_bounds__(kPaThreads, kPaMinBlocks) k_group_l2(const __grid_constant__ GroupRangeArgs A) {
+    if (!A.plan->on || A.plan->smem) return;
     const GroupRangePlan P = *A.plan;
-    if (!P.on || P.smem) return;
-    switch (A.nval) {
-        case 0: gr_l2_loop<1>(A, P); break;
-        case 1: gr_l2_loop<2>(A, P); break;
-        case 2: gr_l2_loop<3>(A, P); break;
-        default: gr_l2_loop<4>(A, P); break;
-    }
-}
-
-__global__ void __launch_bounds__(kGrSmemThreads, 1) k_group_smem(const __grid_constant__ GroupRangeArgs A) {
-    extern __shared__ __align__(16) uint32_t gsm[];
-    group_smem_block(A, gsm);
-}
-
-__global__ void __launch_bounds__(kGrEmitThreads) k_group_count(const __grid_constant__ GroupSpec S,
-                                                                const GroupRangePlan* plan, uint32_t* counts) {
-    if (!plan->on) return;
-    const long long e0 = static_cast<long long>(blockIdx.x) * kGrEmitPer, D = plan->entries;
-    if (e0 >= D) return;
-    int c = 0;
-    for (int s = 0; s < kGrEmitPer / kGrEmitThreads; ++s) {
-        const long long e = e0 + s * kGrEmitThreads + threadIdx.x;
-        c += __syncthreads_count(e < D && S.acc[e * S.nacc] != 0);
-    }
-    if (threadIdx.x == 0) counts[blockIdx.x] = static_cast<uint32_t>(c);
-}
-
-__global__ void __launch_bounds__(kGrEmitThreads) k_group_rows(const __grid_constant__ GroupSpec S,
-                                                               const __grid_constant__ GroupOut O,
-                                                               const GroupRangePlan* plan, const uint32_t* counts) {
-    group_rows_block(plan, S, O, counts);
+    group_l2_block<kPaThreads>(A, P);
 }
 
 // ---- finalize ----------------------------------------------------------------
@@ -120,15 +95,25 @@ __global__ void __launch_bounds__(kGrEmitThreads) k_group_rows(const __grid_cons
 __global__ void __launch_bounds__(kFinThreads) k_groupby_finalize_small(const __grid_constant__ GroupSpec S,
                                                                         const __grid_constant__ GroupOut O,
                                                                         const GroupRangePlan* rp) {
-    if (rp && rp->on) return;
     extern __shared__ __align__(16) unsigned char fsm[];
+    if (rp && rp->on) {
+        group_rows_small(rp, S, O);
+        return;
+    }
     finalize_small_block(S, O, fsm);
 }
 
-// Large tables: collect (key, slot) pairs, radix sort, emit.
-__global__ void k_groupby_collect(const __grid_constant__ GroupSpec S, uint64_t* pk, uint32_t* ps,
-                                  long long* n_out, const GroupRangePlan* rp) {
-    if (rp && rp->on) return;
+// Large tables: collect (key, slot) pairs, radix sort, emit. Aggregated by key
+// range: the used entries of the output blocks (counts in the unused hash
+// keys), nothing to sort, and their rows.
+__global__ void __launch_bounds__(kGrEmitThreads) k_groupby_collect(const __grid_constant__ GroupSpec S, uint64_t* pk,
+                                                                    uint32_t* ps, long long* n_out,
+                                                                    const GroupRangePlan* rp) {
+    if (rp && rp->on) {
+        for (int b = blockIdx.x; b < gr_blocks(rp); b += gridDim.x)
+            group_count_block(rp, S, reinterpret_cast<uint32_t*>(S.keys), b);
+        return;
+    }
     // warp-uniform trip count: blockDim is a multiple of 32
     for (long long base = blockIdx.x * static_cast<long long>(blockDim.x); base <= S.cap;
          base += static_cast<long long>(gridDim.x) * blockDim.x) {
@@ -142,10 +127,17 @@ __global__ void k_groupby_collect(const __grid_constant__ GroupSpec S, uint64_t*
     }
 }
 
-__global__ void k_groupby_emit(const __grid_constant__ GroupSpec S, const __grid_constant__ GroupOut O,
-                               const uint64_t* pk, const uint32_t* ps, const long long* n_in,
-                               const GroupRangePlan* rp) {
-    if (rp && rp->on) return;
+__global__ void __launch_bounds__(kGrEmitThreads) k_groupby_emit(const __grid_constant__ GroupSpec S,
+                                                                 const __grid_constant__ GroupOut O, const uint64_t* pk,
+                                                                 const uint32_t* ps, const long long* n_in,
+                                                                 const GroupRangePlan* rp) {
+    if (rp && rp->on) {
+        for (int b = blockIdx.x; b < gr_blocks(rp); b += gridDim.x) {
+            if (!group_rows_block(rp, S, O, reinterpret_cast<const uint32_t*>(S.keys), b)) return;
+            __syncthreads();
+        }
+        return;
+    }
     const long long G = *n_in;
     const bool overflow = static_cast<long long>(*S.ndistinct) > S.max_groups || G > O.capacity;
     if (overflow) {
@@ -288,14 +280,14 @@ tqp_status group_finalize(tqp_ctx* ctx, const GroupSpec& S, const GroupOut& O, c
     uint32_t* v0 = reinterpret_cast<uint32_t*>(k1 + nmax);
     uint32_t* v1 = v0 + nmax;
     TQP_CUDA(cudaMemsetAsync(d_n, 0, sizeof(long long), stream));
-    const int threads = 256;
+    const int threads = kGrEmitThreads;
     const int blocks = static_cast<int>(std::min<long long>((nmax + threads - 1) / threads, ctx->num_sms * 8LL));
     k_groupby_collect<<<blocks, threads, 0, stream>>>(S, k0, v0, d_n, rp);
     bool in1 = false;
     const int end_bit = (S.width + 7) / 8 * 8;
     TQP_TRY(radix_sort_pairs(ctx, k0, v0, k1, v1, d_n, nmax, 0, end_bit, rs, stream, &in1));
     const int eblocks = static_cast<int>(
-        std::max<long long>(1, std::min<long long>((std::min(nmax, O.capacity) + threads - 1) / threads,
+        std::max<long long>(1, std::min<long long>((std::min(nmax, rp ? nmax : O.capacity) + threads - 1) / threads,
                                                    ctx->num_sms * 8LL)));
     k_groupby_emit<<<eblocks, threads, 0, stream>>>(S, O, in1 ? k1 : k0, in1 ? v1 : v0, d_n, rp);
     TQP_CUDA(cudaGetLastError());
@@ -519,10 +511,11 @@ static bool lower_group_range(const tqp_table* t, const GroupArgs& A, GroupRange
     return true;
 }
 
-// The kernels over key ranges; the hash path's that follow them return at once
-// when the plan turns out on.
-static tqp_status launch_group_range(tqp_ctx* ctx, const GroupSpec& S, const GroupOut& O, GroupRangeArgs& R,
-                                     GroupRangePlan* plan, uint32_t* counts, cudaStream_t stream) {
+// The aggregation over key ranges (the plan zeroed); the hash path's that
+// follows returns at once when the plan turns out on, and its output kernels
+// write the groups of either.
+static tqp_status launch_group_range(tqp_ctx* ctx, const GroupSpec& S, GroupRangeArgs& R, GroupRangePlan* plan,
+                                     cudaStream_t stream) {
     R.plan = plan;
     R.acc = S.acc;
     R.max_entries = std::min<long long>(S.cap + 1, kGrMaxEntries);
@@ -530,16 +523,18 @@ static tqp_status launch_group_range(tqp_ctx* ctx, const GroupSpec& S, const Gro
     auto grid = [](long long work, long long per, long long most) {
         return static_cast<unsigned>(std::max<long long>(1, std::min<long long>((work + per - 1) / per, most)));
     };
-    TQP_CUDA(cudaMemsetAsync(plan, 0, sizeof(*plan), stream));
-    k_group_range<<<grid(n, 8192, 4 * sms), kDirThreads, 0, stream>>>(R);
-    k_group_clear<<<grid((S.cap + 1) * S.nacc, 4096, 8 * sms), 256, 0, stream>>>(S, plan);
-    static SmemFlags attr_done;
-    TQP_TRY(allow_smem(ctx, reinterpret_cast<const void*>(k_group_smem), attr_done));
-    k_group_smem<<<grid(n, kGrSmemThreads * 4, sms), kGrSmemThreads, kGrSmemBytes, stream>>>(R);
-    k_group_l2<<<grid(n, kPaThreads * 4, kPaMinBlocks * sms), kPaThreads, 0, stream>>>(R);
-    const unsigned eb = grid(R.max_entries, kGrEmitPer, kGrMaxEntries / kGrEmitPer + 1);
-    k_group_count<<<eb, kGrEmitThreads, 0, stream>>>(S, plan, counts);
-    k_group_rows<<<eb, kGrEmitThreads, 0, stream>>>(S, O, plan, counts);
+    const size_t bytes = static_cast<size_t>(S.cap + 1) * (8 + 8 * S.nacc);
+    const bool fused = bytes <= kGrClearBytes;
+    k_group_range<<<std::max(grid(n, 8192, 4 * sms), fused ? grid(bytes, kGrClearPer, 4 * sms) : 1u), kDirThreads, 0,
+                    stream>>>(R, S, fused);
+    if (!fused) k_group_clear<<<grid((S.cap + 1) * S.nacc, 4096, 8 * sms), 256, 0, stream>>>(S, plan);
+    static SmemFlags attr_done[2];
+    const bool split = n >= kGrSplitRows;
+    const auto agg = split ? k_group_agg<false> : k_group_agg<true>;
+    TQP_TRY(allow_smem(ctx, reinterpret_cast<const void*>(agg), attr_done[split]));
+    const long long smem = std::min<long long>(n / kGrRowsPerEntry * (4 + 8 * R.nval), kGrSmemBytes);
+    agg<<<grid(n, kGrThreads * 4, sms), kGrThreads, static_cast<size_t>(smem), stream>>>(R);
+    if (split) k_group_l2<<<grid(n, kPaThreads * 4, kPaMinBlocks * sms), kPaThreads, 0, stream>>>(R);
     TQP_CUDA(cudaGetLastError());
     return TQP_OK;
 }
@@ -620,16 +615,13 @@ tqp_status launch_groupby(tqp_ctx* ctx, const tqp_table* t, const tqp_pred* pred
     // over key ranges, if they turn out small (and the caller set no shape of the staged scans)
     GroupRangeArgs R;
     GroupRangePlan* rp = nullptr;
-    uint32_t* counts = nullptr;
     if (!direct && topk == 0 && !user_shape(ctx) && lower_group_range(t, A, &R)) {
-        // no scratch of its own: the plan lies beside the scan's ticket, the blocks' counts in the
-        // hash table's keys (unused when the plan is on; one word per kGrEmitPer entries)
-        static_assert(sizeof(GroupRangePlan) <= 192, "beside the ticket");
+        static_assert(sizeof(GroupRangePlan) <= 192, "the plan lies beside the ticket");
         rp = reinterpret_cast<GroupRangePlan*>(ticket + 8);
-        counts = static_cast<uint32_t*>(tab);
+        TQP_CUDA(cudaMemsetAsync(ticket, 0, 256, stream));
     }
     TQP_TRY(group_table_init(&A.S, tab, cap, max_groups, stream, !direct && !rp));
-    if (rp) TQP_TRY(launch_group_range(ctx, A.S, O, R, rp, counts, stream));
+    if (rp) TQP_TRY(launch_group_range(ctx, A.S, R, rp, stream));
     if (direct) {
         // two launches: the range pass (which also clears the table), then the
         // aggregation, whose last CTA finalizes the table unless top-k follows
@@ -691,7 +683,7 @@ tqp_status launch_groupby(tqp_ctx* ctx, const tqp_table* t, const tqp_pred* pred
         A.ctl.ticket = ticket;
         A.ctl.err = ctx->d_err;
         A.ctl.wait_cap = ctx->wait_cap;
-        TQP_CUDA(cudaMemsetAsync(ticket, 0, 8, stream));
+        if (!rp) TQP_CUDA(cudaMemsetAsync(ticket, 0, 8, stream));
         k_groupby<<<static_cast<int>(A.ctl.nchunks), kEngineThreads, smem, stream>>>(A, rp);
         TQP_CUDA(cudaGetLastError());
     }
