@@ -20,9 +20,21 @@ constexpr int kSortWarps = kSortThreads / kWarp;
 constexpr int kSortItems = 16;                          // per thread
 constexpr int kSortTile = kSortThreads * kSortItems;    // 4096
 constexpr int kSortSlice = kSortTile / kSortWarps;      // 512 per warp
-constexpr int kSortBlocksPerSm = 4;
+constexpr int kSortScanThreads = 1024;                  // of a scan of its own
+constexpr int kSortBlocksPerSm = 8;
+constexpr long long kSortOneLaunch = 1LL << 22;         // items up to which the passes share a launch
+
+// A pass of a shared launch reads what an earlier one wrote from other SMs (L2
+// only); a launch of its own may read through L1, which the second read of a
+// tile hits.
+template <bool kShared, class T>
+__device__ __forceinline__ T rs_load(const T* p) {
+    if constexpr (kShared) return __ldcg(p);
+    else return __ldg(p);
+}
 
 // Digit counts of tiles blockIdx.x, blockIdx.x + gridDim.x, ...
+template <bool kShared>
 __device__ __forceinline__ void rs_upsweep(const uint64_t* keys, long long n, int shift, uint32_t* hist, long long ntiles,
                                            unsigned long long* digit_tot, uint32_t* cnt) {
     for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
@@ -32,33 +44,35 @@ __device__ __forceinline__ void rs_upsweep(const uint64_t* keys, long long n, in
         if (base < n) {
             for (int i = 0; i < kSortItems; ++i) {
                 const long long idx = base + i * kSortThreads + threadIdx.x;
-                if (idx < n) atomicAdd(&cnt[(__ldcg(&keys[idx]) >> shift) & 0xFF], 1u);
+                if (idx < n) atomicAdd(&cnt[(rs_load<kShared>(&keys[idx]) >> shift) & 0xFF], 1u);
             }
         }
         __syncthreads();
         const uint32_t c = cnt[threadIdx.x];
         hist[static_cast<long long>(threadIdx.x) * ntiles + tile] = c;
         if (c) atomicAdd(&digit_tot[threadIdx.x], static_cast<unsigned long long>(c));
+        if constexpr (!kShared) break;  // (a block per tile)
     }
 }
 
 // Digits blockIdx.x, blockIdx.x + gridDim.x, ...: each digit's tile counts to
 // output positions (all smaller digits' totals, then the tiles before).
+template <bool kShared, int kThreads>
 __device__ __forceinline__ void rs_scan(uint32_t* hist, long long ntiles, const unsigned long long* digit_tot,
                                         unsigned long long* wsum) {
     const int lane = threadIdx.x % kWarp, w = threadIdx.x / kWarp;
     for (int d = blockIdx.x; d < 256; d += gridDim.x) {
-        unsigned long long x = static_cast<int>(threadIdx.x) < d ? __ldcg(&digit_tot[threadIdx.x]) : 0ULL;
+        unsigned long long x = static_cast<int>(threadIdx.x) < d ? rs_load<kShared>(&digit_tot[threadIdx.x]) : 0ULL;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
         if (lane == 0) wsum[w] = x;
         __syncthreads();
         unsigned long long carry = 0;
-        for (int i = 0; i < kSortWarps; ++i) carry += wsum[i];
+        for (int i = 0; i < kThreads / kWarp; ++i) carry += wsum[i];
         uint32_t* row = hist + static_cast<long long>(d) * ntiles;
-        for (long long off = 0; off < ntiles; off += kSortThreads) {
+        for (long long off = 0; off < ntiles; off += kThreads) {
             const long long i = off + threadIdx.x;
-            const unsigned long long v = i < ntiles ? __ldcg(&row[i]) : 0u;
+            const unsigned long long v = i < ntiles ? (kShared ? __ldcg(&row[i]) : row[i]) : 0u;
             unsigned long long incl = v;
 #pragma unroll
             for (int o = 1; o < kWarp; o <<= 1) {
@@ -69,7 +83,7 @@ __device__ __forceinline__ void rs_scan(uint32_t* hist, long long ntiles, const 
             if (lane == kWarp - 1) wsum[w] = incl;
             __syncthreads();
             unsigned long long before = 0, total = 0;
-            for (int j = 0; j < kSortWarps; ++j) {
+            for (int j = 0; j < kThreads / kWarp; ++j) {
                 const unsigned long long y = wsum[j];
                 before += (j < w) ? y : 0ULL;
                 total += y;
@@ -82,6 +96,7 @@ __device__ __forceinline__ void rs_scan(uint32_t* hist, long long ntiles, const 
 }
 
 // Tiles blockIdx.x, blockIdx.x + gridDim.x, ... to their places.
+template <bool kShared>
 __device__ __forceinline__ void rs_downsweep(const uint64_t* kin, const uint32_t* vin, uint64_t* kout, uint32_t* vout,
                                              long long n, int shift, const uint32_t* hist, long long ntiles,
                                              uint32_t (*wcnt)[256]) {
@@ -95,7 +110,7 @@ __device__ __forceinline__ void rs_downsweep(const uint64_t* kin, const uint32_t
         // phase 1: per-warp digit counts of the warp's slice
         for (int i = 0; i < kSortSlice / kWarp; ++i) {
             const long long idx = s0 + i * kWarp + lane;
-            const int dg = idx < n ? static_cast<int>((__ldcg(&kin[idx]) >> shift) & 0xFF) : 256;
+            const int dg = idx < n ? static_cast<int>((rs_load<kShared>(&kin[idx]) >> shift) & 0xFF) : 256;
             const uint32_t peers = __match_any_sync(0xffffffffu, dg);
             if (dg < 256 && lane == __ffs(peers) - 1) wcnt[w][dg] += __popc(peers);
         }
@@ -103,7 +118,7 @@ __device__ __forceinline__ void rs_downsweep(const uint64_t* kin, const uint32_t
         // phase 2: per-warp bases = global tile offset + counts of earlier warps
         {
             const int d = threadIdx.x;  // 256 threads, one digit each
-            uint32_t run = __ldcg(&hist[static_cast<long long>(d) * ntiles + tile]);
+            uint32_t run = rs_load<kShared>(&hist[static_cast<long long>(d) * ntiles + tile]);
             for (int ww = 0; ww < kSortWarps; ++ww) {
                 const uint32_t c = wcnt[ww][d];
                 wcnt[ww][d] = run;
@@ -118,8 +133,8 @@ __device__ __forceinline__ void rs_downsweep(const uint64_t* kin, const uint32_t
             uint32_t v = 0;
             int dg = 256;
             if (idx < n) {
-                k = __ldcg(&kin[idx]);
-                v = __ldcg(&vin[idx]);
+                k = rs_load<kShared>(&kin[idx]);
+                v = rs_load<kShared>(&vin[idx]);
                 dg = static_cast<int>((k >> shift) & 0xFF);
             }
             const uint32_t peers = __match_any_sync(0xffffffffu, dg);
@@ -132,13 +147,14 @@ __device__ __forceinline__ void rs_downsweep(const uint64_t* kin, const uint32_t
             if (dg < 256 && lane == __ffs(peers) - 1) wcnt[w][dg] += __popc(peers);
             __syncwarp();
         }
+        if constexpr (!kShared) break;
         __syncthreads();
     }
 }
 
 // All passes in one cooperative launch. An empty input (a build side of unique
-// keys, a group-by over key ranges) costs this one launch instead of four per
-// pass: 12 to 16 launches of about 2 us each.
+// keys) costs this one launch instead of three per pass: 12 to 16 launches of
+// about 2 us each.
 __global__ void __launch_bounds__(kSortThreads, kSortBlocksPerSm) k_rs_sort(uint64_t* k0, uint32_t* v0, uint64_t* k1,
                                                                             uint32_t* v1, long long* n_ptr, int begin_bit,
                                                                             int end_bit, unsigned long long* digit_tot,
@@ -151,12 +167,12 @@ __global__ void __launch_bounds__(kSortThreads, kSortBlocksPerSm) k_rs_sort(uint
     unsigned int arrivals = 0;
     bool ok = true;
     for (int shift = begin_bit; ok && shift < end_bit; shift += 8) {
-        rs_upsweep(k0, n, shift, hist, ntiles, digit_tot, wcnt[0]);
+        rs_upsweep<true>(k0, n, shift, hist, ntiles, digit_tot, wcnt[0]);
         if (!(ok = grid_barrier(bar, arrivals += gridDim.x, err, wait_cap))) break;
-        rs_scan(hist, ntiles, digit_tot, wsum);
+        rs_scan<true, kSortThreads>(hist, ntiles, digit_tot, wsum);
         if (!(ok = grid_barrier(bar, arrivals += gridDim.x, err, wait_cap))) break;
         if (blockIdx.x == 0) digit_tot[threadIdx.x] = 0;  // (read by the scans only; the next barrier orders it)
-        rs_downsweep(k0, v0, k1, v1, n, shift, hist, ntiles, wcnt);
+        rs_downsweep<true>(k0, v0, k1, v1, n, shift, hist, ntiles, wcnt);
         ok = grid_barrier(bar, arrivals += gridDim.x, err, wait_cap);
         uint64_t* k = k0;
         k0 = k1;
@@ -169,6 +185,30 @@ __global__ void __launch_bounds__(kSortThreads, kSortBlocksPerSm) k_rs_sort(uint
     if (!ok && threadIdx.x == 0) *n_ptr = 0;
 }
 
+// The same by a launch per step, where the input fills the chip and is known to
+// be there: a block per tile and reads through L1. Sort-based group-by, us (one
+// launch / this): 1M rows 278 / 306, 2M 450 / 472, 4M 879 / 883, 8M 1924 / 1893,
+// 60M rows of 64-bit keys 19060 / 18371; a join's 8M unique build rows 183 / 261.
+__global__ void __launch_bounds__(kSortThreads) k_rs_upsweep(const uint64_t* keys, const long long* n_ptr, int shift,
+                                                             uint32_t* hist, long long ntiles,
+                                                             unsigned long long* digit_tot) {
+    __shared__ uint32_t cnt[256];
+    rs_upsweep<false>(keys, *n_ptr, shift, hist, ntiles, digit_tot, cnt);
+}
+
+__global__ void __launch_bounds__(kSortScanThreads) k_rs_scan(uint32_t* hist, long long ntiles,
+                                                              const unsigned long long* digit_tot) {
+    __shared__ unsigned long long wsum[kSortScanThreads / kWarp];
+    rs_scan<false, kSortScanThreads>(hist, ntiles, digit_tot, wsum);
+}
+
+__global__ void __launch_bounds__(kSortThreads) k_rs_downsweep(const uint64_t* kin, const uint32_t* vin, uint64_t* kout,
+                                                               uint32_t* vout, const long long* n_ptr, int shift,
+                                                               const uint32_t* hist, long long ntiles) {
+    __shared__ uint32_t wcnt[kSortWarps][256];
+    rs_downsweep<false>(kin, vin, kout, vout, *n_ptr, shift, hist, ntiles, wcnt);
+}
+
 // Scratch needed by radix_sort_pairs for up to n_max items.
 size_t radix_sort_scratch(long long n_max) {
     const long long ntiles = (n_max + kSortTile - 1) / kSortTile;
@@ -179,15 +219,30 @@ size_t radix_sort_scratch(long long n_max) {
 // input; (k1, v1) are a second buffer of the same size.  *result_in_1 tells
 // which buffer holds the sorted output.  *d_n is 0 afterwards when a wait of the
 // sort expired, so kernels that read the output take the count from there.
+// `optional`: there is usually nothing to sort.
 tqp_status radix_sort_pairs(const tqp_ctx* ctx, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, long long* d_n,
                             long long n_max, int begin_bit, int end_bit, void* scratch, cudaStream_t stream,
-                            bool* result_in_1) {
+                            bool* result_in_1, bool optional) {
     *result_in_1 = false;
     if (n_max <= 0 || end_bit <= begin_bit) return TQP_OK;
     long long ntiles = (n_max + kSortTile - 1) / kSortTile;
     unsigned long long* digit_tot = static_cast<unsigned long long*>(scratch);
     unsigned int* bar = reinterpret_cast<unsigned int*>(digit_tot + 256);  // (one zeroing for both)
     uint32_t* hist = reinterpret_cast<uint32_t*>(digit_tot + 256 + 16);
+    if (n_max > kSortOneLaunch && !optional) {
+        const unsigned blocks = static_cast<unsigned>(ntiles);
+        for (int shift = begin_bit; shift < end_bit; shift += 8) {
+            TQP_CUDA(cudaMemsetAsync(digit_tot, 0, 256 * sizeof(unsigned long long), stream));
+            k_rs_upsweep<<<blocks, kSortThreads, 0, stream>>>(k0, d_n, shift, hist, ntiles, digit_tot);
+            k_rs_scan<<<256, kSortScanThreads, 0, stream>>>(hist, ntiles, digit_tot);
+            k_rs_downsweep<<<blocks, kSortThreads, 0, stream>>>(k0, v0, k1, v1, d_n, shift, hist, ntiles);
+            TQP_CUDA(cudaGetLastError());
+            std::swap(k0, k1);
+            std::swap(v0, v1);
+            *result_in_1 = !*result_in_1;
+        }
+        return TQP_OK;
+    }
     TQP_CUDA(cudaMemsetAsync(digit_tot, 0, 256 * sizeof(unsigned long long) + sizeof(unsigned int), stream));
     const int most = std::min(resident_blocks(ctx->device, reinterpret_cast<const void*>(k_rs_sort), kSortThreads, 0),
                               kSortBlocksPerSm) * ctx->num_sms;
