@@ -555,8 +555,9 @@ __global__ void k_pair_lens(PairTable T, const uint64_t* skey, const long long* 
     }
 }
 
+template <int R>
 __global__ void __launch_bounds__(kJpThreads, kJpMinBlocks) k_join_pairs(const __grid_constant__ PairArgs A) {
-    join_pairs_tile(A);
+    join_pairs_tile<R>(A);
 }
 
 static tqp_status launch_join_pairs(tqp_ctx* ctx, const tqp_table* build, int32_t build_key, const tqp_table* probe,
@@ -570,7 +571,8 @@ static tqp_status launch_join_pairs(tqp_ctx* ctx, const tqp_table* build, int32_
     T.wide = bc.type == TQP_I64;
     T.cap = ht_cap(nb) * ht_scale(ctx);
     A.n = probe->num_rows;
-    A.ntiles = (A.n + kJpTile - 1) / kJpTile;
+    const int rows = jp_rows(A.n, ctx->num_sms);
+    A.ntiles = (A.n + kJpThreads * rows - 1) / (kJpThreads * rows);
     const size_t tab = T.wide ? static_cast<size_t>(T.cap + 1) * 16 : static_cast<size_t>(T.cap) * 8;
     const size_t words = static_cast<size_t>(A.ntiles) + 2;  // look-back words, ticket, rows to sort
     T.mem = arena_alloc(ctx, tab);
@@ -616,7 +618,8 @@ static tqp_status launch_join_pairs(tqp_ctx* ctx, const tqp_table* build, int32_
     A.status = sc + 2;
     A.err = ctx->d_err;
     A.wait_cap = ctx->wait_cap;
-    k_join_pairs<<<static_cast<unsigned>(A.ntiles), kJpThreads, 0, stream>>>(A);
+    const auto kern = rows == 1 ? k_join_pairs<1> : (rows == 4 ? k_join_pairs<4> : k_join_pairs<kJpRows>);
+    kern<<<static_cast<unsigned>(A.ntiles), kJpThreads, 0, stream>>>(A);
     TQP_CUDA(cudaGetLastError());
     return TQP_OK;
 }

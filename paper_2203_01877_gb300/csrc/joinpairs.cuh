@@ -17,13 +17,17 @@
 //     into runs (ascending rows per key) takes its row count from that flag.
 // A look-back step reads 128 tiles' words, four per lane: with 8192-row tiles
 // the prefix then advances faster than the tiles arrive.
+// Small inputs take smaller tiles (jp_rows): 1000 rows against 100K scattered
+// 64-bit keys 78 -> 50 us; 200 rows with 100K build rows each (20M pairs) 183 ->
+// 29 ms, since one warp wrote them all. At 600K rows four rows per lane and 16 are
+// level, at 1M 16 win (48 against 54 us). Pairs past the capacity are not walked
+// through: 20K rows x 1000, counted with capacity 0, 2384 -> 144 us.
 //
 // Measured (60M probe rows, 1.5M unique build keys; staged form -> this): keys
 // scattered over int32 1651 -> 572 us, dense 935 -> 508; 6M rows with ten build
 // rows per scattered key (60M pairs) 1162 -> 358 (about 800 before the lanes of a
-// warp shared the pairs of its rows); 100K rows 115 -> 49. Without the look-back
-// (offsets guessed, for timing) the scattered case takes 490 us, without the
-// lookups 351.
+// warp shared the pairs of its rows). Without the look-back (offsets guessed, for
+// timing) the scattered case takes 490 us, without the lookups 351.
 #pragma once
 
 #include "engine.cuh"
@@ -34,9 +38,7 @@ namespace tqp {
 constexpr int kJpThreads = 512;
 constexpr int kJpMinBlocks = 2;
 constexpr int kJpWarps = kJpThreads / kWarp;
-constexpr int kJpRows = 16;                       // per lane
-constexpr int kJpGroup = 4;                       // rows of a lane in flight together
-constexpr int kJpTile = kJpThreads * kJpRows;     // 8192
+constexpr int kJpRows = 16;                       // per lane; small inputs take fewer (jp_rows)
 constexpr int kJpBucket = 4;
 // A value: the build row of a key's only row, flagged; or the start of the
 // key's run in `bidx`, its length in `rlen`.  All ones: no row.
@@ -150,49 +152,50 @@ __device__ __forceinline__ uint32_t jp_match(const JpBucket& b, uint32_t key, bo
 }
 
 // The values of the lane's rows r0 + 32 j; kJpNone where absent or past the table.
-template <class Key>
+template <class Key, int R>
 __device__ __forceinline__ void jp_lookup(const PairArgs& A, bool direct, unsigned long long lo, unsigned long long range,
-                                          long long r0, uint32_t (&val)[kJpRows]) {
+                                          long long r0, uint32_t (&val)[R]) {
+    constexpr int kGroup = R < 4 ? R : 4;  // rows of a lane in flight together
     const Key* kp = reinterpret_cast<const Key*>(A.key);
     const uint32_t* w = static_cast<const uint32_t*>(A.T.mem);
     if (direct) {
-        unsigned long long d[kJpRows];
+        unsigned long long d[R];
 #pragma unroll
-        for (int j = 0; j < kJpRows; ++j)
+        for (int j = 0; j < R; ++j)
             d[j] = r0 + kWarp * j < A.n ? static_cast<unsigned long long>(static_cast<int64_t>(__ldcs(kp + r0 + kWarp * j))) - lo
                                         : ~0ULL;
 #pragma unroll
-        for (int j = 0; j < kJpRows; ++j) val[j] = d[j] < range ? __ldg(w + d[j]) : kJpNone;
+        for (int j = 0; j < R; ++j) val[j] = d[j] < range ? __ldg(w + d[j]) : kJpNone;
         return;
     }
     // all key loads in flight together
     uint32_t todo = 0;
-    Key x[kJpRows];
+    Key x[R];
 #pragma unroll
-    for (int j = 0; j < kJpRows; ++j) x[j] = r0 + kWarp * j < A.n ? __ldcs(kp + r0 + kWarp * j) : Key(0);
+    for (int j = 0; j < R; ++j) x[j] = r0 + kWarp * j < A.n ? __ldcs(kp + r0 + kWarp * j) : Key(0);
 #pragma unroll
-    for (int j = 0; j < kJpRows; ++j) {
+    for (int j = 0; j < R; ++j) {
         const int64_t k = static_cast<int64_t>(x[j]);
         val[j] = static_cast<uint32_t>(k);
         // (a 64-bit probe key outside int32 has no equal key of a narrow build column)
         todo |= static_cast<uint32_t>((sizeof(Key) < 8 || k == static_cast<int32_t>(k)) && r0 + kWarp * j < A.n) << j;
     }
 #pragma unroll
-    for (int g = 0; g < kJpRows; g += kJpGroup) {
-        uint32_t left = (todo >> g) & ((1u << kJpGroup) - 1), key[kJpGroup], h[kJpGroup];
+    for (int g = 0; g < R; g += kGroup) {
+        uint32_t left = (todo >> g) & ((1u << kGroup) - 1), key[kGroup], h[kGroup];
 #pragma unroll
-        for (int j = 0; j < kJpGroup; ++j) {
+        for (int j = 0; j < kGroup; ++j) {
             key[j] = val[g + j];
             h[j] = pt_home(A.T, key[j]);
             val[g + j] = kJpNone;
         }
         for (long long k = 0; left && k < A.T.cap; ++k) {  // (a full bucket sends a row to the next one)
-            JpBucket b[kJpGroup];
+            JpBucket b[kGroup];
 #pragma unroll
-            for (int j = 0; j < kJpGroup; ++j)
+            for (int j = 0; j < kGroup; ++j)
                 if ((left >> j) & 1u) b[j] = jp_load_bucket(w + 2 * static_cast<size_t>(h[j]));
 #pragma unroll
-            for (int j = 0; j < kJpGroup; ++j) {
+            for (int j = 0; j < kGroup; ++j) {
                 if (!((left >> j) & 1u)) continue;
                 bool more;
                 val[g + j] = jp_match(b[j], key[j], &more);
@@ -278,6 +281,7 @@ __device__ __forceinline__ unsigned long long jp_lookback(unsigned long long* st
     return excl;
 }
 
+template <int R>
 static __device__ __forceinline__ void join_pairs_tile(const PairArgs& A) {
     __shared__ long long tile_sm;
     __shared__ unsigned long long wtot[kJpWarps];
@@ -288,24 +292,24 @@ static __device__ __forceinline__ void join_pairs_tile(const PairArgs& A) {
     const bool direct = pt_direct(A.T, &lo, &range);
     __syncthreads();
     const long long tile = tile_sm;
-    const long long r0 = tile * kJpTile + w * (kWarp * kJpRows) + lane;
+    const long long r0 = tile * (kJpThreads * R) + w * (kWarp * R) + lane;
     // pairs per row: bit j of `one` for a row of one pair; rows of longer runs in `many`
     uint32_t one = 0, many = 0;
-    uint32_t val[kJpRows];
+    uint32_t val[R];
     if (!direct && A.T.wide) {
 #pragma unroll
-        for (int j = 0; j < kJpRows; ++j) val[j] = jp_lookup_wide(A, r0 + kWarp * j);
+        for (int j = 0; j < R; ++j) val[j] = jp_lookup_wide(A, r0 + kWarp * j);
     } else if (A.key_type == TQP_I32) {
-        jp_lookup<int32_t>(A, direct, lo, range, r0, val);
+        jp_lookup<int32_t, R>(A, direct, lo, range, r0, val);
     } else if (A.key_type == TQP_I64) {
-        jp_lookup<long long>(A, direct, lo, range, r0, val);
+        jp_lookup<long long, R>(A, direct, lo, range, r0, val);
     } else {
-        jp_lookup<unsigned char>(A, direct, lo, range, r0, val);
+        jp_lookup<unsigned char, R>(A, direct, lo, range, r0, val);
     }
     // inner: the row's pairs; outer: also (r, -1) without a match; semi / anti: (r, -1) or none
     const bool outer = A.kind == TQP_JOIN_LEFT_OUTER, inner = A.kind == TQP_JOIN_INNER;
 #pragma unroll
-    for (int j = 0; j < kJpRows; ++j) {
+    for (int j = 0; j < R; ++j) {
         const bool in = r0 + kWarp * j < A.n, hit = val[j] != kJpNone;
         const bool run = (inner || outer) && !(val[j] & kJpRow);
         const bool keep = inner ? hit && !run : (outer ? !run : hit == (A.kind == TQP_JOIN_LEFT_SEMI));
@@ -319,7 +323,7 @@ static __device__ __forceinline__ void join_pairs_tile(const PairArgs& A) {
         total = __reduce_add_sync(0xffffffffu, __popc(one));
     } else {
 #pragma unroll
-        for (int j = 0; j < kJpRows; ++j)
+        for (int j = 0; j < R; ++j)
             if ((many >> j) & 1u) total += __ldg(&A.T.rlen[val[j]]);
         total += __popc(one);
 #pragma unroll
@@ -352,7 +356,7 @@ static __device__ __forceinline__ void join_pairs_tile(const PairArgs& A) {
     const uint32_t lt = lanemask_lt();
     if (flat) {
 #pragma unroll
-        for (int j = 0; j < kJpRows; ++j) {
+        for (int j = 0; j < R; ++j) {
             const bool k = (one >> j) & 1u;
             const uint32_t m = __ballot_sync(0xffffffffu, k);
             const unsigned long long p = pos + __popc(m & lt);
@@ -365,10 +369,10 @@ static __device__ __forceinline__ void join_pairs_tile(const PairArgs& A) {
         }
         return;
     }
-    for (int j = 0; j < kJpRows; ++j) {
+    for (int j = 0; j < R; ++j) {
         uint32_t x = kJpNone;
 #pragma unroll
-        for (int q = 0; q < kJpRows; ++q)
+        for (int q = 0; q < R; ++q)
             if (q == j) x = val[q];
         const bool run = (many >> j) & 1u;
         const unsigned long long c = run ? __ldg(&A.T.rlen[x]) : (one >> j) & 1u;
@@ -379,10 +383,13 @@ static __device__ __forceinline__ void join_pairs_tile(const PairArgs& A) {
             if (lane >= o) incl += y;
         }
         const unsigned long long tot = __shfl_sync(0xffffffffu, incl, kWarp - 1);
-        if (tot < (1ULL << 31)) {
+        if (pos >= cap) {
+            // (no pair of these rows is written)
+        } else if (tot < (1ULL << 31)) {
+            const uint32_t writes = static_cast<uint32_t>(cap - pos < tot ? cap - pos : tot);
             // the lanes share the slot's pairs: pair t belongs to the first lane whose inclusive count is above t
             const uint32_t in32 = static_cast<uint32_t>(incl), ex32 = static_cast<uint32_t>(incl - c);
-            for (uint32_t t0 = 0; t0 < tot; t0 += kWarp) {
+            for (uint32_t t0 = 0; t0 < writes; t0 += kWarp) {
                 const uint32_t t = t0 + lane;
                 int o = 0;
 #pragma unroll
@@ -390,7 +397,7 @@ static __device__ __forceinline__ void join_pairs_tile(const PairArgs& A) {
                     if (__shfl_sync(0xffffffffu, in32, o + step - 1) <= t) o += step;
                 const uint32_t y = __shfl_sync(0xffffffffu, x, o), first = __shfl_sync(0xffffffffu, ex32, o);
                 const unsigned long long p = pos + t;
-                if (t < tot && p < cap) {
+                if (t < writes) {
                     __stcs(A.out_build + p, y & kJpRow ? (y == kJpNone ? -1 : static_cast<int32_t>(y & ~kJpRow))
                                                        : static_cast<int32_t>(__ldg(&A.T.bidx[y + (t - first)])));
                     __stcs(A.out_probe + p, static_cast<int32_t>(r0 - lane + kWarp * j + o));
@@ -406,6 +413,14 @@ static __device__ __forceinline__ void join_pairs_tile(const PairArgs& A) {
         }
         pos += tot;
     }
+}
+
+// Rows per lane: a tile is a block's, so an input of few rows takes fewer of
+// them, to spread over the SMs (and its rows over the warps that write the
+// pairs of long runs).
+inline int jp_rows(long long n, long long sms) {
+    const long long one = kJpMinBlocks * sms * kJpThreads;  // rows that fill the chip at one per lane
+    return n <= one ? 1 : (n <= 4 * one ? 4 : kJpRows);
 }
 
 }  // namespace tqp
