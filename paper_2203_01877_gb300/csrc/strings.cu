@@ -212,18 +212,20 @@ __global__ void __launch_bounds__(kStrThreads) k_str_prepass(const __grid_consta
 // is bound by integer issue. Here a lane holds its string's 32-bit words; a
 // segment of a LIKE pattern is a list of 4-byte (value, mask) chunks (`_`: mask
 // 0), its match positions are one 32-bit mask -- the chunk compared with the
-// four-byte window at every position, later chunks ANDed in at their offset --
-// and the segments are placed leftmost-first with bit operations. IN compares
+// four-byte window at every position, later chunks ANDed in at their offset; one
+// or two bytes: the positions of each byte -- and the segments are placed leftmost-first with bit operations. IN compares
 // whole words against each of a short list. Still bound by issue (63% of the
 // slots, 333 warp instructions per 32 strings of 24 bytes before the length was
-// found with one bit scan). 20M rows, `%xy%` and a price bound: 477 -> 292 us;
-// a prefix 311 -> 206, a suffix 317 -> 222, eight IN values 692 -> 275. Longer lists are searched by the general
-// form, and patterns of more segments or wider strings matched by it.
+// found with one bit scan). 20M rows, `%xy%` and a price bound: 477 -> 277 us; a
+// prefix 311 -> 206, a suffix 317 -> 222, eight IN values 692 -> 275. Middle
+// segments of one byte, 4M rows of 24 bytes, `a%b%c%d%e%f`: byte-wise 129, with
+// windows 156, byte by byte 121. Longer lists are searched by the general form,
+// and patterns of more segments or wider strings matched by it.
 constexpr int kSfThreads = 256;
 constexpr int kSfMinBlocks = 4;
 constexpr int kSfMaxWords = 8;
 constexpr int kSfSegs = 8;           // LIKE segments
-constexpr int kSfValues = 32;        // IN values
+constexpr int kSfNumbers = 10;       // values of a numeric IN list; of a string one: sf_values()
 constexpr int kSfWords = 1024;       // program words of a launch
 
 struct StrFastPred {
@@ -248,10 +250,32 @@ struct StrFast {
     uint32_t words[kSfWords];
 };
 
+// The string's bytes equal to c: bit p for byte p. Seven instructions per word: a
+// byte of x is zero iff neither its low seven bits carry into bit 7 nor bit 7 is
+// set; the four bits are gathered at the top with one multiplication.
+template <int NW>
+__device__ __forceinline__ uint32_t sf_equal(const uint32_t (&w)[NW], uint32_t c) {
+    const uint32_t all = c * 0x01010101u;
+    uint32_t E = 0;
+#pragma unroll
+    for (int i = 0; i < NW; ++i) {
+        const uint32_t x = w[i] ^ all;
+        const uint32_t z = ~(((x & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | x | 0x7F7F7F7Fu);
+        E = (E >> 4) | ((z * 0x00204081u) & 0xF0000000u);
+    }
+    return E >> (32 - 4 * NW);
+}
+
 // Match positions of a segment of `len` bytes (len >= 1): bit p set when it matches at byte p.
 template <int NW>
 __device__ __forceinline__ uint32_t sf_find(const uint32_t (&w)[NW], const uint32_t* chunk, int len) {
     uint32_t M = ~0u;
+    if (len <= 2) {  // byte by byte: a window at every position is 20 instructions per word
+        const uint32_t v = chunk[0], m = chunk[1];
+        if (m & 0xFFu) M = sf_equal<NW>(w, v & 0xFFu);
+        if (m & 0xFF00u) M &= sf_equal<NW>(w, (v >> 8) & 0xFFu) >> 1;
+        return M;
+    }
     for (int c = 0; 4 * c < len && M; ++c) {
         const uint32_t v = chunk[2 * c], m = chunk[2 * c + 1];
         uint32_t hit = 0;
@@ -448,6 +472,13 @@ __global__ void __launch_bounds__(kSfThreads, kSfMinBlocks) k_str_fast(const __g
     }
 }
 
+// The longest IN list that is compared value by value; a longer one is searched
+// by the general form. A value costs its words, a string that goes through shared
+// memory starts behind. 4M rows, general / here, us: 12 bytes, 16 values 83 / 80,
+// 24 values 86 / 89; 24 bytes, 10 values 88 / 77, 16 values 92 / 97; 25 bytes, 4
+// values 80 / 77, 6 values 82 / 87; int32, 10 values 56 / 56, 12 values 55 / 58.
+static int sf_values(int nw, bool stage) { return stage ? std::min(14, 36 / nw) : 64 / nw; }
+
 // The launch above from the general one; false outside its shapes.
 static bool lower_str_fast(const StrLaunch& L, StrFast* F, int* words_per_string) {
     F->n = L.n;
@@ -470,7 +501,7 @@ static bool lower_str_fast(const StrLaunch& L, StrFast* F, int* words_per_string
             stage = stage || q.width % 4 != 0;
         }
         if (q.op == TQP_IN) {
-            if (q.count > kSfValues) return false;
+            if (q.type != TQP_CHAR && q.count > kSfNumbers) return false;
             const int bytes = q.type == TQP_CHAR ? q.width : 8;
             for (int v = 0; v < q.count; ++v)
                 for (int b = 0; b < bytes; b += 4) {
@@ -514,7 +545,10 @@ static bool lower_str_fast(const StrLaunch& L, StrFast* F, int* words_per_string
     if (used > kSfWords) return false;
     F->nwords = used;
     F->stage_bytes = stage ? (kWarp * maxw + 4 + 15) / 16 * 16 : 0;
-    *words_per_string = maxw <= 8 ? 2 : (maxw <= 16 ? 4 : (maxw <= 24 ? 6 : 8));
+    const int nw = maxw <= 8 ? 2 : (maxw <= 16 ? 4 : (maxw <= 24 ? 6 : 8));
+    *words_per_string = nw;
+    for (int k = 0; k < L.npred; ++k)
+        if (L.p[k].op == TQP_IN && L.p[k].type == TQP_CHAR && L.p[k].count > sf_values(nw, stage)) return false;
     return true;
 }
 
