@@ -519,7 +519,6 @@ def make_plan(fact: TableRef, preds=(), dim: TableRef | None = None, fact_fk=0, 
     pa = make_preds(preds, fact)
     for i in range(len(preds)):
         p.preds[i] = pa[i]
-    p._keep = pa._keep
     p.npreds = len(preds)
     p.emit_row_ids = int(bool(emit_row_ids))
     p.dim = C.pointer(dim.t) if dim is not None else None
@@ -538,7 +537,7 @@ def make_plan(fact: TableRef, preds=(), dim: TableRef | None = None, fact_fk=0, 
     p.max_groups = int(max_groups)
     p.join_kind = JOIN_KINDS[join_kind] if isinstance(join_kind, str) else int(join_kind)
     p.prepared = prepared.h if prepared is not None else None
-    p._keep = (fact, dim, prepared)  # keep the tables' C structs alive
+    p._keep = (fact, dim, prepared, pa._keep)  # the tables' C structs, the predicates' values and patterns
     return p
 
 
