@@ -67,6 +67,13 @@ __global__ void __launch_bounds__(kFdThreads, kFdMinBlocks) k_filter_direct(cons
 }
 constexpr int kFilterVariant = 1;
 
+// The form of a filter: the tuner's choice for calls of tqp_filter; in a plan or
+// a shared scan the tuned variant is that operator's.
+static int filter_variant(const tqp_ctx* ctx) {
+    if (ctx->force_variant >= 0) return ctx->force_variant;
+    return strncmp(ctx->cur_key, "filter ", 7) == 0 ? tuned_variant(ctx, kFilterVariant) : kFilterVariant;
+}
+
 __global__ void __launch_bounds__(kCompactThreads) k_compact(const uint32_t* __restrict__ mask,
                                                              const uint32_t* __restrict__ block_tot, long long n,
                                                              int32_t* __restrict__ row_ids, long long capacity) {
@@ -238,7 +245,7 @@ tqp_status launch_filter(tqp_ctx* ctx, const tqp_table* t, const tqp_pred* preds
     }
     const bool ids = d_row_ids != nullptr;
     FilterDirectArgs D;
-    if (!force && !user_shape(ctx) && tuned_variant(ctx, kFilterVariant) == 1 && lower_filter_direct(t, A, &D)) {
+    if (!force && !user_shape(ctx) && filter_variant(ctx) == 1 && lower_filter_direct(t, A, &D)) {
         lay = filter_scratch_layout(n, (n + kFdStep - 1) / kFdStep * kFdStep, ids);
         void* scratch = arena_alloc(ctx, lay.bytes);
         if (!scratch) return arena_oom(ctx, lay.bytes);

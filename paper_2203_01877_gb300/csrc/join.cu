@@ -713,5 +713,5 @@ extern "C" tqp_status tqp_hash_join_kind(tqp_ctx* ctx, const tqp_table* build, i
         return launch_hash_join(ctx, build, build_key, probe, probe_key, join_kind, d_build_idx, d_probe_idx,
                                 capacity, d_count, st);
     };
-    return tuned(ctx, key, st, kTuneHt | kTuneVariant, run);
+    return tuned(ctx, key, st, kTuneHt | kTuneVariant | kTuneV0Shapeless, run);  // (0: joinpairs.cuh)
 }
