@@ -191,8 +191,12 @@ TQP_API size_t tqp_ctx_arena_bytes(const tqp_ctx* ctx);
 
 /* Override the scan launch shape used by this context's calls: rows per
  * tile (a multiple of 1024, at most 8192), pipeline stages (2..4) and CTAs
- * per SM (1..2).  All zero restores the built-in choice.  Used by the
- * autotuner and by tuning sweeps; results never depend on it. */
+ * per SM (1..2).  All zero restores the built-in choice.  Operators that also
+ * have a form without a staged scan (filters, pair joins, joined aggregations,
+ * group-bys of many groups) take their staged form under an override, so that
+ * the shape has an effect; it is often the slower one.  A shared scan narrows a
+ * shape that leaves no room for its row queues.  Used by tuning sweeps; results
+ * never depend on it. */
 TQP_API tqp_status tqp_ctx_set_tuning(tqp_ctx* ctx, int32_t tile_rows, int32_t stages, int32_t ctas_per_sm);
 
 /* Force the algorithm of operators that have two, for this context's calls
@@ -202,14 +206,17 @@ TQP_API tqp_status tqp_ctx_set_tuning(tqp_ctx* ctx, int32_t tile_rows, int32_t s
  *     Algorithm 1: the build keys are radix-sorted with their rows and each
  *     probe key is bucketized into them);
  *   tqp_filter: 0 = the staged scan, 1 = plain vector loads (one to four
- *     conditions, a sum that is a product of two affine factors, or none);
+ *     conditions, of them at most two on int64, three on int32 and two on uint8
+ *     columns; a sum that is a product of two affine factors, or none; other
+ *     filters take the staged scan);
  *   grouped join plans with at least 2^20 fact rows: 0 = the radix-partitioned
  *     aggregation (the probe side partitioned by group, each partition
  *     aggregated in shared memory), 1 = the fused probe (every joined row
  *     added to its key's or group's accumulators with L2 reductions).
  * -1 restores the default (the autotuner's choice, which times both; else 0 for
- * tqp_hash_join, 1 for tqp_filter and 1, the fused probe, for grouped join
- * plans).
+ * tqp_hash_join, 1, the fused probe, for grouped join plans and 1 for
+ * tqp_filter, but for a few shapes of counts and row ids without a sum that the
+ * staged scan streams faster from 2^23 rows on).
  * Errors: TQP_ERR_INVALID_ARG. */
 TQP_API tqp_status tqp_ctx_set_variant(tqp_ctx* ctx, int32_t variant);
 

@@ -58,20 +58,33 @@ __global__ void __launch_bounds__(kEngineThreads, 2) k_filter(const __grid_const
     run_engine(A.G, A.ctl, body, smem, args_bytes<FilterArgs>());
 }
 
-// The built-in form (variant 1): plain vector loads (filterdirect.cuh). The staged
-// scan (variant 0) keeps what falls outside its shapes -- no condition or more
-// than four, sums that are not products of two affine factors -- and launch
-// shapes set by the caller.
+// Variant 1, the built-in form but for plain_loads_win: plain vector loads
+// (filterdirect.cuh). The staged scan (variant 0) keeps what falls outside its
+// shapes -- no condition, more than four, more than two on 64-bit columns, three
+// on 32-bit or two on 8-bit ones, sums that are not products of two affine
+// factors -- and launch shapes set by the caller.
 __global__ void __launch_bounds__(kFdThreads, kFdMinBlocks) k_filter_direct(const __grid_constant__ FilterDirectArgs A) {
     filter_direct_block(A, blockIdx.x, gridDim.x);
 }
-constexpr int kFilterVariant = 1;
 
-// The form of a filter: the tuner's choice for calls of tqp_filter; in a plan or
-// a shared scan the tuned variant is that operator's.
+// The form of a filter, -1 for the built-in choice: the tuner's for calls of
+// tqp_filter; in a plan or a shared scan the tuned variant is that operator's.
 static int filter_variant(const tqp_ctx* ctx) {
     if (ctx->force_variant >= 0) return ctx->force_variant;
-    return strncmp(ctx->cur_key, "filter ", 7) == 0 ? tuned_variant(ctx, kFilterVariant) : kFilterVariant;
+    return strncmp(ctx->cur_key, "filter ", 7) == 0 ? tuned_variant(ctx, -1) : -1;
+}
+
+// Built in: the plain loads, but for two 64-bit conditions, or one beside two
+// narrower ones (not both of 8 bits), without a sum, from 2^23 rows to 2^27. A
+// step of these has too few bytes in flight for what it waits, and the staged
+// scan streams them faster: 24M rows, counts only, us staged / plain loads: two
+// int64 87 / 100 (30M rows), int64 and two int32 1.12 times, int64, int32 and
+// uint8 86 / 91, with another int32 98 / 106; at 4M rows plain loads take 0.90 of
+// the staged time, at 200M 0.94 to 1.04.
+static bool plain_loads_win(const FilterDirectArgs& D) {
+    if (D.has_sum || D.n < (1LL << 23) || D.n >= (1LL << 27)) return true;
+    const int narrow = D.nword + D.nbyte;
+    return !((D.nwide == 2 && narrow == 0) || (D.nwide == 1 && narrow >= 2 && D.nword >= 1));
 }
 
 __global__ void __launch_bounds__(kCompactThreads) k_compact(const uint32_t* __restrict__ mask,
@@ -245,7 +258,9 @@ tqp_status launch_filter(tqp_ctx* ctx, const tqp_table* t, const tqp_pred* preds
     }
     const bool ids = d_row_ids != nullptr;
     FilterDirectArgs D;
-    if (!force && !user_shape(ctx) && filter_variant(ctx) == 1 && lower_filter_direct(t, A, &D)) {
+    const int variant = filter_variant(ctx);
+    const bool plain = !force && !user_shape(ctx) && variant != 0 && lower_filter_direct(t, A, &D);
+    auto run_plain = [&]() -> tqp_status {
         lay = filter_scratch_layout(n, (n + kFdStep - 1) / kFdStep * kFdStep, ids);
         void* scratch = arena_alloc(ctx, lay.bytes);
         if (!scratch) return arena_oom(ctx, lay.bytes);
@@ -255,9 +270,15 @@ tqp_status launch_filter(tqp_ctx* ctx, const tqp_table* t, const tqp_pred* preds
         A.G.n = n;
         return launch_filter_with(A, grid, smem, lay, scratch, ctx->d_err, ctx->wait_cap, d_row_ids, capacity, d_count,
                                   d_sum, stream, &D, static_cast<int>(g));
-    }
+    };
+    if (plain && (variant == 1 || plain_loads_win(D))) return run_plain();
     TQP_TRY(shape_filter(ctx, t, staged, bpr, ids, force, &A, &smem, &grid, &lay));
+    const size_t used = ctx->used;
     void* scratch = arena_alloc(ctx, lay.bytes);
+    if (!scratch && plain) {  // (its mask is not rounded up to whole tiles)
+        ctx->used = used;
+        return run_plain();
+    }
     if (!scratch) return arena_oom(ctx, lay.bytes);
     return launch_filter_with(A, grid, smem, lay, scratch, ctx->d_err, ctx->wait_cap, d_row_ids, capacity, d_count,
                               d_sum, stream);
