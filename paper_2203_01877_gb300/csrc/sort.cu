@@ -21,8 +21,10 @@ constexpr int kSortItems = 16;                          // per thread
 constexpr int kSortTile = kSortThreads * kSortItems;    // 4096
 constexpr int kSortSlice = kSortTile / kSortWarps;      // 512 per warp
 constexpr int kSortScanThreads = 1024;                  // of a scan of its own
-constexpr int kSortBlocksPerSm = 8;
-constexpr long long kSortOneLaunch = 1LL << 22;         // items up to which the passes share a launch
+constexpr int kSortFewBlocks = 4;                       // per SM, at 64 registers: what waits least at the barriers
+constexpr int kSortManyBlocks = 8;                      // at 32 registers, above kSortOneLaunch: 4M rows 879 us, with 4 895
+constexpr long long kSortGraphItems = 1LL << 19;        // items up to which a captured sort takes a launch per step
+constexpr long long kSortOneLaunch = 3LL << 20;         // items up to which the passes share a launch
 
 // A pass of a shared launch reads what an earlier one wrote from other SMs (L2
 // only); a launch of its own may read through L1, which the second read of a
@@ -155,7 +157,8 @@ __device__ __forceinline__ void rs_downsweep(const uint64_t* kin, const uint32_t
 // All passes in one cooperative launch. An empty input (a build side of unique
 // keys) costs this one launch instead of three per pass: 12 to 16 launches of
 // about 2 us each.
-__global__ void __launch_bounds__(kSortThreads, kSortBlocksPerSm) k_rs_sort(uint64_t* k0, uint32_t* v0, uint64_t* k1,
+template <int kBlocksPerSm>
+__global__ void __launch_bounds__(kSortThreads, kBlocksPerSm) k_rs_sort(uint64_t* k0, uint32_t* v0, uint64_t* k1,
                                                                             uint32_t* v1, long long* n_ptr, int begin_bit,
                                                                             int end_bit, unsigned long long* digit_tot,
                                                                             uint32_t* hist, long long ntiles,
@@ -229,7 +232,12 @@ tqp_status radix_sort_pairs(const tqp_ctx* ctx, uint64_t* k0, uint32_t* v0, uint
     unsigned long long* digit_tot = static_cast<unsigned long long*>(scratch);
     unsigned int* bar = reinterpret_cast<unsigned int*>(digit_tot + 256);  // (one zeroing for both)
     uint32_t* hist = reinterpret_cast<uint32_t*>(digit_tot + 256 + 16);
-    if (n_max > kSortOneLaunch && !optional) {
+    // A captured launch costs less than a barrier: a graph of a MIN plan over 1000
+    // rows takes 141 us with one launch, 133 with all of them; over 2M 450 and 465.
+    cudaStreamCaptureStatus captured = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &captured) != cudaSuccess) cudaGetLastError();
+    const bool steps = n_max > kSortOneLaunch || (captured == cudaStreamCaptureStatusActive && n_max <= kSortGraphItems);
+    if (steps && !optional) {
         const unsigned blocks = static_cast<unsigned>(ntiles);
         for (int shift = begin_bit; shift < end_bit; shift += 8) {
             TQP_CUDA(cudaMemsetAsync(digit_tot, 0, 256 * sizeof(unsigned long long), stream));
@@ -244,13 +252,16 @@ tqp_status radix_sort_pairs(const tqp_ctx* ctx, uint64_t* k0, uint32_t* v0, uint
         return TQP_OK;
     }
     TQP_CUDA(cudaMemsetAsync(digit_tot, 0, 256 * sizeof(unsigned long long) + sizeof(unsigned int), stream));
-    const int most = std::min(resident_blocks(ctx->device, reinterpret_cast<const void*>(k_rs_sort), kSortThreads, 0),
-                              kSortBlocksPerSm) * ctx->num_sms;
+    const bool few = n_max <= kSortOneLaunch;
+    const void* kern = few ? reinterpret_cast<const void*>(k_rs_sort<kSortFewBlocks>)
+                           : reinterpret_cast<const void*>(k_rs_sort<kSortManyBlocks>);
+    const int most = std::min(resident_blocks(ctx->device, kern, kSortThreads, 0),
+                              few ? kSortFewBlocks : kSortManyBlocks) * ctx->num_sms;
     const int grid = static_cast<int>(std::min<long long>(most, std::max<long long>(ntiles, 32)));
     int* err = ctx->d_err;
     long long cap = ctx->wait_cap;
     void* args[] = {&k0, &v0, &k1, &v1, &d_n, &begin_bit, &end_bit, &digit_tot, &hist, &ntiles, &bar, &err, &cap};
-    TQP_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_rs_sort), dim3(grid), dim3(kSortThreads), args, 0,
+    TQP_CUDA(cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(kSortThreads), args, 0,
                                          stream));
     *result_in_1 = ((end_bit - begin_bit + 7) / 8) % 2 != 0;
     return TQP_OK;

@@ -1,4 +1,4 @@
-"""GPU: the radix sort on both sides of the size where its passes leave the shared launch (2^22 items), through the
+"""GPU: the radix sort on both sides of the size where its passes leave the shared launch (3 * 2^20 items), through the
 sort-based group-by (64-bit keys: eight passes) and the sort-based join (repeated build keys in canonical order)."""
 import numpy as np
 import pytest
@@ -19,7 +19,7 @@ def ctx():
     c.close()
 
 
-@pytest.mark.parametrize("n", [(1 << 22) - 1, 1 << 22, (1 << 22) + 1, (1 << 22) + 4097])
+@pytest.mark.parametrize("n", [(3 << 20) - 1, 3 << 20, (3 << 20) + 1, (3 << 20) + 4097])
 def test_group_by(ctx, n):
     rng = np.random.default_rng(n)
     pool = rng.integers(-2**62, 2**62, 700)
@@ -27,7 +27,7 @@ def test_group_by(ctx, n):
     check(ctx, cols, [(1, "gt", -900)], [0], [("sum", [("col", 1)]), ("count", None)], capacity=700)
 
 
-@pytest.mark.parametrize("n", [1 << 22, (1 << 22) + 4097])
+@pytest.mark.parametrize("n", [3 << 20, (3 << 20) + 4097])
 def test_join(ctx, n):
     import torch
     import paper_2203_01877_gb300 as tqp
