@@ -277,8 +277,9 @@ __device__ __forceinline__ uint64_t gr_key(const GroupRangePlan* plan, const Gro
     return key;
 }
 
-// The groups of at most kSmallCap + 1 entries, by one block of kFinThreads.
-static __device__ void group_rows_small(const GroupRangePlan* plan, const GroupSpec& S, const GroupOut& O) {
+// The groups of at most kSmallCap + 1 entries, by one block of kFinThreads. (A
+// call: in line it costs the hash path's output 1 us.)
+static __device__ __noinline__ void group_rows_small(const GroupRangePlan* plan, const GroupSpec& S, const GroupOut& O) {
     constexpr int kPer = kSmallCap / kFinThreads + 1;
     __shared__ uint32_t wcnt[kFinThreads / kWarp];
     const long long D = plan->entries;
