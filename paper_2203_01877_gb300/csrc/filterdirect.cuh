@@ -244,9 +244,9 @@ static __device__ __noinline__ uint32_t fd_tail(const FilterDirectArgs& A, long 
 }
 
 template <int NW, int NN>
-__device__ __forceinline__ void fd_loop(const FilterDirectArgs& A, long long vb, long long vg, int lane, int w, FdTotals& T) {
-    __shared__ uint32_t queue[kFdThreads / kWarp][kFdQueue];
-    FdQueue Q{queue[w], 0};
+__device__ __forceinline__ void fd_loop(const FilterDirectArgs& A, long long vb, long long vg, int lane, int w,
+                                        uint32_t* queue, FdTotals& T) {
+    FdQueue Q{queue, 0};
     const long long seg = static_cast<long long>(A.steps) * kFdStep;  // a divisor of kCompactRows
     const long long stride = vg * (kFdThreads / kWarp) * seg;
     for (long long s0 = (vb * (kFdThreads / kWarp) + w) * seg; s0 < A.n; s0 += stride) {
@@ -274,20 +274,21 @@ __device__ __forceinline__ void fd_loop(const FilterDirectArgs& A, long long vb,
 // Block vb of vg working on this filter.
 static __device__ __forceinline__ void filter_direct_block(const FilterDirectArgs& A, long long vb, long long vg) {
     __shared__ unsigned long long red[2][kFdThreads / kWarp];
+    __shared__ uint32_t queue[kFdThreads / kWarp][kFdQueue];  // (one for all the forms of fd_loop)
     const int lane = threadIdx.x % kWarp, w = threadIdx.x / kWarp;
     FdTotals T;
     switch (A.nwide * (kFdWord + 1) + A.nword) {
-        case 0: fd_loop<0, 0>(A, vb, vg, lane, w, T); break;
-        case 1: fd_loop<0, 1>(A, vb, vg, lane, w, T); break;
-        case 2: fd_loop<0, 2>(A, vb, vg, lane, w, T); break;
-        case 3: fd_loop<0, 3>(A, vb, vg, lane, w, T); break;
-        case 4: fd_loop<1, 0>(A, vb, vg, lane, w, T); break;
-        case 5: fd_loop<1, 1>(A, vb, vg, lane, w, T); break;
-        case 6: fd_loop<1, 2>(A, vb, vg, lane, w, T); break;
-        case 7: fd_loop<1, 3>(A, vb, vg, lane, w, T); break;
-        case 8: fd_loop<2, 0>(A, vb, vg, lane, w, T); break;
-        case 9: fd_loop<2, 1>(A, vb, vg, lane, w, T); break;
-        default: fd_loop<2, 2>(A, vb, vg, lane, w, T); break;  // (at most kFdConds in all)
+        case 0: fd_loop<0, 0>(A, vb, vg, lane, w, queue[w], T); break;
+        case 1: fd_loop<0, 1>(A, vb, vg, lane, w, queue[w], T); break;
+        case 2: fd_loop<0, 2>(A, vb, vg, lane, w, queue[w], T); break;
+        case 3: fd_loop<0, 3>(A, vb, vg, lane, w, queue[w], T); break;
+        case 4: fd_loop<1, 0>(A, vb, vg, lane, w, queue[w], T); break;
+        case 5: fd_loop<1, 1>(A, vb, vg, lane, w, queue[w], T); break;
+        case 6: fd_loop<1, 2>(A, vb, vg, lane, w, queue[w], T); break;
+        case 7: fd_loop<1, 3>(A, vb, vg, lane, w, queue[w], T); break;
+        case 8: fd_loop<2, 0>(A, vb, vg, lane, w, queue[w], T); break;
+        case 9: fd_loop<2, 1>(A, vb, vg, lane, w, queue[w], T); break;
+        default: fd_loop<2, 2>(A, vb, vg, lane, w, queue[w], T); break;  // (at most kFdConds in all)
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) T.sum += __shfl_xor_sync(0xffffffffu, T.sum, o);
