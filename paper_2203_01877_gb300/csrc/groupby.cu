@@ -30,7 +30,7 @@ namespace tqp {
 
 tqp_status radix_sort_pairs(const tqp_ctx* ctx, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, long long* d_n,
                             long long n_max, int begin_bit, int end_bit, void* scratch, cudaStream_t stream,
-                            bool* result_in_1, bool optional = false);
+                            bool* result_in_1, SortFill fill = kSortAll);
 size_t radix_sort_scratch(long long n_max);
 
 
@@ -285,7 +285,7 @@ tqp_status group_finalize(tqp_ctx* ctx, const GroupSpec& S, const GroupOut& O, c
     k_groupby_collect<<<blocks, threads, 0, stream>>>(S, k0, v0, d_n, rp);
     bool in1 = false;
     const int end_bit = (S.width + 7) / 8 * 8;
-    TQP_TRY(radix_sort_pairs(ctx, k0, v0, k1, v1, d_n, nmax, 0, end_bit, rs, stream, &in1));
+    TQP_TRY(radix_sort_pairs(ctx, k0, v0, k1, v1, d_n, nmax, 0, end_bit, rs, stream, &in1, kSortSome));
     const int eblocks = static_cast<int>(
         std::max<long long>(1, std::min<long long>((std::min(nmax, rp ? nmax : O.capacity) + threads - 1) / threads,
                                                    ctx->num_sms * 8LL)));

@@ -175,6 +175,11 @@ void expr_col_ids(const tqp_expr* e, std::vector<int>& cols);
 // floor(log2(max(n, 1))): the row-count part of a shape class.
 int rows_class(long long n);
 
+// What is known of a radix sort's items before it runs: n_max of them are there
+// (kSortAll), some part (kSortSome: a group table's), or usually none (kSortRarely:
+// the rows of a join's repeated build keys).
+enum SortFill { kSortAll, kSortSome, kSortRarely };
+
 // Resident blocks per SM of a kernel (1 when the driver gives no answer).
 int resident_blocks(int device, const void* kernel, int threads, size_t smem);
 // Persistent grid size for an engine kernel.

@@ -31,7 +31,7 @@ namespace tqp {
 
 tqp_status radix_sort_pairs(const tqp_ctx* ctx, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, long long* d_n,
                             long long n_max, int begin_bit, int end_bit, void* scratch, cudaStream_t stream,
-                            bool* result_in_1, bool optional = false);
+                            bool* result_in_1, SortFill fill = kSortAll);
 size_t radix_sort_scratch(long long n_max);
 
 __global__ void k_ht_init(JoinHT H) {
@@ -598,7 +598,7 @@ static tqp_status launch_join_pairs(tqp_ctx* ctx, const tqp_table* build, int32_
         int bits = 1;
         while ((1LL << bits) <= T.cap) ++bits;
         bool in1 = false;
-        TQP_TRY(radix_sort_pairs(ctx, k0, v0, k1, v1, n_sort, nb, 0, (bits + 7) / 8 * 8, rs, stream, &in1, true));
+        TQP_TRY(radix_sort_pairs(ctx, k0, v0, k1, v1, n_sort, nb, 0, (bits + 7) / 8 * 8, rs, stream, &in1, kSortRarely));
         const uint64_t* sk = in1 ? k1 : k0;
         uint32_t* rlen = reinterpret_cast<uint32_t*>(in1 ? k0 : k1);  // (the sort's other key buffer)
         T.bidx = in1 ? v1 : v0;

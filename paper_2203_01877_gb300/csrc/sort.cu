@@ -10,7 +10,7 @@
 //             peers and per-warp digit bases, so equal digits keep input
 //             order (stability) and stores land in ascending position order.
 // The item count lives in device memory (it is usually produced by a kernel);
-// blocks stride over the tiles of an upper bound, and tiles past the count are skipped.
+// buffers and launches are sized for an upper bound, the work follows the count.
 #include "host.h"
 
 namespace tqp {
@@ -21,10 +21,17 @@ constexpr int kSortItems = 16;                          // per thread
 constexpr int kSortTile = kSortThreads * kSortItems;    // 4096
 constexpr int kSortSlice = kSortTile / kSortWarps;      // 512 per warp
 constexpr int kSortScanThreads = 1024;                  // of a scan of its own
-constexpr int kSortFewBlocks = 4;                       // per SM, at 64 registers: what waits least at the barriers
-constexpr int kSortManyBlocks = 8;                      // at 32 registers, above kSortOneLaunch: 4M rows 879 us, with 4 895
+// Blocks per SM of the shared launch: four at 64 registers wait least at the
+// barriers; eight at 32 registers sort more items faster (8M build rows, each
+// four times: 1001 us, with four 1088; 1.5M groups in a table of 4M: 1175, with
+// four 1065).
+constexpr int kSortFewBlocks = 4;
+constexpr int kSortManyBlocks = 8;
 constexpr long long kSortGraphItems = 1LL << 19;        // items up to which a captured sort takes a launch per step
 constexpr long long kSortOneLaunch = 3LL << 20;         // items up to which the passes share a launch
+
+// Tiles of the items there are (the buffers and launches are sized for an upper bound).
+__device__ __forceinline__ long long rs_tiles(long long n) { return (n + kSortTile - 1) / kSortTile; }
 
 // A pass of a shared launch reads what an earlier one wrote from other SMs (L2
 // only); a launch of its own may read through L1, which the second read of a
@@ -161,12 +168,13 @@ template <int kBlocksPerSm>
 __global__ void __launch_bounds__(kSortThreads, kBlocksPerSm) k_rs_sort(uint64_t* k0, uint32_t* v0, uint64_t* k1,
                                                                             uint32_t* v1, long long* n_ptr, int begin_bit,
                                                                             int end_bit, unsigned long long* digit_tot,
-                                                                            uint32_t* hist, long long ntiles,
-                                                                            unsigned int* bar, int* err, long long wait_cap) {
+                                                                            uint32_t* hist, unsigned int* bar, int* err,
+                                                                            long long wait_cap) {
     __shared__ uint32_t wcnt[kSortWarps][256];
     __shared__ unsigned long long wsum[kSortWarps];
     const long long n = *n_ptr;
     if (n == 0) return;
+    const long long ntiles = rs_tiles(n);
     unsigned int arrivals = 0;
     bool ok = true;
     for (int shift = begin_bit; ok && shift < end_bit; shift += 8) {
@@ -193,23 +201,24 @@ __global__ void __launch_bounds__(kSortThreads, kBlocksPerSm) k_rs_sort(uint64_t
 // launch / this): 1M rows 278 / 306, 2M 450 / 472, 4M 879 / 883, 8M 1924 / 1893,
 // 60M rows of 64-bit keys 19060 / 18371; a join's 8M unique build rows 183 / 261.
 __global__ void __launch_bounds__(kSortThreads) k_rs_upsweep(const uint64_t* keys, const long long* n_ptr, int shift,
-                                                             uint32_t* hist, long long ntiles,
-                                                             unsigned long long* digit_tot) {
+                                                             uint32_t* hist, unsigned long long* digit_tot) {
     __shared__ uint32_t cnt[256];
-    rs_upsweep<false>(keys, *n_ptr, shift, hist, ntiles, digit_tot, cnt);
+    const long long n = *n_ptr;
+    rs_upsweep<false>(keys, n, shift, hist, rs_tiles(n), digit_tot, cnt);
 }
 
-__global__ void __launch_bounds__(kSortScanThreads) k_rs_scan(uint32_t* hist, long long ntiles,
+__global__ void __launch_bounds__(kSortScanThreads) k_rs_scan(uint32_t* hist, const long long* n_ptr,
                                                               const unsigned long long* digit_tot) {
     __shared__ unsigned long long wsum[kSortScanThreads / kWarp];
-    rs_scan<false, kSortScanThreads>(hist, ntiles, digit_tot, wsum);
+    rs_scan<false, kSortScanThreads>(hist, rs_tiles(*n_ptr), digit_tot, wsum);
 }
 
 __global__ void __launch_bounds__(kSortThreads) k_rs_downsweep(const uint64_t* kin, const uint32_t* vin, uint64_t* kout,
                                                                uint32_t* vout, const long long* n_ptr, int shift,
-                                                               const uint32_t* hist, long long ntiles) {
+                                                               const uint32_t* hist) {
     __shared__ uint32_t wcnt[kSortWarps][256];
-    rs_downsweep<false>(kin, vin, kout, vout, *n_ptr, shift, hist, ntiles, wcnt);
+    const long long n = *n_ptr;
+    rs_downsweep<false>(kin, vin, kout, vout, n, shift, hist, rs_tiles(n), wcnt);
 }
 
 // Scratch needed by radix_sort_pairs for up to n_max items.
@@ -222,10 +231,10 @@ size_t radix_sort_scratch(long long n_max) {
 // input; (k1, v1) are a second buffer of the same size.  *result_in_1 tells
 // which buffer holds the sorted output.  *d_n is 0 afterwards when a wait of the
 // sort expired, so kernels that read the output take the count from there.
-// `optional`: there is usually nothing to sort.
+// `fill`: how far the items are known to reach n_max.
 tqp_status radix_sort_pairs(const tqp_ctx* ctx, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, long long* d_n,
                             long long n_max, int begin_bit, int end_bit, void* scratch, cudaStream_t stream,
-                            bool* result_in_1, bool optional) {
+                            bool* result_in_1, SortFill fill) {
     *result_in_1 = false;
     if (n_max <= 0 || end_bit <= begin_bit) return TQP_OK;
     long long ntiles = (n_max + kSortTile - 1) / kSortTile;
@@ -236,14 +245,14 @@ tqp_status radix_sort_pairs(const tqp_ctx* ctx, uint64_t* k0, uint32_t* v0, uint
     // rows takes 141 us with one launch, 133 with all of them; over 2M 450 and 465.
     cudaStreamCaptureStatus captured = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(stream, &captured) != cudaSuccess) cudaGetLastError();
-    const bool steps = n_max > kSortOneLaunch || (captured == cudaStreamCaptureStatusActive && n_max <= kSortGraphItems);
-    if (steps && !optional) {
+    const bool graph = captured == cudaStreamCaptureStatusActive && n_max <= kSortGraphItems;
+    if (fill == kSortAll ? n_max > kSortOneLaunch || graph : fill == kSortSome && graph) {
         const unsigned blocks = static_cast<unsigned>(ntiles);
         for (int shift = begin_bit; shift < end_bit; shift += 8) {
             TQP_CUDA(cudaMemsetAsync(digit_tot, 0, 256 * sizeof(unsigned long long), stream));
-            k_rs_upsweep<<<blocks, kSortThreads, 0, stream>>>(k0, d_n, shift, hist, ntiles, digit_tot);
-            k_rs_scan<<<256, kSortScanThreads, 0, stream>>>(hist, ntiles, digit_tot);
-            k_rs_downsweep<<<blocks, kSortThreads, 0, stream>>>(k0, v0, k1, v1, d_n, shift, hist, ntiles);
+            k_rs_upsweep<<<blocks, kSortThreads, 0, stream>>>(k0, d_n, shift, hist, digit_tot);
+            k_rs_scan<<<256, kSortScanThreads, 0, stream>>>(hist, d_n, digit_tot);
+            k_rs_downsweep<<<blocks, kSortThreads, 0, stream>>>(k0, v0, k1, v1, d_n, shift, hist);
             TQP_CUDA(cudaGetLastError());
             std::swap(k0, k1);
             std::swap(v0, v1);
@@ -252,7 +261,7 @@ tqp_status radix_sort_pairs(const tqp_ctx* ctx, uint64_t* k0, uint32_t* v0, uint
         return TQP_OK;
     }
     TQP_CUDA(cudaMemsetAsync(digit_tot, 0, 256 * sizeof(unsigned long long) + sizeof(unsigned int), stream));
-    const bool few = n_max <= kSortOneLaunch;
+    const bool few = fill != kSortRarely;
     const void* kern = few ? reinterpret_cast<const void*>(k_rs_sort<kSortFewBlocks>)
                            : reinterpret_cast<const void*>(k_rs_sort<kSortManyBlocks>);
     const int most = std::min(resident_blocks(ctx->device, kern, kSortThreads, 0),
@@ -260,7 +269,7 @@ tqp_status radix_sort_pairs(const tqp_ctx* ctx, uint64_t* k0, uint32_t* v0, uint
     const int grid = static_cast<int>(std::min<long long>(most, std::max<long long>(ntiles, 32)));
     int* err = ctx->d_err;
     long long cap = ctx->wait_cap;
-    void* args[] = {&k0, &v0, &k1, &v1, &d_n, &begin_bit, &end_bit, &digit_tot, &hist, &ntiles, &bar, &err, &cap};
+    void* args[] = {&k0, &v0, &k1, &v1, &d_n, &begin_bit, &end_bit, &digit_tot, &hist, &bar, &err, &cap};
     TQP_CUDA(cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(kSortThreads), args, 0,
                                          stream));
     *result_in_1 = ((end_bit - begin_bit + 7) / 8) % 2 != 0;

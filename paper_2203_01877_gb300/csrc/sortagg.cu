@@ -22,7 +22,7 @@ namespace tqp {
 
 tqp_status radix_sort_pairs(const tqp_ctx* ctx, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, long long* d_n,
                             long long n_max, int begin_bit, int end_bit, void* scratch, cudaStream_t stream,
-                            bool* result_in_1, bool optional = false);
+                            bool* result_in_1, SortFill fill = kSortAll);
 size_t radix_sort_scratch(long long n_max);
 
 constexpr int kSaThreads = 256;
