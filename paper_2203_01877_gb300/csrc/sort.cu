@@ -244,7 +244,10 @@ tqp_status radix_sort_pairs(const tqp_ctx* ctx, uint64_t* k0, uint32_t* v0, uint
     // A captured launch costs less than a barrier: a graph of a MIN plan over 1000
     // rows takes 141 us with one launch, 133 with all of them; over 2M 450 and 465.
     cudaStreamCaptureStatus captured = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(stream, &captured) != cudaSuccess) cudaGetLastError();
+    if (cudaStreamIsCapturing(stream, &captured) != cudaSuccess) {
+        cudaGetLastError();
+        captured = cudaStreamCaptureStatusNone;
+    }
     const bool graph = captured == cudaStreamCaptureStatusActive && n_max <= kSortGraphItems;
     if (fill == kSortAll ? n_max > kSortOneLaunch || graph : fill == kSortSome && graph) {
         const unsigned blocks = static_cast<unsigned>(ntiles);
