@@ -81,6 +81,10 @@ tqp_status tuned_call(tqp_ctx* ctx, const char* key, cudaStream_t stream, int op
     TQP_CUDA(cudaEventCreate(&ev[1]));
     tqp_tuning best{0, 0, 0, 0, 0};
     double best_ms = 1e30;
+    // the fastest candidate with a launch shape: its shape is kept also where a
+    // shapeless variant wins, for calls that force the other one
+    tqp_tuning shaped{0, 0, 0, 0, 0};
+    double shaped_ms = 1e30;
     const int hts = (opts & kTuneHt) ? 2 : 1;
     const int nvar = (opts & kTuneVariant) ? 2 : 1;
     for (int V = nvar - 1; V >= 0; --V)
@@ -103,12 +107,21 @@ tqp_status tuned_call(tqp_ctx* ctx, const char* key, cudaStream_t stream, int op
                         best_ms = ms;
                         best = ctx->forced;
                     }
+                    if (!shapeless && ms < shaped_ms) {
+                        shaped_ms = ms;
+                        shaped = ctx->forced;
+                    }
                 }
     ctx->forced = tqp_tuning{0, 0, 0, 0, 0};
     cudaEventDestroy(ev[0]);
     cudaEventDestroy(ev[1]);
     clear_error();
     if (best.tile_rows == 0) return run(arg);  // no candidate ran: report the built-in shape's result
+    if (shaped.tile_rows > 0) {
+        best.tile_rows = shaped.tile_rows;
+        best.stages = shaped.stages;
+        best.ctas_per_sm = shaped.ctas_per_sm;
+    }
     {
         std::lock_guard<std::mutex> lk(ctx->tuner->mu);
         ctx->tuner->table[key] = best;
