@@ -42,7 +42,7 @@ tqp_status launch_part_join(tqp_ctx* ctx, const PlanJoinArgs& J, const tqp_table
 // Fact rows from which a grouped join plan can take the radix-partitioned
 // aggregation (variant 0).  The built-in choice is the fused probe (variant 1)
 // at every size: 60M rows, 1.5M build rows, 150K groups and top-100 take 620 us
-// against 2057 us partitioned with dense keys, 1987 against 3100 us with
+// against 2046 us partitioned with dense keys, 1112 against 3090 us with
 // scattered ones.  Below this size the autotuner does not time it.
 constexpr long long kPartJoinMinRows = 1LL << 20;
 constexpr int kJoinVariant = 1;
