@@ -400,9 +400,15 @@ tqp_status mq_lower_group(const tqp_ctx* ctx, const tqp_table* t, const std::vec
         return fail(TQP_ERR_UNSUPPORTED, "shared scan: lookup tables exceed the shared-memory budget");
     const std::vector<DExpr> ex = mq_exprs(qs, members);
     const bool few = mq_few(members.size(), ex.size());
-    A->body_bytes = mq_body_bytes(few, static_cast<int>(ex.size()), static_cast<int>(words.size()),
-                                  static_cast<int>(breaks.size()));
-    const int body_smem = extra_smem + A->body_bytes;
+    const int nexpr = static_cast<int>(ex.size());
+    int body_smem = 0;
+    auto set_queue = [&](int queued) {
+        A->queued = queued;
+        A->body_bytes = mq_body_bytes(few, nexpr, queued, static_cast<int>(words.size()),
+                                      static_cast<int>(breaks.size()));
+        body_smem = extra_smem + A->body_bytes;
+    };
+    set_queue(kMqQueued);
     const std::vector<int> staged = mq_staged(qs, members, *A);
     if (staged.size() > static_cast<size_t>(kMaxStaged))
         return fail(TQP_ERR_UNSUPPORTED, "shared scan: more than %d columns", kMaxStaged);
@@ -414,7 +420,7 @@ tqp_status mq_lower_group(const tqp_ctx* ctx, const tqp_table* t, const std::vec
     // beside the tables and kMqShapeBytes; one that only the row queues push
     // over is narrowed (results do not depend on it).
     tqp_status gs = make_geom(ctx, t, staged, tu, body_smem, &A->G, smem);
-    const long long shape = static_cast<long long>(*smem) - mq_queue_bytes(few, static_cast<int>(ex.size())) + kMqShapeBytes;
+    const long long shape = static_cast<long long>(*smem) - mq_queue_bytes(few, nexpr, A->queued) + kMqShapeBytes;
     if (shape > ctx->smem_optin)
         gs = fail(TQP_ERR_UNSUPPORTED, "scan needs %lld bytes of shared memory (device allows %d)", shape, ctx->smem_optin);
     else

@@ -24,8 +24,8 @@
 //     values;
 //   * accumulation, few queries (up to kMqFew; kMqFewCounts without sums): each
 //     lane keeps its own rows' totals of every query in registers. A step with more
-//     than 32 passing rows adds each lane's rows at once, the rest goes through the
-//     queue, so that the adds of 32 rows share their instructions;
+//     than kMqQueued passing rows adds each lane's rows at once, the rest goes
+//     through the queue, so that the adds of 32 rows share their instructions;
 //     20M rows of four int32 columns, us, with a shared-memory atomic per (row,
 //     passing query) pair / the transposed queue for any number of queries / this:
 //     3 queries of 2% each 114 / 103 / 90, of 20% 193 / 258 / 114; 5 of 20% 295 /
@@ -64,21 +64,31 @@ constexpr int kMqFewCounts = 4;
 inline bool mq_few(size_t nq, size_t nexpr) { return nq <= static_cast<size_t>(nexpr ? kMqFew : kMqFewCounts); }
 
 // Queued rows (pass mask and tile row) of a consumer warp: fewer than kWarp, then
-// a step's where it has at most kWarp (few queries), or half a step's.
-__host__ __device__ constexpr int mq_queue(bool few) { return (few ? 2 : 1 + kMqRows / 2) * kWarp; }
+// half a step's (few queries: a whole step's where it has no more).
+constexpr int kMqQueue = (1 + kMqRows / 2) * kWarp;
 
-// The queues; many queries: and 32 values of a second expression per warp (the
-// first one's take the place of the rows they belong to).
-__host__ __device__ constexpr int mq_queue_bytes(bool few, int nexpr) {
-    return kConsumerWarps * (mq_queue(few) + (!few && nexpr > 1 ? kWarp : 0)) * 8;
+// Few queries: steps with at most this many passing rows use the queue. It is
+// half a step because the adds of 64 queued rows cost about as much as those of a
+// lane's own four; the worst sizes are those just above it, whose steps take
+// either way. 20M rows of int32, one sum, us, with the line at 32 / 48 / 64 rows
+// (and transposed masks for any number of queries): 8 queries that pass 25% of the
+// rows 129 / 90 / 90 (111), 35% 120 / 118 / 100 (131), 45% 120 / 123 / 116 (159);
+// 3 queries 25% 104 / 81 / 81 (129), 45% 90 / 92 / 100 (192).
+constexpr int kMqQueued = kMqRows / 2 * kWarp;
+
+// The queues (none where `queued` is 0: few queries only); many queries: and 32
+// values of a second expression per warp (the first one's take the place of the
+// rows they belong to).
+__host__ __device__ constexpr int mq_queue_bytes(bool few, int nexpr, int queued) {
+    return queued ? kConsumerWarps * (kMqQueue + (!few && nexpr > 1 ? kWarp : 0)) * 8 : 0;
 }
 // Shared memory of the queues that a launch shape has to leave room for.
 constexpr int kMqShapeBytes = 3072;
 
 // Shared memory of one launch's body: row queues | mask words | breakpoints.
 __host__ __device__ constexpr int mq_words_bytes(int nwords) { return (nwords * 4 + 15) / 16 * 16; }
-__host__ __device__ constexpr int mq_body_bytes(bool few, int nexpr, int nwords, int nbreaks) {
-    return (mq_queue_bytes(few, nexpr) + mq_words_bytes(nwords) + nbreaks * 8 + 127) / 128 * 128;
+__host__ __device__ constexpr int mq_body_bytes(bool few, int nexpr, int queued, int nwords, int nbreaks) {
+    return (mq_queue_bytes(few, nexpr, queued) + mq_words_bytes(nwords) + nbreaks * 8 + 127) / 128 * 128;
 }
 
 // One condition column of a launch.
@@ -115,6 +125,7 @@ struct MultiArgs {
     int32_t nwords;       // mask words used
     int32_t nbreaks;      // breakpoints used
     int32_t body_bytes;   // shared memory of the body (mq_body_bytes, or the largest in a batch)
+    int32_t queued;       // kMqQueued; 0 (few queries only): no queues
     MqCol c[kMaxStaged];
     ProdForm e[kMqExprs];
     int32_t ecol[kMqExprs][2];   // table column of each factor (-1: constant)
@@ -185,7 +196,7 @@ constexpr int kMqFastCols = 4;  // condition columns of the fast path
 template <bool kFew>
 struct MultiBody {
     static constexpr int kMinBlocks = 2;
-    static constexpr int kSmemBytes = mq_body_bytes(kFew, kMqExprs, kMqWords, kMqBreaks);  // the largest launch
+    static constexpr int kSmemBytes = mq_body_bytes(kFew, kMqExprs, kMqQueued, kMqWords, kMqBreaks);  // the largest launch
     static constexpr int kU = kMqRows;  // rows per lane per step
 
     const MultiArgs& A;
@@ -211,7 +222,7 @@ struct MultiBody {
     __device__ MultiBody(const MultiArgs& a, unsigned char* sm, const uint32_t* words, const int64_t* breaks,
                          const MqOut* out)
         : A(a), outp(out) {
-        const int qbytes = mq_queue_bytes(kFew, a.nexpr);
+        const int qbytes = mq_queue_bytes(kFew, a.nexpr, a.queued);
         uint32_t* ws = reinterpret_cast<uint32_t*>(sm + qbytes);
         int64_t* bs = reinterpret_cast<int64_t*>(sm + qbytes + mq_words_bytes(a.nwords));
         for (int i = threadIdx.x; i < a.nwords; i += blockDim.x) ws[i] = words[i];
@@ -221,8 +232,8 @@ struct MultiBody {
         const int warp = threadIdx.x / kWarp;
         const int lane = threadIdx.x % kWarp;
         const int cw = warp < kConsumerWarps ? warp : 0;
-        queue = reinterpret_cast<unsigned long long*>(sm) + cw * mq_queue(kFew);
-        val1 = reinterpret_cast<unsigned long long*>(sm) + kConsumerWarps * mq_queue(kFew) + cw * kWarp;
+        queue = reinterpret_cast<unsigned long long*>(sm) + cw * kMqQueue;
+        val1 = reinterpret_cast<unsigned long long*>(sm) + kConsumerWarps * kMqQueue + cw * kWarp;
         if (lane < a.nq) {
             rlo = out[lane].rlo;
             rhi = out[lane].rhi;
@@ -376,12 +387,18 @@ struct MultiBody {
         }
         if (n == 0) return;
         if constexpr (kFew) {
-            if (n > kWarp) {  // many passing rows: each lane its own
+            if (n > A.queued) {  // many passing rows: each lane its own
                 int64_t x0[U], x1[U];
 #pragma unroll
                 for (int j = 0; j < U; ++j) x0[j] = x1[j] = 0;
-                if (A.nexpr > 0) values<U>(G, v, 0, r0, x0);
-                if (A.nexpr > 1) values<U>(G, v, 1, r0, x1);
+                // one copy of the code: a small scan waits for its instructions (500K rows that
+                // all pass, two sums, 28 us against 34 with two; 20M rows 116 against 108)
+#pragma unroll 1
+                for (int e = A.nexpr - 1; e >= 0; --e) {
+#pragma unroll
+                    for (int j = 0; j < U; ++j) x1[j] = x0[j];
+                    values<U>(G, v, e, r0, x0);
+                }
 #pragma unroll
                 for (int j = 0; j < U; ++j)
                     add_row(m[j], static_cast<unsigned long long>(x0[j]), static_cast<unsigned long long>(x1[j]));
@@ -399,7 +416,8 @@ struct MultiBody {
             if (!kFew)
                 while (qn >= kWarp) flush(G, v, qn - kWarp, lane);
         }
-        if (kFew && qn >= kWarp) flush(G, v, qn - kWarp, lane);
+        if (kFew)
+            while (qn >= kWarp) flush(G, v, qn - kWarp, lane);
     }
 
     // General path (a ragged last tile, searched tables, more than
