@@ -416,10 +416,21 @@ tqp_status mq_lower_group(const tqp_ctx* ctx, const tqp_table* t, const std::vec
     int bpr = 0;
     for (int c : staged) bpr += t->cols[c].type == TQP_I64 ? 8 : (t->cols[c].type == TQP_I32 ? 4 : 1);
     tqp_tuning tu = tu_in ? *tu_in : default_tuning(ctx, bpr, body_smem);
+    if (few && !tu_in) {  // the queue is left out where it costs a resident CTA
+        set_queue(0);
+        const tqp_tuning bare = default_tuning(ctx, bpr, body_smem);
+        if (bare.ctas_per_sm > tu.ctas_per_sm) tu = bare;
+        else set_queue(kMqQueued);
+    }
     // A shape set by the caller or the tuner is refused where it does not fit
     // beside the tables and kMqShapeBytes; one that only the row queues push
-    // over is narrowed (results do not depend on it).
+    // over loses them (few queries) or is narrowed (results do not depend on it).
     tqp_status gs = make_geom(ctx, t, staged, tu, body_smem, &A->G, smem);
+    if (gs == TQP_ERR_UNSUPPORTED && few && A->queued) {
+        set_queue(0);
+        clear_error();
+        gs = make_geom(ctx, t, staged, tu, body_smem, &A->G, smem);
+    }
     const long long shape = static_cast<long long>(*smem) - mq_queue_bytes(few, nexpr, A->queued) + kMqShapeBytes;
     if (shape > ctx->smem_optin)
         gs = fail(TQP_ERR_UNSUPPORTED, "scan needs %lld bytes of shared memory (device allows %d)", shape, ctx->smem_optin);

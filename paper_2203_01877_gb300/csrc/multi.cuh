@@ -34,7 +34,9 @@
 //     sums over two columns: 99 transposed, 118 per row.
 //     The queues' shared memory is kept small because a launch shape has to fit
 //     beside it: with 160 rows per warp twelve queries over six int64 columns lose a
-//     resident CTA (519 -> 919 us);
+//     resident CTA (519 -> 919 us). Few queries do without the queue where it alone
+//     would cost one: every step adds its lanes' rows (10M rows of six
+//     int64 columns, four queries, us: 281 with one CTA per SM, 177 so);
 //   * per-query row ranges: a query may cover only rows [rlo, rhi) of the
 //     scan (queries over slices of one table).  Per tile a ballot splits the
 //     queries into those covering the whole tile and those touching part of

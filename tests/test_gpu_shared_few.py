@@ -1,4 +1,5 @@
-"""GPU: shared scans of few queries whose steps of 128 rows pass about as many rows as the queue's line (64)."""
+"""GPU: shared scans of few queries whose steps of 128 rows pass about as many rows as the queue's line (64), and
+over wide rows, where the row queues would cost a resident CTA and are left out."""
 import numpy as np
 import pytest
 
@@ -40,3 +41,13 @@ def test_about_half_a_step(ctx, n, nq, nexpr, percent):
     cols = [rng.integers(-2**30, 2**30, n), rng.integers(0, 1000, n).astype(np.int32)]
     w = 10 * percent // nq
     _run(ctx, cols, [([(1, "between", q * w, q * w + w - 1)], SUMS[q % nexpr]) for q in range(nq)])
+
+
+@pytest.mark.parametrize("n", [1, 1023, 1025, 400_003])
+@pytest.mark.parametrize("span", [1, 40, 150])
+@pytest.mark.parametrize("nexpr", [1, 2])
+def test_six_wide_columns(ctx, n, span, nexpr):
+    rng = np.random.default_rng(n + span)
+    cols = [rng.integers(0, 300, n) for _ in range(6)]
+    queries = [([(q, "between", q * span, q * span + span - 1), (q + 3, "lt", 200)], SUMS[q % nexpr]) for q in range(3)]
+    _run(ctx, cols, queries + [([(c, "lt", 250) for c in range(6)], SUMS[0])])
