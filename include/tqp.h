@@ -216,7 +216,7 @@ TQP_API tqp_status tqp_ctx_set_tuning(tqp_ctx* ctx, int32_t tile_rows, int32_t s
  * -1 restores the default (the autotuner's choice, which times both; else 0 for
  * tqp_hash_join, 1, the fused probe, for grouped join plans and 1 for
  * tqp_filter, but for a few shapes of counts and row ids without a sum that the
- * staged scan streams faster from 2^23 rows on).
+ * staged scan streams faster from 5 * 2^20 rows on).
  * Errors: TQP_ERR_INVALID_ARG. */
 TQP_API tqp_status tqp_ctx_set_variant(tqp_ctx* ctx, int32_t variant);
 

@@ -74,17 +74,36 @@ static int filter_variant(const tqp_ctx* ctx) {
     return strncmp(ctx->cur_key, "filter ", 7) == 0 ? tuned_variant(ctx, -1) : -1;
 }
 
-// Built in: the plain loads, but for two 64-bit conditions, or one beside two
-// narrower ones (not both of 8 bits), without a sum, from 2^23 rows to 2^27. A
-// step of these has too few bytes in flight for what it waits, and the staged
-// scan streams them faster: 24M rows, counts only, us staged / plain loads: two
-// int64 87 / 100 (30M rows), int64 and two int32 1.12 times, int64, int32 and
-// uint8 86 / 91, with another int32 98 / 106; at 4M rows plain loads take 0.90 of
-// the staged time, at 200M 0.94 to 1.04.
-static bool plain_loads_win(const FilterDirectArgs& D) {
-    if (D.has_sum || D.n < (1LL << 23) || D.n >= (1LL << 27)) return true;
-    const int narrow = D.nword + D.nbyte;
-    return !((D.nwide == 2 && narrow == 0) || (D.nwide == 1 && narrow >= 2 && D.nword >= 1));
+// Built in: the plain loads, but without a sum the staged scan for a few mixes
+// whose steps of plain loads have too few bytes in flight for what they wait, and
+// which the staged scan streams faster. Plain / staged time, counts only (with row
+// ids), 5% of the rows passing:
+//   rows                       4.5M       8M          24M         60M         140M
+//   two int64               0.92 (.94) 1.06 (1.05) 1.11 (1.15) 1.10 (1.09) 1.01 (1.04)
+//   with an uint8           0.96 (1.0) 1.17 (1.19) 1.18 (1.14) 1.09 (1.09) 1.02 (1.04)
+//   int64, two int32        0.96 (.94) 1.12 (1.10) 1.12 (1.12) 1.08 (1.10) 1.04 (1.07)
+//   int64, int32, uint8     0.89 (.94) 1.06 (1.10) 1.06 (1.05) 1.00 (1.02) 0.96 (1.00)
+//   with another int32      0.93 (.94) 1.11 (1.07) 1.08 (1.06) 1.03 (1.03) 0.98 (1.00)
+//   with another uint8      0.89 (.94) 1.08 (1.07) 1.04 (1.01) 0.96 (1.00) 0.92 (0.97)
+//   int64, int32            0.87 (.90) 0.91 (0.95) 1.00 (1.00) 1.04 (0.97) 0.95 (0.93)
+// and 1.05 for the last one's counts at 40M and 50M. Every other mix takes 0.64 to
+// 1.04 of the staged time from 2^23 rows on (int64 and three int32 0.72 to 0.91, two
+// int64 and an int32 0.78 to 1.02). With a sum the plain loads read its columns only
+// where rows pass: int64 and two int32 at 24M rows take 1.14 of the staged time with
+// 5% of the rows passing, 0.97 with 50%, 0.45 with 95% of each condition.
+static bool plain_loads_win(const FilterDirectArgs& D, bool ids) {
+    const long long n = D.n;
+    if (D.has_sum || n < (5LL << 20)) return true;
+    if (D.nwide == 2 && D.nword == 0) {
+        if (D.nbyte == 0) return n < (1LL << 23) || (!ids && n >= (1LL << 27));
+        return D.nbyte != 1;
+    }
+    if (D.nwide != 1) return true;
+    if (D.nword == 2 && D.nbyte == 0) return false;
+    if (D.nword >= 1 && D.nbyte == 1) return n >= (1LL << 26);
+    if (D.nword == 1 && D.nbyte == 2) return n >= (1LL << 25);
+    if (D.nword == 1 && D.nbyte == 0) return ids || n < (1LL << 25) || n >= (1LL << 26);
+    return true;
 }
 
 __global__ void __launch_bounds__(kCompactThreads) k_compact(const uint32_t* __restrict__ mask,
@@ -271,7 +290,7 @@ tqp_status launch_filter(tqp_ctx* ctx, const tqp_table* t, const tqp_pred* preds
         return launch_filter_with(A, grid, smem, lay, scratch, ctx->d_err, ctx->wait_cap, d_row_ids, capacity, d_count,
                                   d_sum, stream, &D, static_cast<int>(g));
     };
-    if (plain && (variant == 1 || plain_loads_win(D))) return run_plain();
+    if (plain && (variant == 1 || plain_loads_win(D, ids))) return run_plain();
     TQP_TRY(shape_filter(ctx, t, staged, bpr, ids, force, &A, &smem, &grid, &lay));
     const size_t used = ctx->used;
     void* scratch = arena_alloc(ctx, lay.bytes);
