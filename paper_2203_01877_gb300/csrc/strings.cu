@@ -225,7 +225,7 @@ constexpr int kSfThreads = 256;
 constexpr int kSfMinBlocks = 4;
 constexpr int kSfMaxWords = 8;
 constexpr int kSfSegs = 8;           // LIKE segments
-constexpr int kSfNumbers = 10;       // values of a numeric IN list; of a string one: sf_values()
+constexpr int kSfNumbers = 10;       // values of a numeric IN list, many rows (sf_list); of a string one: sf_values()
 constexpr int kSfWords = 1024;       // program words of a launch
 
 struct StrFastPred {
@@ -477,6 +477,14 @@ __global__ void __launch_bounds__(kSfThreads, kSfMinBlocks) k_str_fast(const __g
 // memory starts behind. 4M rows, general / here, us: 12 bytes, 16 values 83 / 80,
 // 24 values 86 / 89; 24 bytes, 10 values 88 / 77, 16 values 92 / 97; 25 bytes, 4
 // values 80 / 77, 6 values 82 / 87; int32, 10 values 56 / 56, 12 values 55 / 58.
+// Few rows wait for memory and launches, not for issue, and longer lists win too: 27
+// bytes, 8 values of a text (of random letters), here / general, 400K rows 0.87
+// (0.84), 1M 0.94 (0.97), 2M 1.00 (1.13), 16M 1.12 (1.43); 32 values 200K 0.83
+// (0.80), 400K 1.03 (1.04), 700K 1.24 (1.27).
+static int sf_list(long long n, int most) {
+    if (n < (1LL << 19)) return 32;
+    return n < 3 * (1LL << 19) ? std::max(most, 10) : most;
+}
 static int sf_values(int nw, bool stage) { return stage ? std::min(14, 36 / nw) : 64 / nw; }
 
 // The launch above from the general one; false outside its shapes.
@@ -501,7 +509,7 @@ static bool lower_str_fast(const StrLaunch& L, StrFast* F, int* words_per_string
             stage = stage || q.width % 4 != 0;
         }
         if (q.op == TQP_IN) {
-            if (q.type != TQP_CHAR && q.count > kSfNumbers) return false;
+            if (q.type != TQP_CHAR && q.count > sf_list(L.n, kSfNumbers)) return false;
             const int bytes = q.type == TQP_CHAR ? q.width : 8;
             for (int v = 0; v < q.count; ++v)
                 for (int b = 0; b < bytes; b += 4) {
@@ -548,7 +556,8 @@ static bool lower_str_fast(const StrLaunch& L, StrFast* F, int* words_per_string
     const int nw = maxw <= 8 ? 2 : (maxw <= 16 ? 4 : (maxw <= 24 ? 6 : 8));
     *words_per_string = nw;
     for (int k = 0; k < L.npred; ++k)
-        if (L.p[k].op == TQP_IN && L.p[k].type == TQP_CHAR && L.p[k].count > sf_values(nw, stage)) return false;
+        if (L.p[k].op == TQP_IN && L.p[k].type == TQP_CHAR && L.p[k].count > sf_list(L.n, sf_values(nw, stage)))
+            return false;
     return true;
 }
 
